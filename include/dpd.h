@@ -79,12 +79,12 @@ typedef struct dpd_params {
     uint32_t replica;      /* XORed into the high key word                   */
     int32_t exclude_bonded;/* 1 (paper): no pair force inside an agent       */
     int32_t noise;         /* 0: uniform alpha, 1: Gaussian alpha            */
-    int32_t tile;          /* cell-block side in cells: 0 = default, else
-                              one of 4, 8, 16                                */
+    int32_t tile;          /* cell-block side in cells: 0 = default (by the
+                              number of blocks), else one of 4, 8, 16        */
     int32_t variant;       /* pair-kernel variant: 0 = default (fastest),
-                              1 = thread-per-bead, 2 = pair queue,
-                              3 = grid-order pair queue, 4 = flat range
-                              enumeration, 5 = pair queue over merged
+                              1 = thread-per-bead, 2 = candidate masks and
+                              pair queue, 3 = grid-order pair queue, 4 = flat
+                              range enumeration, 5 = pair queue over merged
                               ranges.  tile = variant = 0 takes the
                               shape dpd_autotune cached for this workload,
                               else the built-in default.  Every shape gives
@@ -257,8 +257,9 @@ int dpd_profile_step(dpd_ctx *ctx, double ms[3]);
 
 /* ------------------------------------------------------------------------
  * Batched ensemble: R replicas (uneven box sizes, bead counts and parameters)
- * advanced together by one persistent kernel per call, captured into a CUDA
- * graph per step count.  Each replica is a full context reachable through
+ * advanced together: variant 2 (the default) by one launch per phase over the
+ * work of all replicas, captured into CUDA graphs; the other variants by one
+ * persistent kernel per call.  Each replica is a full context reachable through
  * dpd_batch_replica, so states, observables and logs use the calls above;
  * replicas must not be passed to dpd_destroy (they belong to the batch).
  * All replicas share the tile side and pair-kernel variant of p[0].
@@ -275,10 +276,9 @@ int dpd_batch_replica(dpd_batch *b, int r, dpd_ctx **view);
 /* The paper's initial condition for every replica, replica r with seed + r. */
 int dpd_batch_init_random(dpd_batch *b, uint64_t seed);
 
-/* Advance every replica n steps in one persistent launch (asynchronous).
- * Every replica must hold a state.  Grid-wide waits inside the kernel are
- * bounded; a wait that gives up is reported as DPD_ERR_TIMEOUT by
- * dpd_batch_sync. */
+/* Advance every replica n steps (asynchronous).  Every replica must hold a
+ * state.  Waits inside the kernels are bounded; a wait that gives up is
+ * reported as DPD_ERR_TIMEOUT by dpd_batch_sync. */
 int dpd_batch_step(dpd_batch *b, int64_t n);
 
 /* Wait, then return the batch's latched status (the first error of the
@@ -291,16 +291,15 @@ int dpd_batch_sync(dpd_batch *b);
  * the batch usable. */
 int dpd_batch_barrier_selftest(dpd_batch *b);
 
-/* Replica count, blocks of the persistent launch, (replica, cell block) items. */
+/* Replica count, resident force blocks, (replica, cell block) items. */
 int dpd_batch_info(dpd_batch *b, int *n_replicas, int *grid, int *n_work_tiles);
 
-/* Profile of the persistent kernel (no counterpart in the paper): runs
- * nsteps (1..64) ordinary steps of every replica (they advance, as with
- * dpd_batch_step) with the kernel's phase log on.  out[0..2]: mean ms per step
- * of the scan, scatter and force/integrate phases between grid-barrier
- * releases; out[3..5]: the mean over blocks of the ms a block spent working in
- * that phase (the difference is time spent waiting at the barrier).
- * Allocates a small log buffer.  Synchronises. */
+/* Phase profile (no counterpart in the paper): runs nsteps (1..64) ordinary
+ * steps of every replica (they advance, as with dpd_batch_step) with the phase
+ * log on.  out[0..2]: mean ms per step of the scan, scatter and
+ * force/integrate phases; out[3..5]: the mean over resident blocks of the ms a
+ * block spent working in that phase (the difference is time spent waiting for
+ * the others).  Allocates a small log buffer.  Synchronises. */
 int dpd_batch_profile(dpd_batch *b, int nsteps, double out[6]);
 
 /* Kernel-shape autotuner (no counterpart in the paper: its runs used a CPU

@@ -1,24 +1,26 @@
-// Batched ensemble: R replicas of uneven size and parameters advanced by one
-// persistent kernel (include/dpd.h, dpd_batch_*).
+// Batched ensemble: R replicas of uneven size and parameters advanced together
+// (include/dpd.h, dpd_batch_*).
 //
 // Each replica is an ordinary context (its own buffers, cell list, thermo log
 // and canonical state), so every single-system call also works on it through
 // dpd_batch_replica.  The batch adds a device table of the replicas' Sys
-// descriptors, three work lists and one kernel that runs n whole steps for all
-// replicas: per step three phases (cell scan, scatter, fused force/integrate)
-// separated by grid-wide barriers.  In the scan phase block b takes work
-// items b, b + G, b + 2G, ... (G blocks) of the list of 4096-cell chunks of
-// the replicas' decoupled look-back scans.  The scatter phase's items
-// (1024-bead chunks, shuffled once with a fixed seed so that a replica's
-// chunks spread out) and the force phase's items (replica, cell block),
-// ordered by estimated cost, largest first, are handed out by two counters
-// that are cleared before each launch and never reset inside it (every
-// block's last, failing take of a step keeps the count per step fixed),
-// which balances uneven items across blocks.  The kernel is
-// launched with no more blocks than can be resident at once and every
-// barrier wait is bounded: a block that gives up latches DPD_ERR_TIMEOUT in
-// the batch's error word instead of hanging.  The launch for a given step
-// count is captured once into a CUDA graph and replayed.
+// descriptors and three work lists: 4096-cell chunks of the replicas'
+// decoupled look-back scans, 1024-bead scatter chunks (shuffled once with a
+// fixed seed so that a replica's chunks spread out) and (replica, cell block)
+// force items ordered by estimated cost, largest first.
+//
+// Variant 2 (the default) launches one kernel per phase over its list, the
+// force items in up to three classes of mean density, captured into CUDA
+// graphs of 1 and 8 steps.  The other variants run n whole steps in one
+// persistent kernel, the phases separated by grid-wide barriers: in the scan
+// phase block b takes items b, b + G, b + 2G, ... (G blocks); the scatter and
+// force items are handed out by two counters that are cleared before each
+// launch and never reset inside it (every block's last, failing take of a
+// step keeps the count per step fixed).  That kernel is launched with no more
+// blocks than can be resident at once and every barrier wait is bounded: a
+// block that gives up latches DPD_ERR_TIMEOUT in the batch's error word
+// instead of hanging.  Its launch for a given step count is captured once into
+// a CUDA graph and replayed.
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -189,6 +191,61 @@ __global__ void __launch_bounds__(TILE_THREADS, B == 16 ? 5 : 8)
     }
 }
 
+// ---- variant 2: one launch per phase over the work items of all replicas ----
+// The persistent kernel holds its scan and scatter beside the force tile, which
+// spilled (288 bytes at the 56 registers that three 384-thread tiles leave), and
+// one launch shape for every replica: 0.74 ms a step for the 256 replicas of
+// 4.7 M beads, 0.55 of it the force phase.  As ordinary launches each phase has
+// its own registers, blocks come from the hardware queue instead of a counter, and
+// the force items go in classes of mean density with threads and shared memory of
+// their own (a dilute tile needs a third of a dense one's).
+// busy (a profiling launch): the blocks' working times in ns are added to it.
+__device__ __forceinline__ void add_busy(unsigned long long *busy, unsigned long long t0)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(busy, gtimer() - t0);
+}
+
+__global__ void __launch_bounds__(SCAN_NT)
+    k_ens_scan(const Sys *__restrict__ sys, const uint32_t *__restrict__ items, unsigned long long *busy)
+{
+    __shared__ uint32_t s_buf[SCAN_BUF];
+    const unsigned long long t0 = busy ? gtimer() : 0;
+    const Sys &d = sys[items[blockIdx.x]];
+    scan_decoupled_t<SCAN_NT>(d, (d.ncells + SCAN_TILE - 1) / SCAN_TILE, s_buf);
+    if (busy) add_busy(busy, t0);
+}
+
+template <int B>
+__global__ void __launch_bounds__(ENS_CHUNK / 4)
+    k_ens_scatter(const Sys *__restrict__ sys, const uint32_t *__restrict__ items, unsigned long long *busy)
+{
+    const unsigned long long t0 = busy ? gtimer() : 0;
+    const uint32_t w = items[blockIdx.x];
+    const Sys &d = sys[w >> 22];
+    const int k0 = (int)(w & 0x3fffffu) * ENS_CHUNK;
+    scatter_chunk<B>(d, k0, min(d.n, k0 + ENS_CHUNK));
+    if (busy) add_busy(busy, t0);
+}
+
+template <int B>
+__global__ void __launch_bounds__(tile_threads<B, 2>(), tile_ctas<B, 2>())
+    k_ens_force(const Sys *__restrict__ sys, const uint32_t *__restrict__ items, int flags, unsigned long long *busy)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    // the replica's descriptor in shared memory: the pair loop reads its
+    // constants (twenty Philox round keys among them) for every pair
+    __shared__ __align__(16) uint32_t s_sys[sizeof(Sys) / 4];
+    static_assert(sizeof(Sys) % 4 == 0, "copied by words");
+    const unsigned long long t0 = busy ? gtimer() : 0;
+    const uint32_t w = items[blockIdx.x];
+    for (int i = threadIdx.x; i < (int)(sizeof(Sys) / 4); i += blockDim.x)
+        s_sys[i] = reinterpret_cast<const uint32_t *>(sys + (w >> 22))[i];
+    __syncthreads();
+    force_tile_m<B, false>(*reinterpret_cast<const Sys *>(s_sys), (int)(w & 0x3fffffu), flags, smem);
+    if (busy) add_busy(busy, t0);
+}
+
 // Self-test of the bounded barrier: block 0 never arrives, every other block
 // must give up after the spin limit and latch DPD_ERR_TIMEOUT.
 __global__ void k_barrier_selftest(unsigned *bar, int *berr)
@@ -211,11 +268,20 @@ struct dpd_batch {
     unsigned *d_bar = nullptr;
     int *d_err = nullptr;
     unsigned long long *d_ctr = nullptr;   // work counters: [0] force phase, [1] scatter phase
-    int n_scan = 0, n_scat = 0, n_tiles = 0, B = 8, var = 2, cap = 0, grid = 0;
+    int n_scan = 0, n_scat = 0, n_tiles = 0, B = 8, var = 2, grid = 0;
     size_t smem = 0;
     cudaGraphExec_t g = nullptr;
     int64_t g_steps = -1;
     int *h_pin = nullptr;
+    // variant 2: the force items by classes of threads per tile, each launched
+    // on a stream of its own beside the others, and the step graphs
+    struct Class { int nt, cap, first, n, slots; size_t smem; };
+    std::vector<Class> cls;
+    static constexpr int MAX_CLASSES = 3;
+    cudaStream_t side[MAX_CLASSES - 1] = {};
+    cudaEvent_t fork = nullptr, join[MAX_CLASSES - 1] = {};
+    cudaGraphExec_t g1 = nullptr, g8 = nullptr, gfin = nullptr;
+    int scan_slots = 0, scat_slots = 0;
 };
 
 #define CUB(x)                                                                      \
@@ -250,13 +316,150 @@ static void ens_launch(dpd_batch *b, int nsteps, int final_last, unsigned long l
                                                                   final_last, b->d_ctr, tlog);
 }
 
+template <int B>
+static int ens_prepare2(dpd_batch *b)
+{
+    int dev = 0, nsm = 0, occ = 0;
+    CUB(cudaGetDevice(&dev));
+    CUB(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    cudaFuncAttributes fa;
+    CUB(cudaFuncGetAttributes(&fa, k_ens_force<B>));
+    CUB(cudaFuncSetAttribute(k_ens_force<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             max_dynamic_smem() - (int)fa.sharedSizeBytes));
+    b->grid = 0;
+    for (auto &c : b->cls) {
+        if (c.smem + fa.sharedSizeBytes > (size_t)max_dynamic_smem()) return DPD_ERR_INVALID_ARG;
+        CUB(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ens_force<B>, c.nt, c.smem));
+        if (occ < 1) return DPD_ERR_INVALID_ARG;
+        c.slots = std::min(nsm * occ, c.n);
+        b->grid = std::max(b->grid, nsm * occ);
+    }
+    CUB(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ens_scan, SCAN_NT, 0));
+    b->scan_slots = std::min(nsm * occ, b->n_scan);
+    CUB(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ens_scatter<B>, ENS_CHUNK / 4, 0));
+    b->scat_slots = std::min(nsm * occ, b->n_scat);
+    return DPD_OK;
+}
+
+template <int B>
+static void ens_scatter2(dpd_batch *b, unsigned long long *busy)
+{
+    k_ens_scatter<B><<<b->n_scat, ENS_CHUNK / 4, 0, b->st>>>(b->d_sys, b->d_scat, busy);
+}
+template <int B>
+static void ens_force2(dpd_batch *b, const dpd_batch::Class &c, cudaStream_t st, int flags, unsigned long long *busy)
+{
+    k_ens_force<B><<<c.n, c.nt, c.smem, st>>>(b->d_sys, b->d_tiles + c.first, flags, busy);
+}
+
+static void ens_scan_scatter(dpd_batch *b, int phase, unsigned long long *busy)
+{
+    if (phase == 0) k_ens_scan<<<b->n_scan, SCAN_NT, 0, b->st>>>(b->d_sys, b->d_scan, busy);
+    else if (b->B == 4) ens_scatter2<4>(b, busy);
+    else if (b->B == 8) ens_scatter2<8>(b, busy);
+    else ens_scatter2<16>(b, busy);
+}
+static void ens_force_class(dpd_batch *b, size_t i, cudaStream_t st, int flags, unsigned long long *busy)
+{
+    if (b->B == 4) ens_force2<4>(b, b->cls[i], st, flags, busy);
+    else if (b->B == 8) ens_force2<8>(b, b->cls[i], st, flags, busy);
+    else ens_force2<16>(b, b->cls[i], st, flags, busy);
+}
+
+// One step of every replica on the batch's stream; the force classes run
+// beside one another (the denser ones first).
+static int ens_step2(dpd_batch *b, int flags)
+{
+    ens_scan_scatter(b, 0, nullptr);
+    ens_scan_scatter(b, 1, nullptr);
+    const size_t n = b->cls.size();
+    if (n > 1) CUB(cudaEventRecord(b->fork, b->st));
+    for (size_t i = 1; i < n; ++i) CUB(cudaStreamWaitEvent(b->side[i - 1], b->fork, 0));
+    for (size_t i = 0; i < n; ++i) ens_force_class(b, i, i ? b->side[i - 1] : b->st, flags, nullptr);
+    for (size_t i = 1; i < n; ++i) {
+        CUB(cudaEventRecord(b->join[i - 1], b->side[i - 1]));
+        CUB(cudaStreamWaitEvent(b->st, b->join[i - 1], 0));
+    }
+    CUB(cudaGetLastError());
+    return DPD_OK;
+}
+
+static int ens_capture2(dpd_batch *b, int iters, int last_flags, cudaGraphExec_t *out)
+{
+    cudaGraph_t g = nullptr;
+    CUB(cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal));
+    int rc = DPD_OK;
+    for (int i = 0; i < iters && rc == DPD_OK; ++i) rc = ens_step2(b, i == iters - 1 ? last_flags : F_ADVANCE);
+    const cudaError_t e = cudaStreamEndCapture(b->st, &g);
+    if (rc != DPD_OK || e != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return rc != DPD_OK ? rc : DPD_ERR_CUDA;
+    }
+    const cudaError_t e2 = cudaGraphInstantiate(out, g, 0);
+    cudaGraphDestroy(g);
+    CUB(e2);
+    return DPD_OK;
+}
+
+static void ens_free_graphs(dpd_batch *b)
+{
+    for (cudaGraphExec_t *g : {&b->g, &b->g1, &b->g8, &b->gfin}) {
+        if (*g) cudaGraphExecDestroy(*g);
+        *g = nullptr;
+    }
+}
+
+// Threads, tile capacity and shared memory of every class and replica, and the
+// force items of each class in a row (d_tiles keeps the order of `tiles`).  The
+// capacity takes what shared memory the class's residency leaves (tiles that
+// cluster stay off the global-memory path), or cap_min if that is more.
+static void ens_classes(dpd_batch *b, std::vector<Sys> &sys, std::vector<uint32_t> &tiles)
+{
+    long long blocks = (long long)tiles.size();
+    std::vector<int> cls_of(b->R);
+    b->cls.clear();
+    for (int k = dpd_batch::MAX_CLASSES; k >= 1; --k) {
+        dpd_batch::Class c{0, 0, 0, 0, 0, 0};
+        for (int r = 0; r < b->R; ++r) {
+            dpd_ctx *x = b->reps[r];
+            const int nt = tile_nt(mean_owned(&x->p, b->B), blocks, b->B, 2);
+            if ((nt + 127) / 128 != k) continue;
+            c.nt = std::max(c.nt, nt);
+            c.cap = std::max(c.cap, sys[r].cap);
+            cls_of[r] = (int)b->cls.size();
+        }
+        if (c.nt) b->cls.push_back(c);
+    }
+    for (auto &c : b->cls) {
+        const size_t per_sm = 228 * 1024, own = 1024 + sizeof(Sys) + 64;
+        const size_t fit = std::max<size_t>(1, std::min<size_t>(per_sm / (force_smem(b->B, 2, c.cap, c.nt, false) + own),
+                                                               65536 / 56 / (size_t)c.nt));
+        while (c.cap + 32 <= 4096 && force_smem(b->B, 2, c.cap + 32, c.nt, true) <= 200 * 1024 &&
+               per_sm / (force_smem(b->B, 2, c.cap + 32, c.nt, false) + own) >= fit)
+            c.cap += 32;
+        c.smem = force_smem(b->B, 2, c.cap, c.nt, false);
+    }
+    std::stable_sort(tiles.begin(), tiles.end(),
+                     [&](uint32_t u, uint32_t v) { return cls_of[u >> 22] < cls_of[v >> 22]; });
+    for (uint32_t w : tiles) ++b->cls[cls_of[w >> 22]].n;
+    for (size_t i = 1; i < b->cls.size(); ++i) b->cls[i].first = b->cls[i - 1].first + b->cls[i - 1].n;
+    for (int r = 0; r < b->R; ++r) {
+        const auto &c = b->cls[cls_of[r]];
+        dpd_ctx *x = b->reps[r];
+        sys[r].nt = x->d.nt = c.nt;
+        sys[r].cap = x->d.cap = c.cap;
+        x->smem = c.smem;
+    }
+}
+
 static int ens_dispatch_prepare(dpd_batch *b)
 {
+    if (b->var == 2) return b->B == 4 ? ens_prepare2<4>(b) : b->B == 8 ? ens_prepare2<8>(b) : ens_prepare2<16>(b);
     if (b->var == 1) return b->B == 4 ? ens_prepare<4, 1>(b) : b->B == 8 ? ens_prepare<8, 1>(b) : ens_prepare<16, 1>(b);
     if (b->var == 3) return b->B == 4 ? ens_prepare<4, 3>(b) : b->B == 8 ? ens_prepare<8, 3>(b) : ens_prepare<16, 3>(b);
     if (b->var == 4) return b->B == 4 ? ens_prepare<4, 4>(b) : b->B == 8 ? ens_prepare<8, 4>(b) : ens_prepare<16, 4>(b);
     if (b->var == 5) return b->B == 4 ? ens_prepare<4, 5>(b) : b->B == 8 ? ens_prepare<8, 5>(b) : ens_prepare<16, 5>(b);
-    return b->B == 4 ? ens_prepare<4, 2>(b) : b->B == 8 ? ens_prepare<8, 2>(b) : ens_prepare<16, 2>(b);
+    return DPD_ERR_INVALID_ARG;
 }
 
 static void ens_dispatch_launch(dpd_batch *b, int nsteps, int final_last, unsigned long long *tlog = nullptr)
@@ -277,10 +480,6 @@ static void ens_dispatch_launch(dpd_batch *b, int nsteps, int final_last, unsign
         if (b->B == 4) ens_launch<4, 5>(b, nsteps, final_last, tlog);
         else if (b->B == 8) ens_launch<8, 5>(b, nsteps, final_last, tlog);
         else ens_launch<16, 5>(b, nsteps, final_last, tlog);
-    } else {
-        if (b->B == 4) ens_launch<4, 2>(b, nsteps, final_last, tlog);
-        else if (b->B == 8) ens_launch<8, 2>(b, nsteps, final_last, tlog);
-        else ens_launch<16, 2>(b, nsteps, final_last, tlog);
     }
 }
 
@@ -324,12 +523,17 @@ static int ens_build_tables(dpd_batch *b)
     std::stable_sort(order.begin(), order.end(), [&sys](uint32_t a, uint32_t c) { return sys[a].ncells > sys[c].ncells; });
     for (uint32_t r : order)
         for (int k = 0; k < (sys[r].ncells + SCAN_TILE - 1) / SCAN_TILE; ++k) scan.push_back(r);
-    // every replica's tile plan fits the common shared-memory size
-    for (int r = 0; r < b->R; ++r) sys[r].cap = cap;
-    for (int r = 0; r < b->R; ++r) b->reps[r]->d.cap = cap;
-    b->cap = cap;
-    // the dynamic buffer also serves the scan phase's transpose
-    b->smem = std::max(force_smem(b->B, b->var, cap, false), sizeof(uint32_t) * (size_t)SCAN_BUF);
+    if (b->var == 2) {
+        ens_classes(b, sys, tiles);
+    } else {
+        // every replica's tile plan fits the common shared-memory size; the
+        // dynamic buffer also serves the scan phase's transpose
+        b->smem = std::max(force_smem(b->B, b->var, cap, TILE_THREADS, false), sizeof(uint32_t) * (size_t)SCAN_BUF);
+        for (int r = 0; r < b->R; ++r) {
+            sys[r].cap = b->reps[r]->d.cap = cap;
+            b->reps[r]->smem = b->smem;
+        }
+    }
     b->n_scan = (int)scan.size();
     b->n_scat = (int)scat.size();
     b->n_tiles = (int)tiles.size();
@@ -351,14 +555,56 @@ static int ens_build_tables(dpd_batch *b)
     CUB(cudaMemsetAsync(b->d_bar, 0, 64, b->st));
     for (int r = 0; r < b->R; ++r) {
         dpd_ctx *c = b->reps[r];
-        c->smem = b->smem;
-        const int rc = set_force_smem(c->B, b->var, cap);
+        const int rc = set_force_smem(c->B, b->var, c->d.cap, c->d.nt);
         if (rc) return rc;
     }
     int rc = ens_dispatch_prepare(b);
     if (rc) return rc;
     CUB(cudaStreamSynchronize(b->st));
     return DPD_OK;
+}
+
+// Profile of the phase launches: their times between events, one class of
+// force items after the other, and the mean time that a resident block worked.
+static int ens_profile2(dpd_batch *b, int nsteps, double out[6])
+{
+    struct Events {
+        cudaEvent_t e[4] = {};
+        ~Events() { for (auto x : e) if (x) cudaEventDestroy(x); }
+    } ev;
+    for (auto &x : ev.e) CUB(cudaEventCreate(&x));
+    constexpr int NB = 2 + dpd_batch::MAX_CLASSES;
+    unsigned long long *busy = nullptr, h[NB];
+    CUB(cudaMalloc(&busy, sizeof h));
+    cudaError_t e = cudaMemsetAsync(busy, 0, sizeof h, b->st);
+    for (int p = 0; p < 6; ++p) out[p] = 0.0;
+    for (int s = 0; s < nsteps && e == cudaSuccess; ++s) {
+        cudaEventRecord(ev.e[0], b->st);
+        ens_scan_scatter(b, 0, busy);
+        cudaEventRecord(ev.e[1], b->st);
+        ens_scan_scatter(b, 1, busy + 1);
+        cudaEventRecord(ev.e[2], b->st);
+        for (size_t i = 0; i < b->cls.size(); ++i)
+            ens_force_class(b, i, b->st, F_ADVANCE | (s == nsteps - 1 ? F_FINAL : 0), busy + 2 + i);
+        cudaEventRecord(ev.e[3], b->st);
+        e = cudaEventSynchronize(ev.e[3]);
+        for (int p = 0; p < 3 && e == cudaSuccess; ++p) {
+            float ms = 0.f;
+            e = cudaEventElapsedTime(&ms, ev.e[p], ev.e[p + 1]);
+            out[p] += ms / nsteps;
+        }
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(h, busy, sizeof h, cudaMemcpyDeviceToHost);
+    cudaFree(busy);
+    if (e != cudaSuccess) return DPD_ERR_CUDA;
+    for (dpd_ctx *c : b->reps) {
+        c->step += nsteps;
+        c->sorted_canonical = true;
+    }
+    out[3] = (double)h[0] / b->scan_slots / nsteps / 1e6;
+    out[4] = (double)h[1] / b->scat_slots / nsteps / 1e6;
+    for (size_t i = 0; i < b->cls.size(); ++i) out[5] += (double)h[2 + i] / b->cls[i].slots / nsteps / 1e6;
+    return dpd_batch_sync(b);
 }
 
 extern "C" {
@@ -376,7 +622,12 @@ int dpd_batch_create(const dpd_params *p, int R, void *stream, dpd_batch **out)
     // one shape for every replica: the caller's, the tuned one, or the default
     std::vector<dpd_params> q(p, p + R);
     {
-        int t = p[0].tile ? p[0].tile : DEFAULT_TILE, v = p[0].variant ? p[0].variant : DEFAULT_VARIANT;
+        int v = p[0].variant ? p[0].variant : DEFAULT_VARIANT, t = p[0].tile ? p[0].tile : DEFAULT_TILE;
+        if (!p[0].tile && v == DEFAULT_VARIANT) {
+            long long blocks16 = 0;
+            for (int r = 0; r < R; ++r) blocks16 += blocks_of(&p[r], 16);
+            t = default_tile(blocks16);
+        }
         if (!p[0].tile && !p[0].variant) tuned_shape(p, R, &t, &v);
         for (auto &e : q) { e.tile = t; e.variant = v; }
     }
@@ -398,6 +649,13 @@ int dpd_batch_create(const dpd_params *p, int R, void *stream, dpd_batch **out)
         if (rc == DPD_OK) b->reps[r]->batch_owned = true;
     }
     if (rc == DPD_OK && cudaMallocHost((void **)&b->h_pin, 64) != cudaSuccess) rc = DPD_ERR_OOM;
+    if (rc == DPD_OK && b->var == 2) {
+        bool ok = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
+        for (int i = 0; i < dpd_batch::MAX_CLASSES - 1; ++i)
+            ok = ok && cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking) == cudaSuccess &&
+                 cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming) == cudaSuccess;
+        if (!ok) rc = DPD_ERR_CUDA;
+    }
     if (rc == DPD_OK) rc = ens_build_tables(b);
     if (rc) {
         dpd_batch_destroy(b);
@@ -411,7 +669,12 @@ void dpd_batch_destroy(dpd_batch *b)
 {
     if (!b) return;
     if (b->st) cudaStreamSynchronize(b->st);
-    if (b->g) cudaGraphExecDestroy(b->g);
+    ens_free_graphs(b);
+    for (int i = 0; i < dpd_batch::MAX_CLASSES - 1; ++i) {
+        if (b->join[i]) cudaEventDestroy(b->join[i]);
+        if (b->side[i]) cudaStreamDestroy(b->side[i]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
     for (dpd_ctx *c : b->reps) {
         if (c) {
             c->batch_owned = false;
@@ -447,6 +710,20 @@ int dpd_batch_step(dpd_batch *b, int64_t n)
     for (dpd_ctx *c : b->reps)
         if (!c->have_state) return DPD_ERR_STATE;
     if (n == 0) return DPD_OK;
+    if (b->var == 2) {
+        int rc = DPD_OK;
+        if (!b->g1 && (rc = ens_capture2(b, 1, F_ADVANCE, &b->g1))) return rc;
+        if (!b->g8 && (rc = ens_capture2(b, 8, F_ADVANCE, &b->g8))) return rc;
+        if (!b->gfin && (rc = ens_capture2(b, 1, F_ADVANCE | F_FINAL, &b->gfin))) return rc;
+        for (int64_t i = 0; i < (n - 1) / 8; ++i) CUB(cudaGraphLaunch(b->g8, b->st));
+        for (int64_t i = 0; i < (n - 1) % 8; ++i) CUB(cudaGraphLaunch(b->g1, b->st));
+        CUB(cudaGraphLaunch(b->gfin, b->st));
+        for (dpd_ctx *c : b->reps) {
+            c->step += n;
+            c->sorted_canonical = true;
+        }
+        return DPD_OK;
+    }
     if (!b->g || b->g_steps != n) {
         if (b->g) cudaGraphExecDestroy(b->g);
         b->g = nullptr;
@@ -476,8 +753,22 @@ int dpd_batch_sync(dpd_batch *b)
     CUB(cudaStreamSynchronize(b->st));
     int status = DPD_OK;
     if (b->h_pin[0] & ERR_TIMEOUT) status = DPD_ERR_TIMEOUT;
+    bool grown = false;
     for (dpd_ctx *c : b->reps) {
+        const unsigned long long seen = c->ovf_seen;
         const int rc = dpd_internal_latched(c);
+        if (rc && status == DPD_OK) status = rc;
+        // tiles of this replica took the global-memory path: a quarter more
+        // room for its class, as a single system's
+        if (b->var == 2 && c->ovf_seen > seen) {
+            c->d.cap = std::min(4096, ((c->d.cap * 5 / 4) + 31) & ~31);
+            while (force_smem(b->B, 2, c->d.cap, tile_threads<16, 2>(), true) > 200 * 1024) c->d.cap -= 32;
+            grown = true;
+        }
+    }
+    if (grown) {
+        ens_free_graphs(b);
+        const int rc = ens_build_tables(b);
         if (rc && status == DPD_OK) status = rc;
     }
     return status;
@@ -506,6 +797,7 @@ int dpd_batch_profile(dpd_batch *b, int nsteps, double out[6])
     if (!b || !out || nsteps < 1 || nsteps > 64) return DPD_ERR_INVALID_ARG;
     for (dpd_ctx *c : b->reps)
         if (!c->have_state) return DPD_ERR_STATE;
+    if (b->var == 2) return ens_profile2(b, nsteps, out);
     const size_t n_blk = 3ull * nsteps * (size_t)b->grid, n_rel = 4ull * nsteps;
     unsigned long long *dlog = nullptr;
     CUB(cudaMalloc(&dlog, 8 * (n_blk + n_rel)));

@@ -140,12 +140,12 @@ __global__ void k_kick_bin(Sys d)
 }
 
 template <int B, bool COUNT, int VAR>
-__global__ void __launch_bounds__(TILE_THREADS, 10) k_force(Sys d, int flags)
+__global__ void __launch_bounds__(tile_threads<B, VAR>(), tile_ctas<B, VAR>()) k_force(Sys d, int flags)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     Thermo3 th{0.0, 0.0, 0.0};
     force_tile<B, COUNT, VAR>(d, blockIdx.x, flags, smem, th);
-    if (flags & (F_ADVANCE | F_FINAL)) {
+    if (VAR != 2 && (flags & (F_ADVANCE | F_FINAL))) {   // variant 2 adds its thermo partials itself
         __syncthreads();
         thermo_flush_tile(d, th, (double *)(smem + tile_flush_off<B, VAR>()));
     }
@@ -249,6 +249,24 @@ void fill_geometry(Sys &d, const dpd_params *p, int B)
     d.ntx = (nc + B - 1) / B;
     d.n = (int)p->n_beads;
     d.ncells = nc * nc;
+    // Candidate filter in cell units.  Offsets reach B/2 + 1 cells from the
+    // tile's middle, so a half holds them to half an ulp: 2^-9 below 8 (2^-8
+    // below 16); a separation component is off by at most twice that and its
+    // own rounding (2^-11 below 2), the distance by sqrt(2) of it, the square
+    // by two roundings of 2^-11 each.
+    const double ulp2 = B / 2 + 1 < 4 ? std::ldexp(1.0, -10) : B / 2 + 1 < 8 ? std::ldexp(1.0, -9) : std::ldexp(1.0, -8);
+    const double off = std::sqrt(2.0) * (2.0 * ulp2 + std::ldexp(1.0, -11)), rcc = p->rc * nc / p->L;
+    d.near2 = (float)((rcc + off) * (rcc + off) * (1.0 + std::ldexp(1.0, -9)));
+    // Lanes per staged row: the smallest of 8, 16, 32 that a row's mean
+    // population fills, so dilute rows share a warp.
+    const double row = (double)p->n_beads * (B + 2) / ((double)nc * nc);
+    d.rowl = row <= 6.0 ? 3 : row <= 13.0 ? 4 : 5;
+}
+
+double mean_owned(const dpd_params *p, int B)
+{
+    const int nc = n_cells_side(p->L, p->rc), b = std::min(B, nc);
+    return (double)p->n_beads * b * b / ((double)nc * nc);
 }
 
 int tile_capacity(const dpd_params *p, int B)
@@ -257,18 +275,45 @@ int tile_capacity(const dpd_params *p, int B)
     const double cs = p->L / nc;
     const double rho = (double)p->n_beads / (p->L * p->L);
     const double mean = rho * ((B + 2) * cs) * ((B + 2) * cs);
-    // mean staged population plus a margin of eight Poisson standard
-    // deviations, kept small so that ten tiles stay resident per SM at
+    // mean staged population plus a margin of 6.5 Poisson standard
+    // deviations, kept small so that nine tiles stay resident per SM at
     // density 3 (1.3 x mean measured 4% slower at 8 x 8 cells and 17% at
     // 16 x 16); a tile above it takes the (slower, exact) global-memory path,
     // and a context that sees such tiles grows its capacity at the next
     // synchronising call
-    int cap = (int)std::ceil(mean + 8.0 * std::sqrt(mean) + 32.0);
+    int cap = (int)std::ceil(mean + 6.5 * std::sqrt(mean));
     cap = (cap + 31) & ~31;
     return std::min(std::max(cap, 256), 4096);   // queue entries pack bead slots in 12 bits
 }
 
-size_t force_smem(int B, int var, int cap, bool count)
+// Cell-block side when the caller and the tuner leave it open: 16 x 16 blocks
+// carry the smaller halo (1.27 staged beads per owned one instead of 1.56) and
+// win from two blocks per SM on (us a step at density 1.6: 512 x 512 cells 44.8
+// against 52.3, 256 x 256 cells 21.5 against 21.1; 1024 x 1024 at density 3: 278
+// against 303).
+int default_tile(long long blocks16) { return blocks16 >= 304 ? 16 : 8; }
+
+long long blocks_of(const dpd_params *p, int B)
+{
+    const long long nt = (n_cells_side(p->L, p->rc) + B - 1) / B;
+    return nt * nt;
+}
+
+// Threads per tile: about two owned beads each where the blocks fill the chip
+// (16 x 16 blocks of 1024 x 1024 cells, us a step at 128 / 192 / 256 / 384
+// threads: 394 / 322 / 296 / 278 at density 3, 145 / 131 / 134 / 151 at 1.6,
+// 76 / 82 / 90 / 99 at 0.8; 8 x 8 blocks take 128 at every density), the most
+// where a block's own latency is the step's (4 blocks per SM or fewer: 128 x 128
+// cells in 8 x 8 blocks, 14.8 at 192 against 16.0 at 128).
+int tile_nt(double own, long long blocks, int B, int var)
+{
+    if (var != 2) return TILE_THREADS;
+    if (blocks <= 640) return B == 16 ? 384 : B == 8 ? 192 : 128;
+    if (B != 16) return 128;
+    return std::min(std::max(((int)(0.5 * own) + 32) / 64 * 64, 64), 384);
+}
+
+size_t force_smem(int B, int var, int cap, int nt, bool count)
 {
     if (var == 3) {
         switch (B) {
@@ -291,10 +336,17 @@ size_t force_smem(int B, int var, int cap, bool count)
             default: return TilePlan<16, 5>::bytes(cap, TILE_THREADS, count);
         }
     }
+    if (var == 1) {
+        switch (B) {
+            case 4: return TilePlan<4, 1>::bytes(cap, TILE_THREADS, count);
+            case 8: return TilePlan<8, 1>::bytes(cap, TILE_THREADS, count);
+            default: return TilePlan<16, 1>::bytes(cap, TILE_THREADS, count);
+        }
+    }
     switch (B) {
-        case 4: return TilePlan<4>::bytes(cap, TILE_THREADS, count);
-        case 8: return TilePlan<8>::bytes(cap, TILE_THREADS, count);
-        default: return TilePlan<16>::bytes(cap, TILE_THREADS, count);
+        case 4: return TilePlanM<4>::bytes(cap, nt, count);
+        case 8: return TilePlanM<8>::bytes(cap, nt, count);
+        default: return TilePlanM<16>::bytes(cap, nt, count);
     }
 }
 
@@ -334,10 +386,10 @@ int max_dynamic_smem()
     return smax;
 }
 
-int set_force_smem(int B, int var, int cap)
+int set_force_smem(int B, int var, int cap, int nt)
 {
     const int smax = max_dynamic_smem();
-    if ((int)force_smem(B, var, cap, true) > smax) return DPD_ERR_INVALID_ARG;
+    if ((int)force_smem(B, var, cap, nt, true) > smax) return DPD_ERR_INVALID_ARG;
     int rc = set_force_attrs<4>(smax);
     if (!rc) rc = set_force_attrs<8>(smax);
     if (!rc) rc = set_force_attrs<16>(smax);
@@ -348,8 +400,8 @@ template <int B, int VAR>
 static void launch_force_t(const Sys &d, cudaStream_t st, size_t smem, int flags, bool count)
 {
     const int ntiles = d.ntx * d.ntx;
-    if (count) k_force<B, true, VAR><<<ntiles, TILE_THREADS, force_smem(B, VAR, d.cap, true), st>>>(d, flags);
-    else k_force<B, false, VAR><<<ntiles, TILE_THREADS, smem, st>>>(d, flags);
+    if (count) k_force<B, true, VAR><<<ntiles, d.nt, force_smem(B, VAR, d.cap, d.nt, true), st>>>(d, flags);
+    else k_force<B, false, VAR><<<ntiles, d.nt, smem, st>>>(d, flags);
 }
 
 void launch_force_only(const Sys &d, int B, int var, cudaStream_t st, size_t smem, int flags, bool count)
@@ -475,10 +527,10 @@ constexpr int H_PIN_STATUS = 510;   // h_pin holds 512 doubles; [510], [511]: er
 static void grow_capacity(dpd_ctx *c)
 {
     int cap = std::min(4096, ((c->d.cap * 5 / 4) + 31) & ~31);
-    while (cap > c->d.cap && force_smem(c->B, c->var, cap, true) > 200 * 1024) cap -= 32;
+    while (cap > c->d.cap && force_smem(c->B, c->var, cap, c->d.nt, true) > 200 * 1024) cap -= 32;
     if (cap <= c->d.cap) return;
     c->d.cap = cap;
-    c->smem = force_smem(c->B, c->var, cap, false);
+    c->smem = force_smem(c->B, c->var, cap, c->d.nt, false);
     free_graphs(c);
 }
 
@@ -531,8 +583,8 @@ int dpd_create(const dpd_params *p, void *stream, dpd_ctx **out)
     if (!c) return DPD_ERR_OOM;
     if (cudaGetDevice(&c->dev) != cudaSuccess) { delete c; return DPD_ERR_CUDA; }
     c->p = *p;
-    c->B = p->tile ? p->tile : DEFAULT_TILE;
     c->var = p->variant ? p->variant : DEFAULT_VARIANT;
+    c->B = p->tile ? p->tile : c->var == DEFAULT_VARIANT ? default_tile(blocks_of(p, 16)) : DEFAULT_TILE;
     if (!p->tile && !p->variant) {
         int t = 0, v = 0;
         if (tuned_shape(p, 1, &t, &v)) { c->B = t; c->var = v; }
@@ -547,10 +599,11 @@ int dpd_create(const dpd_params *p, void *stream, dpd_ctx **out)
     fill_geometry(d, p, c->B);
     fill_physics(d, p);
     d.cap = tile_capacity(p, c->B);
-    c->smem = force_smem(c->B, c->var, d.cap, false);
-    if (force_smem(c->B, c->var, d.cap, true) > 200 * 1024) {
-        d.cap = (int)((200 * 1024 - force_smem(c->B, c->var, 0, true)) / (c->var == 3 ? 43 : 41)) & ~31;
-        c->smem = force_smem(c->B, c->var, d.cap, false);
+    d.nt = tile_nt(mean_owned(p, c->B), (long long)d.ntx * d.ntx, c->B, c->var);
+    c->smem = force_smem(c->B, c->var, d.cap, d.nt, false);
+    if (force_smem(c->B, c->var, d.cap, d.nt, true) > 200 * 1024) {
+        d.cap = (int)((200 * 1024 - force_smem(c->B, c->var, 0, d.nt, true)) / (c->var == 2 ? 50 : c->var == 3 ? 43 : 41)) & ~31;
+        c->smem = force_smem(c->B, c->var, d.cap, d.nt, false);
     }
     c->nscan = (d.ncells + SCAN_TILE - 1) / SCAN_TILE;
     const size_t n = (size_t)d.n, nce = (size_t)d.ncells;
@@ -596,7 +649,7 @@ int dpd_create(const dpd_params *p, void *stream, dpd_ctx **out)
     d.scan_status = (unsigned long long *)(b + o_ss);
     d.scan_ticket = (unsigned long long *)(b + o_tk);
     if (cudaMemsetAsync(c->pool, 0, off, c->st) != cudaSuccess ||
-        (rc = set_force_smem(c->B, c->var, d.cap)) != DPD_OK) {
+        (rc = set_force_smem(c->B, c->var, d.cap, d.nt)) != DPD_OK) {
         dpd_destroy(c);
         return rc ? rc : DPD_ERR_CUDA;
     }
@@ -625,7 +678,14 @@ int dpd_set_params(dpd_ctx *c, const dpd_params *p)
     if (p->n_beads != c->p.n_beads || p->L != c->p.L || p->rc != c->p.rc) return DPD_ERR_STATE;
     const int B = p->tile ? p->tile : c->B;
     if (B != c->B) return DPD_ERR_STATE;
-    c->var = p->variant ? p->variant : c->var;
+    const int var = p->variant ? p->variant : c->var;
+    if (var != c->var) {   // another variant's shared-memory plan
+        const int nt = tile_nt(mean_owned(p, c->B), (long long)c->d.ntx * c->d.ntx, c->B, var);
+        if (force_smem(c->B, var, c->d.cap, nt, true) > 200 * 1024) return DPD_ERR_INVALID_ARG;
+        c->var = var;
+        c->d.nt = nt;
+        c->smem = force_smem(c->B, var, c->d.cap, nt, false);
+    }
     c->p = *p;
     fill_physics(c->d, p);
     free_graphs(c);   // kernel arguments carry the parameters

@@ -11,6 +11,8 @@
 //            v_{s+1/2} = v_s + dt/2m f_s, x_{s+1} = wrap(x_s + dt v_{s+1/2}),
 //            binning of x_{s+1} into counts (rank = atomic ticket) -> U.
 #pragma once
+#include <cuda_fp16.h>
+
 #include "dpd_device.cuh"
 
 namespace dpd {
@@ -31,7 +33,15 @@ namespace dpd {
 constexpr int SCAN_BUF = SCAN_TILE + SCAN_TILE / 32;
 __device__ __forceinline__ int scan_pad(int e) { return e + (e >> 5); }
 
-template <int NT>
+// Barrier of the scan's NT threads: the block, or its first NT threads (PART).
+template <int NT, bool PART>
+__device__ __forceinline__ void scan_sync()
+{
+    if constexpr (PART) asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+    else __syncthreads();
+}
+
+template <int NT, bool PART = false>
 __device__ inline void scan_decoupled_t(const Sys &d, int nblocks, uint32_t *s_buf)
 {
     constexpr int IPT = SCAN_TILE / NT;
@@ -46,7 +56,7 @@ __device__ inline void scan_decoupled_t(const Sys &d, int nblocks, uint32_t *s_b
         s_bid = (int)(t % (unsigned long long)nblocks);
         s_epoch = (uint32_t)((t / (unsigned long long)nblocks + 1ull) & 0x3fffffffull);
     }
-    __syncthreads();
+    scan_sync<NT, PART>();
     const int bid = s_bid;
     const unsigned long long ep = s_epoch;
     const int base = bid * SCAN_TILE;
@@ -68,7 +78,7 @@ __device__ inline void scan_decoupled_t(const Sys &d, int nblocks, uint32_t *s_b
         const int idx = base + k * NT + tid;
         if (idx < d.ncells) d.counts[idx] = 0u;
     }
-    __syncthreads();
+    scan_sync<NT, PART>();
     uint32_t sum = 0;
 #pragma unroll 8
     for (int k = 0; k < IPT; ++k) sum += s_buf[scan_pad(tid * IPT + k)];
@@ -81,7 +91,7 @@ __device__ inline void scan_decoupled_t(const Sys &d, int nblocks, uint32_t *s_b
         if (lane >= o) incl += t;
     }
     if (lane == 31) s_warp[wid] = incl;
-    __syncthreads();
+    scan_sync<NT, PART>();
     if (wid == 0) {
         uint32_t w = lane < NT / 32 ? s_warp[lane] : 0u;
         uint32_t wi = w;
@@ -135,7 +145,7 @@ __device__ inline void scan_decoupled_t(const Sys &d, int nblocks, uint32_t *s_b
             if (bid == nblocks - 1) d.cstart[d.ncells] = excl + total;
         }
     }
-    __syncthreads();
+    scan_sync<NT, PART>();
     uint32_t run = s_excl + s_warp[wid] + (incl - sum);
 #pragma unroll 8
     for (int k = 0; k < IPT; ++k) {
@@ -144,7 +154,7 @@ __device__ inline void scan_decoupled_t(const Sys &d, int nblocks, uint32_t *s_b
         s_buf[i] = run;
         run += c;
     }
-    __syncthreads();
+    scan_sync<NT, PART>();
 #pragma unroll 4
     for (int k = 0; k < IPT; ++k) {
         const int e = k * NT + tid, idx = base + e;
@@ -156,7 +166,7 @@ __device__ inline void scan_decoupled_t(const Sys &d, int nblocks, uint32_t *s_b
         double *th = d.thermo + 4 * (size_t)(s1 % THERMO_CAP);
         th[0] = 0.0; th[1] = 0.0; th[2] = 0.0; th[3] = 0.0;
     }
-    __syncthreads();   // s_buf is free again for the caller
+    scan_sync<NT, PART>();   // s_buf is free again for the caller
 }
 
 
@@ -188,7 +198,16 @@ __device__ __forceinline__ void bin_one(const Sys &d, int k)
 
 // ------------------------------------------------------------- integrate ----
 // Thermo partials of one thread, FP64: sum |v|^2, sum v_x, sum v_y.
-struct Thermo3 { double ke, px, py; };
+struct Thermo3 {
+    double ke, px, py;
+    __device__ __forceinline__ void add(float vx, float vy)
+    {
+        const double dvx = (double)vx, dvy = (double)vy;
+        ke = fma(dvx, dvx, fma(dvy, dvy, ke));
+        px += dvx;
+        py += dvy;
+    }
+};
 
 // Pair forces are summed per bead in fixed point, 2^-24 force units per
 // count.  Integer addition is associative, so a bead's force does not depend
@@ -217,49 +236,58 @@ __device__ __forceinline__ float fq_load(const int *a, int fs)
     return fq_to_f((long long)a[0] * 65536ll + (long long)(unsigned)a[fs]);
 }
 
+// Position of a bead's bonded partner through its sorted slot; false (and the
+// error word) if that slot is not a bead.  id < n.
+__device__ __forceinline__ bool partner_global(const Sys &d, int g, uint32_t id, uint2 &xp)
+{
+    const uint32_t ps = d.slot[id ^ 1u];
+    if (ps >= (uint32_t)d.n) {
+        set_err_at(d, ERR_INTERNAL, 2, g, id, ps);
+        return false;
+    }
+    const uint4 p = d.S_xv[ps];
+    xp = make_uint2(p.x, p.y);
+    return true;
+}
+
 // Everything after the pair sum for one owned bead at sorted slot g:
-// bond + propulsion (partner through slot[id ^ 1]), drag, the two half kicks
+// bond + propulsion (partner at xp when `bond`), drag, the two half kicks
 // and the drift, canonical output, binning of the new position.
+// The bead's rank in its new cell comes back from an atomic: it is stored by
+// the next call, or by the caller at the end, so that the round trip passes
+// behind the next bead's work.
 // Every floating-point operation of the step is written with an explicit
 // rounding (fused where a fused multiply-add is meant), so that the kernels
 // that inline this code, whose flags the compiler may or may not know, all
 // produce the same bits.
-template <int B>
-__device__ __forceinline__ void integrate_bead(const Sys &d, int g, uint4 xv, uint32_t id, float fx, float fy,
-                                               int flags, Thermo3 &th)
+struct RankLater {
+    int g;
+    uint32_t rank;
+    __device__ __forceinline__ void store(const Sys &d) const { if (g >= 0) d.U_rank[g] = rank; }
+};
+template <int B, typename THERMO>
+__device__ __forceinline__ void integrate_bead_at(const Sys &d, int g, uint4 xv, uint32_t id, bool bond, uint2 xp,
+                                                  float fx, float fy, int flags, THERMO &th, RankLater &later)
 {
-    if (id >= (uint32_t)d.n) {
-        set_err_at(d, ERR_INTERNAL, 7, g, id, d.n);
-        return;
-    }
-    const uint32_t ps = d.slot[id ^ 1u];
-    if (ps < (uint32_t)d.n) {
-        const uint4 xp = d.S_xv[ps];
+    if (bond) {
         const float dx = mdiff(d, xv.x, xp.x);
         const float dy = mdiff(d, xv.y, xp.y);
         const float r2 = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
         if (r2 > 0.f) {
             const float r = __fsqrt_rn(r2);
-            const float inv = __fdiv_rn(1.0f, r);
+            const float inv = __frcp_rn(r);
             const float ex = __fmul_rn(dx, inv), ey = __fmul_rn(dy, inv);   // from partner to self
             const float fb = __fmul_rn(-d.kbond, __fsub_rn(r, d.r0));
             const float sp = (id & 1u) ? -d.fp : d.fp;                        // n_k = head - tail
             fx = __fmaf_rn(__fadd_rn(fb, sp), ex, fx);
             fy = __fmaf_rn(__fadd_rn(fb, sp), ey, fy);
         }
-    } else {
-        set_err_at(d, ERR_INTERNAL, 2, g, id, ps);
     }
     float vx = vbits(xv.z), vy = vbits(xv.w);
     fx = __fmaf_rn(-d.zeta, vx, fx);
     fy = __fmaf_rn(-d.zeta, vy, fy);
     if (!(flags & F_FIRST)) { vx = __fmaf_rn(d.hdtm, fx, vx); vy = __fmaf_rn(d.hdtm, fy, vy); }
-    {
-        const double dvx = (double)vx, dvy = (double)vy;
-        th.ke = fma(dvx, dvx, fma(dvy, dvy, th.ke));
-        th.px += dvx;
-        th.py += dvy;
-    }
+    th.add(vx, vy);
     if (flags & F_FINAL) {
         d.C_xv[id] = make_uint4(xv.x, xv.y, fbits(vx), fbits(vy));
         d.C_f[id] = make_float2(fx, fy);
@@ -277,10 +305,28 @@ __device__ __forceinline__ void integrate_bead(const Sys &d, int g, uint4 xv, ui
             vx = 0.f; vy = 0.f;
         }
         const int c = cell_of<B>(d, cell_coord(d, nx), cell_coord(d, ny));
-        d.U_rank[g] = atomicAdd(&d.counts[c], 1u);
+        later.store(d);
+        later.g = g;
+        later.rank = atomicAdd(&d.counts[c], 1u);
         d.U_xv[g] = make_uint4(nx, ny, fbits(vx), fbits(vy));
         d.U_id[g] = id;
     }
+}
+
+// The same with the partner looked up through its slot.
+template <int B>
+__device__ __forceinline__ void integrate_bead(const Sys &d, int g, uint4 xv, uint32_t id, float fx, float fy,
+                                               int flags, Thermo3 &th)
+{
+    if (id >= (uint32_t)d.n) {
+        set_err_at(d, ERR_INTERNAL, 7, g, id, d.n);
+        return;
+    }
+    uint2 xp = make_uint2(0u, 0u);
+    const bool bond = partner_global(d, g, id, xp);
+    RankLater later{-1, 0u};
+    integrate_bead_at<B>(d, g, xv, id, bond, xp, fx, fy, flags, th, later);
+    later.store(d);
 }
 
 // ------------------------------------------------------------- pair force ----
@@ -309,7 +355,8 @@ __device__ __forceinline__ float dpd_pair_scalar(const Sys &d, float ux, float u
                                                  uint32_t idi, uint32_t idj, uint32_t s_lo, uint32_t s_hi,
                                                  float &ex, float &ey)
 {
-    const float rinv = rsqrtf(r2u);
+    float rinv;   // r2u is at least 1 (whole units), so the flush of denormals changes nothing
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rinv) : "f"(r2u));
     const float w = __fmaf_rn(-__fmul_rn(r2u, rinv), d.inv_rcu, 1.0f);
     ex = __fmul_rn(ux, rinv);
     ey = __fmul_rn(uy, rinv);
@@ -338,12 +385,25 @@ __device__ __forceinline__ void pair_force_q(const Sys &d, uint2 xi, uint2 xj, f
 
 // ------------------------------------------------------------ force tile ----
 // Shared-memory plan of one tile (B x B owned cells + one-cell halo) for the
-// variants that stage owned beads first (1, 2, 4).  Variant 4 adds, per owned
-// cell, its merged candidate ranges (FLAT_MAXI at most) and a per-warp table
-// of the 32 ranges being enumerated.
+// variants that stage owned beads first (1, 4, 5).  Variants 4 and 5 add, per
+// owned cell, its merged candidate ranges (FLAT_MAXI at most), variant 4 a
+// per-warp table of the 32 ranges being enumerated.
 constexpr int TILE_THREADS = 128;
+// Most threads a tile is launched with (variant 2 takes d.nt of them, by its
+// mean population; the others TILE_THREADS), and the tiles per SM that the
+// registers are bounded for at that many.
+template <int B, int VAR>
+__host__ __device__ constexpr int tile_threads()
+{
+    return VAR != 2 ? TILE_THREADS : B == 16 ? 384 : B == 8 ? 192 : 128;
+}
+template <int B, int VAR>
+__host__ __device__ constexpr int tile_ctas()
+{
+    return VAR != 2 ? 10 : B == 16 ? 3 : B == 8 ? 6 : 9;
+}
 constexpr int FLAT_MAXI = 6;
-template <int B, int VAR = 2>
+template <int B, int VAR>
 struct TilePlan {
     static constexpr int NCL = (B + 2) * (B + 2);   // local cell table
     static constexpr int NH = 4 * B + 4;            // halo cells
@@ -365,28 +425,13 @@ struct TilePlan {
     {
         return (bead_off(nthreads) + (size_t)cap * bead_bytes(count) + 15) & ~size_t(15);
     }
-    // variant 2: per owned cell, its walk descriptor (local cell index, the
-    // neighbour cells owned by the tile and the ones it visits), so a lane
-    // starting a bead reads it instead of deriving it
-    static constexpr bool DESC = VAR == 2;
-    static __host__ __device__ size_t desc_off(int cap, int nthreads, bool count)
+    static __host__ __device__ size_t bytes(int cap, int nthreads, bool count)
     {
         return queue_off(cap, nthreads, count) + (size_t)WARP_BYTES * (size_t)(nthreads / 32);
     }
-    // variant 2 on 8 x 8 blocks: the order in which the tile's lanes take
-    // owned beads (u16 each; measured faster there, slower on 16 x 16)
-    static constexpr bool ORDER = VAR == 2 && B == 8;
-    static __host__ __device__ size_t order_off(int cap, int nthreads, bool count)
-    {
-        return desc_off(cap, nthreads, count) + (DESC ? 4 * (size_t)(B * B) : 0);
-    }
-    static __host__ __device__ size_t bytes(int cap, int nthreads, bool count)
-    {
-        return order_off(cap, nthreads, count) + (ORDER ? 2 * (size_t)cap : 0);
-    }
 };
 
-// Shared arrays of a staged tile (variants 1 and 2): cap beads, cap a multiple
+// Shared arrays of a staged tile: cap beads, cap a multiple
 // of 32 so every array starts 16-byte aligned.
 struct TileArrays {
     uint2 *X;          // fixed-point position
@@ -469,14 +514,8 @@ __device__ __forceinline__ void pairs_thread(const Sys &d, int n_own, int tw, in
     }
 }
 
-// Variant 2: pair queue.  Each lane walks the candidates of one owned bead at
-// a time (taking the next bead from a block-wide counter when it runs out, so
-// warps stay balanced; on 8 x 8 blocks the counter runs through `order`,
-// which lists the beads of the cells that also visit halo cells behind them
-// first, so that the shortest walks come last and the lanes finish closer
-// together); every candidate
-// inside r_c is pushed, packed as
-// (i, j, Newton-3 flag), into the warp's 128-entry buffer.  Whenever 32 pairs
+// The pair queue of variants 4 and 5: every candidate inside r_c is pushed,
+// packed as (i, j, Newton-3 flag), into the warp's buffer.  Whenever 32 pairs
 // are queued the whole warp evaluates them together, so the Philox and force
 // arithmetic runs with every lane active.  Forces land in shared memory
 // through fixed-point atomics on both sides of a Newton-3 pair.
@@ -516,83 +555,6 @@ __device__ __forceinline__ void queue_drain(volatile uint32_t *q, int &qn, EVAL 
         __syncwarp();
         eval(mine);
     }
-}
-
-template <int B, bool COUNT>
-__device__ __forceinline__ void pairs_queue(const Sys &d, int n_own, const int *s_cbeg, const int *s_ccnt,
-                                            const TileArrays &t, volatile uint32_t *q, int *s_next, uint32_t s_lo,
-                                            uint32_t s_hi, const uint32_t *desc, const uint16_t *order)
-{
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    int k = -1, j = 0, je = 0, lc0 = 0;
-    uint32_t visit = 0, own = 0, pid = 0, tag = 0;
-    uint2 xi = make_uint2(0u, 0u);
-    bool more = true;
-    int qn = 0;   // warp-uniform queue length (entries q[0, qn))
-    auto eval = [&](uint32_t code) { queue_eval<COUNT>(d, code, t, s_lo, s_hi); };
-    while (true) {
-        // At most one advance per lane per round (to the next neighbour
-        // range of its bead, or to its next bead), so a lane switching cells
-        // costs the warp one short divergent step instead of a loop.
-        bool have = j < je;
-        if (!have && more) {
-            if (visit == 0u) {
-                k = atomicAdd(s_next, 1);
-                if (k >= n_own) {
-                    more = false;
-                } else {
-                    if constexpr (TilePlan<B, 2>::ORDER) k = order[k];
-                    xi = t.X[k];
-                    const uint32_t lcb = t.lc[k];
-                    const uint32_t dsc = desc[(lcb >> 4) * B + (lcb & 15u)];
-                    lc0 = (int)(dsc & 0x1ffu);
-                    own = (dsc >> 9) & 0x1ffu;
-                    visit = dsc >> 18;
-                    pid = d.excl ? (t.id[k] ^ 1u) : 0xffffffffu;
-                }
-            }
-            if (more) {
-                const int nb = __ffs(visit) - 1;
-                visit &= visit - 1u;
-                const int ox_ = (int)((NB_DX >> (2 * nb)) & 3u) - 1, oy_ = (int)((NB_DY >> (2 * nb)) & 3u) - 1;
-                const int lc = lc0 + oy_ * (B + 2) + ox_;
-                j = s_cbeg[lc];
-                je = j + s_ccnt[lc];
-                if (nb == 0) j = k + 1;
-                tag = (uint32_t)k | (((own >> nb) & 1u) << 24);
-                have = j < je;
-            }
-        }
-        if (!__any_sync(FULL, have || more)) break;
-        // two candidates per lane per round (j and j + 1 while in range),
-        // tested branch-free; one append point per round
-        bool p0 = false, p1 = false;
-        uint32_t c0 = 0, c1 = 0;
-        if (have) {
-            const uint2 xj = t.X[j];
-            p0 = in_range(d, xi.x, xi.y, xj.x, xj.y) & (t.id[j] != pid);
-            c0 = tag | ((uint32_t)j << 12);
-            ++j;
-            if (j < je) {
-                const uint2 xk = t.X[j];
-                p1 = in_range(d, xi.x, xi.y, xk.x, xk.y) & (t.id[j] != pid);
-                c1 = tag | ((uint32_t)j << 12);
-                ++j;
-            }
-        }
-        const unsigned m0 = __ballot_sync(FULL, p0);
-        const unsigned m1 = __ballot_sync(FULL, p1);
-        const int n0 = __popc(m0);
-        if (p0) q[qn + __popc(m0 & lt)] = c0;
-        if (p1) q[qn + n0 + __popc(m1 & lt)] = c1;
-        qn += n0 + __popc(m1);
-        __syncwarp();
-        queue_drain<2>(q, qn, eval);
-    }
-    __syncwarp();
-    if (lane < qn) eval(q[lane]);
 }
 
 // Variant 4: flat enumeration.  Every owned cell has a short list of candidate
@@ -752,8 +714,8 @@ __device__ __forceinline__ void pairs_flat(const Sys &d, int n_own, int total, i
     if (lane < qn) eval(q[lane]);
 }
 
-// Variant 5: the lane walk of variant 2 over the merged candidate ranges of
-// variant 4's cell tables.  A lane holds one range of one bead; when it runs
+// Variant 5: a lane walk over the merged candidate ranges of variant 4's cell
+// tables.  A lane holds one range of one bead; when it runs
 // out it takes the next range of its bead (or the next bead), one step per
 // round, so a bead costs about 2.3 range switches instead of one per
 // neighbour cell; every round each lane tests CPR candidates and the pairs
@@ -869,6 +831,29 @@ __device__ void force_tile_global(const Sys &d, uint32_t g0, int n_own, uint32_t
     }
 }
 
+// Block reduction of a tile's thermo partials into the FP64 ring slot of
+// `step` (FP64 throughout): every thread's partials to shared memory (buf,
+// 3 blockDim doubles), then warp q adds quantity q (blockDim / 32 values per
+// lane, then across its lanes) and adds it to the slot.  A third of the FP64
+// additions of a shuffle tree in every warp (the FP64 pipe is narrow on this
+// part).  buf is read by warps 0-2 after the call: the caller synchronises
+// before reusing it.
+__device__ __forceinline__ void thermo_flush_tile(const Sys &d, Thermo3 th, double *buf)
+{
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nt = blockDim.x;
+    buf[tid] = th.ke;
+    buf[nt + tid] = th.px;
+    buf[2 * nt + tid] = th.py;
+    __syncthreads();
+    if (wid < 3) {
+        double a = 0.0;
+        for (int i = lane; i < nt; i += 32) a += buf[wid * nt + i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) atomicAdd(&d.thermo[4 * (size_t)(*d.step % THERMO_CAP) + wid], a);
+    }
+}
+
 // ------------------------------------------------- grid-order tile (VAR 3) --
 // The tile's owned and halo cells are staged in shared memory in the row-major
 // order of the local (B+2) x (B+2) cell grid, so every row of the local grid is
@@ -877,7 +862,7 @@ __device__ void force_tile_global(const Sys &d, uint32_t g0, int n_own, uint32_t
 // cell on the tile edge adds at most three ranges of halo cells behind it (W,
 // and SW..SE or parts of that row).  Each lane walks the candidates of one
 // owned bead at a time, CPR candidates per round; pairs inside r_c go through
-// the warp's pair queue as in variant 2 (Newton-3 when the partner is owned).
+// the warp's pair queue (Newton-3 when the partner is owned).
 template <int B>
 struct TilePlanG {
     static constexpr int W = B + 2;
@@ -1147,6 +1132,595 @@ __device__ void force_tile_g(const Sys &d, int tile, int flags, unsigned char *s
     }
 }
 
+// --------------------------------------------- candidate-mask tile (VAR 2) --
+// The default shape.  The tile's owned and halo cells are staged in the
+// row-major order of the local (B + 2) x (B + 2) cell grid, so every row of
+// the grid is one contiguous run of bead slots and a bead's forward half
+// stencil is two runs: the rest of its cell and the cell east of it, and the
+// three cells north of it.  The halo cells behind the tile (left and right
+// columns, bottom row) walk their own forward runs clipped to owned cells, so
+// every pair with an owned bead is met once and no bead has more than two runs.
+//
+// What bounds it: instruction issue.  A walk that advances, tests and queues
+// candidate by candidate spends its instructions on the control around the
+// test; here a lane tests a run of up to 32 slots with no control flow, two
+// candidates per half2 operation, into a 32-bit mask, and control runs once
+// per hit instead (5 hits of 14 candidates per bead at density 3).  The
+// half-precision test works on cell-relative offsets and is a little wider
+// than r_c; every pair it passes takes the exact test before evaluation.
+//
+// 1024 x 1024 cells at density 3: 76 warp instructions per bead against 105 for
+// a walk that tests and queues candidate by candidate, 246 us against 308.
+//
+// The pair (2k, 2k + 1) of an agent is met like any other when its beads lie
+// within r_c; the evaluation then records the two slots for each other, and
+// the integration takes the partner's position from shared memory.  Only a
+// bond longer than r_c goes through slot[] and the sorted state.
+template <int B>
+struct TilePlanM {
+    static constexpr int W = B + 2;
+    static constexpr int NCL = W * W;
+    static constexpr int NINT = 2 * NCL + 1;       // begins (+1), global sources
+    static constexpr int QLEN = 192;               // queued pairs per warp
+    static constexpr int PAD = 32;                 // slots a window may read past the last bead
+    static __host__ __device__ size_t rng_off() { return ((size_t)NINT * 4 + 15) & ~size_t(15); }
+    static __host__ __device__ size_t bead_off(int) { return (rng_off() + 8 * (size_t)NCL + 15) & ~size_t(15); }
+    // per staged bead: state 16, force counts 16, id 4, half2 offset 4,
+    // partner slot 2, local cell 2, slot of an owned bead 2 (+ count 4)
+    static __host__ __device__ size_t bead_bytes(bool count) { return count ? 50 : 46; }
+    static __host__ __device__ size_t queue_off(int cap, int, bool count)
+    {
+        return (bead_off(0) + (size_t)cap * bead_bytes(count) + 4 * PAD + 15) & ~size_t(15);
+    }
+    static __host__ __device__ size_t bytes(int cap, int nthreads, bool count)
+    {
+        return queue_off(cap, nthreads, count) + sizeof(uint32_t) * QLEN * (size_t)(nthreads / 32);
+    }
+};
+
+constexpr uint32_t NO_SLOT = 0xffffu;
+
+struct TileM {
+    uint4 *xv;          // (X, Y, v*x, v*y)
+    int *f;             // force counts, one array per word (x hi, x lo, y hi, y lo), fs apart
+    int fs;
+    uint32_t *id;
+    uint2 *pos;         // slots 2 p and 2 p + 1: (half2 of x, half2 of y), cell units from the tile's middle
+    uint32_t *pl;       // local cell | slot of the bonded partner << 16 (NO_SLOT until met)
+    uint16_t *oslot;    // slot of owned bead k
+    uint32_t *cnt;      // interacting neighbours (COUNT only)
+};
+
+// A force component g (|g| < FQ_MAX) as hi 2^18 + lo counts of 2^-24, the same
+// count as fq's: hi is g in units of 2^-6 to the nearest whole number, lo the
+// exact rest in counts, rounded.  Adding 1.5 2^23 rounds a magnitude below 2^22
+// to a whole number whose bits are the sum's low bits, so this takes FP32 and
+// integer instructions alone (the 64-bit conversion runs on the FP64 pipe,
+// which is one lane wide on this part).
+__device__ __forceinline__ void fq_split(float g, int &hi, int &lo)
+{
+    constexpr float M = 12582912.0f;
+    constexpr int MI = 0x4B400000;
+    const float t = __fmaf_rn(g, 64.0f, M);
+    hi = __float_as_int(t) - MI;
+    lo = __float_as_int(__fmaf_rn(__fmaf_rn(g, 64.0f, __fsub_rn(M, t)), 262144.0f, M)) - MI;
+}
+
+// One queued pair of slots: exact range test, force on both sides (a halo
+// bead's sums are dropped), bonded partners recorded.
+template <bool COUNT>
+__device__ __forceinline__ void mask_eval(const Sys &d, uint32_t code, const TileM &t, uint32_t s_lo, uint32_t s_hi,
+                                          bool &bad)
+{
+    const uint32_t k = code & 0xffffu, j = code >> 16;
+    const uint32_t ik = t.id[k], ij = t.id[j];
+    const uint4 xk = t.xv[k], xj = t.xv[j];
+    const float ux = sep_u(xk.x, xj.x), uy = sep_u(xk.y, xj.y);
+    const float r2u = r2_u(ux, uy);
+    bool on = (r2u < d.rc2u) & (r2u > 0.f);
+    if ((ik ^ ij) == 1u) {
+        reinterpret_cast<uint16_t *>(t.pl)[2 * k + 1] = (uint16_t)j;
+        reinterpret_cast<uint16_t *>(t.pl)[2 * j + 1] = (uint16_t)k;
+        on = on & (d.excl == 0);
+    }
+    if (!on) return;
+    float ex, ey;
+    const float F = dpd_pair_scalar(d, ux, uy, r2u, __fsub_rn(vbits(xk.z), vbits(xj.z)),
+                                    __fsub_rn(vbits(xk.w), vbits(xj.w)), ik, ij, s_lo, s_hi, ex, ey);
+    bad |= !(fabsf(F) < FQ_MAX);
+    int xh, xl, yh, yl;
+    fq_split(__fmul_rn(F, ex), xh, xl);
+    fq_split(__fmul_rn(F, ey), yh, yl);
+    int *a = t.f + k, *b = t.f + j;
+    atomicAdd(a, xh);
+    atomicAdd(a + t.fs, xl);
+    atomicAdd(a + 2 * t.fs, yh);
+    atomicAdd(a + 3 * t.fs, yl);
+    atomicAdd(b, -xh);
+    atomicAdd(b + t.fs, -xl);
+    atomicAdd(b + 2 * t.fs, -yh);
+    atomicAdd(b + 3 * t.fs, -yl);
+    if (COUNT) {
+        atomicAdd(&t.cnt[k], 1u);
+        atomicAdd(&t.cnt[j], 1u);
+    }
+}
+
+__device__ __forceinline__ float fq_load_s(const int *a, int fs)
+{
+    return fq_to_f((long long)a[0] * 262144ll + (long long)a[fs]);
+}
+
+// Two candidates against one bead: 0xffff in the half of each within thr.
+__device__ __forceinline__ uint32_t near2(__half2 xi, __half2 yi, __half2 thr, uint2 p)
+{
+    const __half2 dx = __hsub2(*reinterpret_cast<const __half2 *>(&p.x), xi);
+    const __half2 dy = __hsub2(*reinterpret_cast<const __half2 *>(&p.y), yi);
+    return __hle2_mask(__hfma2(dy, dy, __hmul2(dx, dx)), thr);
+}
+
+// Mask of the slots [a, a + 8 n) (a even, n <= 4 blocks of four slot pairs)
+// within thr: bit p < 16 is slot a + 2 p, bit 16 + p slot a + 2 p + 1.  The
+// blocks go from the last to the first, so that each is shifted in with
+// constant bit positions.
+__device__ __forceinline__ uint32_t near_mask(const uint2 *pos, uint32_t a, int n, __half2 xi, __half2 yi, __half2 thr)
+{
+    uint32_t m = 0u;
+    const uint2 *p = pos + (a >> 1) + 4 * n;
+#pragma unroll 1
+    for (int q = 0; q < n; ++q) {
+        p -= 4;
+        uint32_t b = near2(xi, yi, thr, p[0]) & 0x00010001u;
+        b |= near2(xi, yi, thr, p[1]) & 0x00020002u;
+        b |= near2(xi, yi, thr, p[2]) & 0x00040004u;
+        b |= near2(xi, yi, thr, p[3]) & 0x00080008u;
+        m = (m << 4) | b;
+    }
+    return m;
+}
+// Bits of the first len (0..32) slots of such a mask.
+__device__ __forceinline__ uint32_t first_bits(int len)
+{
+    uint32_t even, odd;
+    asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(even) : "r"((len + 1) >> 1));
+    asm("bmsk.clamp.b32 %0, 16, %1;" : "=r"(odd) : "r"(len >> 1));
+    return even | odd;
+}
+// Position of the highest set bit (all ones for 0).
+__device__ __forceinline__ uint32_t top_bit(uint32_t x)
+{
+    uint32_t p;
+    asm("bfind.u32 %0, %1;" : "=r"(p) : "r"(x));
+    return p;
+}
+__device__ __forceinline__ uint32_t bit_at(uint32_t p)   // 0 for p above 31
+{
+    uint32_t b;
+    asm("shl.b32 %0, 1, %1;" : "=r"(b) : "r"(p));
+    return b;
+}
+// Append the slots of a mask to `to` as codes c + (slot - a) 2^16; the even
+// and the odd slots go side by side.
+__device__ __forceinline__ void append_mask(uint32_t m, uint32_t c, uint32_t *&to)
+{
+    uint32_t ev = m & 0xffffu, od = m >> 16;
+    const int rounds = __reduce_max_sync(0xffffffffu, max(__popc(ev), __popc(od)));
+#pragma unroll 1
+    for (int r = 0; r < rounds; ++r) {
+        const uint32_t p = top_bit(ev), o = top_bit(od);
+        if (ev) *to++ = c + (p << 17);
+        if (od) *to++ = c + 0x10000u + (o << 17);
+        ev ^= bit_at(p);
+        od ^= bit_at(o);
+    }
+}
+
+// Every pair of the tile: a warp takes 32 slots at a time, masks both runs of
+// each (in windows of 32 slots), and appends the hits to its queue q of QLEN
+// entries; then the full warps among the queued pairs are evaluated (at most
+// 31 pairs stay queued) and, when no slots are left, the rest.  A lane knows
+// where its hits go from a scan of the hit counts, so a hit costs its bit, its
+// slot and its store.  A bead's hits lie side by side in the queue, so the
+// evaluation of nb full warps takes every nb-th entry: the atomics of a warp
+// then rarely meet on one bead (side by side they cost 1.7 times the shared
+// wavefronts).
+template <bool COUNT, int QLEN>
+__device__ __forceinline__ void pairs_mask(const Sys &d, uint32_t n_items, const TileM &t, const uint2 *s_rng,
+                                           __half2 thr, uint32_t *q, uint32_t s_lo, uint32_t s_hi)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    uint32_t qn = 0;   // warp-uniform
+    bool bad = false, more = true, next = true;
+    // a*: first slot (even) and l*: slots left of the lane's two runs
+    uint32_t s = threadIdx.x, cut1 = 0, cut2 = 0;
+    int a1 = 0, l1 = 0, a2 = 0, l2 = 0;
+    __half2 xi = __half2half2(__ushort_as_half(0)), yi = xi;
+    do {
+        uint32_t m1 = 0u, m2 = 0u, end = 0u;
+        uint32_t hits = 0;   // warp-uniform
+        if (next) {   // the warp's next 32 slots
+            more = s - (uint32_t)lane < n_items;
+            l1 = l2 = 0;
+            if (s < n_items) {
+                const uint2 r = s_rng[t.pl[s] & 0xffffu];
+                const int b1 = max((int)(r.x & 0xffffu), (int)s + 1), e1 = (int)(r.x >> 16);
+                const int b2 = (int)(r.y & 0xffffu), e2 = (int)(r.y >> 16);
+                a1 = b1 & ~1;
+                a2 = b2 & ~1;
+                l1 = b1 < e1 ? e1 - a1 : 0;
+                l2 = b2 < e2 ? e2 - a2 : 0;
+                cut1 = ~(uint32_t)(b1 & 1);
+                cut2 = ~(uint32_t)(b2 & 1);
+                const uint2 p = t.pos[s >> 1];
+                const int sh = (int)(s & 1u) * 16;
+                xi = __half2half2(__ushort_as_half((unsigned short)(p.x >> sh)));
+                yi = __half2half2(__ushort_as_half((unsigned short)(p.y >> sh)));
+            }
+        }
+        if (more) {
+            const int w1 = min(l1, 32), w2 = min(l2, 32);
+            const int n1 = (__reduce_max_sync(FULL, w1) + 7) >> 3, n2 = (__reduce_max_sync(FULL, w2) + 7) >> 3;
+            // a lane past a run reads from slot 0 on
+            m1 = near_mask(t.pos, w1 ? a1 : 0, n1, xi, yi, thr) & first_bits(w1) & cut1;
+            m2 = near_mask(t.pos, w2 ? a2 : 0, n2, xi, yi, thr) & first_bits(w2) & cut2;
+            end = (uint32_t)(__popc(m1) + __popc(m2));
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(FULL, end, o);
+                if (lane >= o) end += v;
+            }
+            hits = __shfl_sync(FULL, end, 31);
+        }
+        const uint32_t c1 = s | ((uint32_t)a1 << 16), c2 = s | ((uint32_t)a2 << 16);
+        uint32_t done = 0;
+        while (true) {
+            // append the hits of the next lanes, as many as fit whole (a lane
+            // has 64 at most and 31 pairs wait)
+            if (hits != done) {
+                const uint32_t lim = done + (uint32_t)QLEN - qn;
+                const bool go = end <= lim && end > done;
+                const uint32_t x1 = go ? m1 : 0u, x2 = go ? m2 : 0u;
+                uint32_t *to = q + qn + end - done - (uint32_t)(__popc(x1) + __popc(x2));
+                append_mask(x1, c1, to);
+                append_mask(x2, c2, to);
+                const uint32_t upto = hits <= lim ? hits : __reduce_max_sync(FULL, go ? end : done);
+                qn += upto - done;
+                done = upto;
+                __syncwarp();
+            }
+            const uint32_t nb = more ? qn >> 5 : (qn + 31u) >> 5;
+#pragma unroll 1
+            for (uint32_t b = 0; b < nb; ++b) {
+                const uint32_t i = (uint32_t)lane * nb + b;
+                if (i < qn) mask_eval<COUNT>(d, q[i], t, s_lo, s_hi, bad);
+            }
+            if (nb) {
+                const uint32_t left = q[(nb << 5) + lane < (uint32_t)QLEN ? (nb << 5) + lane : 0u];
+                __syncwarp();
+                qn = more ? qn & 31u : 0u;
+                if ((uint32_t)lane < qn) q[lane] = left;
+                __syncwarp();
+            }
+            if (done == hits) break;
+        }
+        next = !__any_sync(FULL, (l1 > 32) | (l2 > 32));
+        if (next) {
+            s += blockDim.x;
+        } else {
+            l1 = max(l1 - 32, 0);
+            l2 = max(l2 - 32, 0);
+            a1 += 32;
+            a2 += 32;
+            cut1 = cut2 = ~0u;
+        }
+    } while (more);
+    if (bad) set_err(d, ERR_NONFINITE);
+}
+
+// Thermo partials of one thread as whole numbers: velocities scaled by a power
+// of two to v' (|v'| below `lim`, or the bead goes to the FP64 sums in `big`) are
+// split exactly into the nearest integer a and the rest r, |r| <= 1/2; then
+// v'^2 = a^2 + r (v' + a), the second term rounded to an integer.  The scale
+// comes from the tile's fastest bead (about 2^28 there), so the rounding is
+// 2^-57 of its v^2 at most, below that of the FP64 sums.  The FP64 pipe is
+// one lane wide on this part (32 cycles per warp instruction): FP64 partials
+// took 2,500 cycles of it per tile of 192 beads, these take 200.
+struct ThermoQ {
+    float sc, lim;      // scale, and the bound on |v'|
+    unsigned long long k;
+    long long px, py;   // 2^-24 units
+    double *big;        // shared: ke, px, py of beads out of the integer range
+    __device__ __forceinline__ void add(float vx, float vy)
+    {
+        const float wx = __fmul_rn(vx, sc), wy = __fmul_rn(vy, sc);
+        if (fabsf(wx) < lim && fabsf(wy) < lim) {   // false for NaN too
+            const int ax = __float2int_rn(wx), ay = __float2int_rn(wy);
+            const float bx = (float)ax, by = (float)ay;
+            const float rx = __fsub_rn(wx, bx), ry = __fsub_rn(wy, by);
+            const float er = __fmaf_rn(rx, __fadd_rn(wx, bx), __fmul_rn(ry, __fadd_rn(wy, by)));
+            k += (unsigned long long)((long long)ax * ax) + (unsigned long long)((long long)ay * ay) +
+                 (unsigned long long)(long long)__float2int_rn(er);
+            px += (long long)ax * 16777216 + __float2int_rn(__fmul_rn(rx, 16777216.0f));
+            py += (long long)ay * 16777216 + __float2int_rn(__fmul_rn(ry, 16777216.0f));
+        } else if (vx != 0.0f || vy != 0.0f) {
+            const double dvx = (double)vx, dvy = (double)vy;
+            atomicAdd(&big[0], fma(dvx, dvx, dvy * dvy));
+            atomicAdd(&big[1], dvx);
+            atomicAdd(&big[2], dvy);
+        }
+    }
+};
+
+// Scale of ThermoQ for a tile whose largest |v*| component has the bits vmax
+// and whose threads add up to `beads` beads each: |v'| below 2^28 at vmax and
+// four times that to the limit (a bit less for every four times more beads
+// than four, so that a thread's a^2 sums stay below 2^63).  Outside the
+// exponents that scale within FP32 (a tile at rest, or blown up) the scale is
+// infinite and every moving bead takes the FP64 sums.
+__device__ __forceinline__ ThermoQ thermo_q(uint32_t vmax, int beads, double *big)
+{
+    const int e = (int)(vmax >> 23);
+    if (e < 40 || e > 200) return ThermoQ{__int_as_float(0x7f800000), 0.0f, 0ull, 0ll, 0ll, big};
+    int up = 28;
+    for (int b = 4; b < beads; b *= 4) --up;
+    return ThermoQ{__int_as_float((127 + up - (e - 126)) << 23), __int_as_float((127 + up + 2) << 23), 0ull, 0ll, 0ll,
+                   big};
+}
+
+// Block sum of the ThermoQ partials into the FP64 ring slot: each 64-bit
+// partial as limbs of 22 bits whose warp sums fit in 32, then three threads put
+// the limb sums together.  buf: 9 words per warp, free on entry (the caller has
+// synchronised); big as in ThermoQ.
+__device__ __forceinline__ void thermo_flush_q(const Sys &d, const ThermoQ &th, int *buf)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    const long long q[3] = {(long long)th.k, th.px, th.py};   // k is below 2^63
+    int *mine = buf + 9 * wid;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int q0 = (int)__reduce_add_sync(FULL, (unsigned)(q[i] & 0x3fffffll));
+        const int q1 = (int)__reduce_add_sync(FULL, (unsigned)((q[i] >> 22) & 0x3fffffll));
+        const int q2 = __reduce_add_sync(FULL, (int)(q[i] >> 44));
+        if (lane == 0) { mine[3 * i] = q0; mine[3 * i + 1] = q1; mine[3 * i + 2] = q2; }
+    }
+    __syncthreads();
+    if (tid < 3) {
+        long long s0 = 0, s1 = 0, s2 = 0;
+        for (int w = 0; w < nw; ++w) {
+            const int *l = buf + 9 * w + 3 * tid;
+            s0 += l[0];
+            s1 += l[1];
+            s2 += l[2];
+        }
+        // sc = 2^x: times 2^-2x (ke) or 2^-(x + 24); the sums of an infinite
+        // scale are all zero
+        const int x = (int)(__float_as_uint(th.sc) >> 23) - 127;
+        const int ex = th.lim == 0.0f ? 0 : (tid == 0 ? -2 * x : -x - 24);
+        const double inv = __hiloint2double((1023 + ex) << 20, 0);
+        const double a = fma((double)s2, 17592186044416.0, fma((double)s1, 4194304.0, (double)s0)) * inv;
+        const double b = th.big[tid];
+        atomicAdd(&d.thermo[4 * (size_t)(*d.step % THERMO_CAP) + tid], b != 0.0 ? a + b : a);
+    }
+}
+
+template <int B, bool COUNT>
+__device__ void force_tile_m(const Sys &d, int tile, int flags, unsigned char *smem)
+{
+    using TP = TilePlanM<B>;
+    constexpr int W = TP::W;
+    const int NT = blockDim.x, tid = threadIdx.x;
+    __shared__ double s_big[3];
+    __shared__ uint32_t s_vmax;
+    int *s_lbeg = (int *)smem;               // counts first, then begins in grid order
+    int *s_lsrc = s_lbeg + TP::NCL + 1;
+    uint2 *s_rng = (uint2 *)(smem + TP::rng_off());
+    const int cap = d.cap;
+    TileM t;
+    {
+        unsigned char *p = smem + TP::bead_off(NT);
+        t.xv = (uint4 *)p;
+        t.f = (int *)(p + 16 * (size_t)cap);
+        t.fs = cap;
+        t.id = (uint32_t *)(p + 32 * (size_t)cap);
+        t.pos = (uint2 *)(p + 36 * (size_t)cap);
+        p += 40 * (size_t)cap + 4 * TP::PAD;
+        t.pl = (uint32_t *)p;
+        t.oslot = (uint16_t *)(p + 4 * (size_t)cap);
+        t.cnt = (uint32_t *)(p + 6 * (size_t)cap);   // COUNT only
+    }
+
+    const int ty = tile / d.ntx, tx = tile - ty * d.ntx;
+    const int x0 = tx * B, y0 = ty * B;
+    const int tw = min(B, d.nc - x0), th_ = min(B, d.nc - y0);
+    const int base = y0 * d.nc + x0 * th_;
+    const uint32_t n = (uint32_t)d.n;
+    const long long step = *d.step;
+    const uint32_t s_lo = (uint32_t)((unsigned long long)step & 0xffffffffull);
+    const uint32_t s_hi = (uint32_t)((unsigned long long)step >> 32);
+    const uint32_t g0 = min(d.cstart[base], n);
+    const uint32_t g1 = max(g0, min(d.cstart[base + tw * th_], n));
+    const int n_own = (int)(g1 - g0);
+
+    // bead counts and global sources of the local grid (cells past the halo
+    // of a ragged tile stay empty)
+    for (int c = tid; c < TP::NCL; c += NT) {
+        const int ly = c / W - 1, lx = c - (ly + 1) * W - 1;
+        int cnt = 0, src = 0;
+        if (lx <= tw && ly <= th_) {
+            const bool owned = lx >= 0 && lx < tw && ly >= 0 && ly < th_;
+            int gc;
+            if (owned) {
+                gc = base + ly * tw + lx;
+            } else {
+                int cx = x0 + lx, cy = y0 + ly;
+                cx += cx < 0 ? d.nc : (cx >= d.nc ? -d.nc : 0);
+                cy += cy < 0 ? d.nc : (cy >= d.nc ? -d.nc : 0);
+                gc = cell_of<B>(d, cx, cy);
+            }
+            const uint32_t lo = owned ? g0 : 0u, hi = owned ? g1 : n;
+            const uint32_t b = min(max(d.cstart[gc], lo), hi), e = min(max(d.cstart[gc + 1], b), hi);
+            src = (int)b;
+            cnt = (int)(e - b);
+        }
+        s_lbeg[c] = cnt;
+        s_lsrc[c] = src;
+    }
+    for (int i = tid; i < cap; i += NT) reinterpret_cast<uint4 *>(t.f)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    if (tid < 32) {   // exclusive scan of the counts in grid order
+        constexpr int PER = (TP::NCL + 31) / 32;
+        int v[PER];
+        int sum = 0;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int c = tid * PER + i;
+            v[i] = c < TP::NCL ? s_lbeg[c] : 0;
+            sum += v[i];
+        }
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int tt = __shfl_up_sync(0xffffffffu, incl, o);
+            if (tid >= o) incl += tt;
+        }
+        int run = incl - sum;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int c = tid * PER + i;
+            if (c < TP::NCL) s_lbeg[c] = run;
+            run += v[i];
+        }
+        if (tid == 31) {
+            s_lbeg[TP::NCL] = incl;
+            s_vmax = 0u;
+            s_big[0] = s_big[1] = s_big[2] = 0.0;
+        }
+    }
+    __syncthreads();
+    const int total = s_lbeg[TP::NCL];
+
+    if (total <= cap && n_own <= total) {
+        // ---- forward runs per local cell: (begin | end << 16) of the first
+        // (a bead starts after itself) and of the second; halo cells are
+        // clipped to owned cells
+        for (int c = tid; c < TP::NCL; c += NT) {
+            const int ly = c / W - 1, lx = c - (ly + 1) * W - 1;
+            uint32_t r1 = 0u, r2 = 0u;
+            if (lx <= tw && ly < th_) {
+                const bool in = lx >= 0 && lx < tw && ly >= 0;
+                const int xa = in ? lx - 1 : max(lx - 1, 0), xb = in ? lx + 1 : min(lx + 1, tw - 1);
+                // second run: the row above, when it holds owned cells or the bead is owned
+                if (in || ly + 1 < th_) r2 = (uint32_t)s_lbeg[(ly + 2) * W + xa + 1] | ((uint32_t)s_lbeg[(ly + 2) * W + xb + 2] << 16);
+                // first run: the own cell and E, or E alone for the left column
+                if (in) r1 = (uint32_t)s_lbeg[c + 2] << 16;
+                else if (ly >= 0 && lx < 0) r1 = (uint32_t)s_lbeg[c + 1] | ((uint32_t)s_lbeg[c + 2] << 16);
+            }
+            s_rng[c] = make_uint2(r1, r2);
+        }
+        // ---- stage the local grid row by row, 2^rowl lanes per row, the loads
+        // of three rows in flight per lane (raw fixed point: a periodic image has the
+        // same coordinates modulo 2^32)
+        uint32_t vmax = 0u;
+        const int G = 1 << d.rowl, dr = NT >> d.rowl, ln = tid & (G - 1);
+        constexpr int U = 3;
+        for (int row0 = tid >> d.rowl; row0 < th_ + 2; row0 += U * dr) {
+            int left = 0;   // most beads of the rows
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int row = row0 + u * dr;
+                if (row < th_ + 2) left = max(left, s_lbeg[row * W + tw + 2] - s_lbeg[row * W]);
+            }
+            for (int l = ln; l < left; l += G) {
+                uint4 xv[U];
+                uint32_t id[U];
+                int src[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int row = row0 + u * dr;
+                    src[u] = -1;
+                    if (row >= th_ + 2) continue;
+                    const int *lb = s_lbeg + row * W, *lg = s_lsrc + row * W;
+                    const int s = lb[0] + l;
+                    if (s >= lb[tw + 2]) continue;
+                    const int c = s < lb[1] ? 0 : (s < lb[tw + 1] ? 1 : tw + 1);
+                    src[u] = (int)min((uint32_t)(s - lb[c] + lg[c]), n - 1);
+                    xv[u] = d.S_xv[src[u]];
+                    id[u] = d.S_id[src[u]];
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (src[u] < 0) continue;
+                    const int row = row0 + u * dr;
+                    const int *lb = s_lbeg + row * W;
+                    const int s = lb[0] + l;
+                    const bool west = s < lb[1], mid = !west && s < lb[tw + 1];
+                    // cell column and offset inside the cell: X n_c = cell 2^32 + offset
+                    const unsigned long long px = (unsigned long long)xv[u].x * (uint32_t)d.nc;
+                    const unsigned long long py = (unsigned long long)xv[u].y * (uint32_t)d.nc;
+                    const int lx = mid ? min(max((int)(px >> 32) - x0, 0), tw - 1) : (west ? -1 : tw);
+                    const float hx = __fmaf_rn((float)(uint32_t)px, 2.3283064365386963e-10f, (float)(lx - B / 2));
+                    const float hy = __fmaf_rn((float)(uint32_t)py, 2.3283064365386963e-10f, (float)(row - 1 - B / 2));
+                    t.xv[s] = xv[u];
+                    t.id[s] = id[u];
+                    __half *h = reinterpret_cast<__half *>(t.pos) + 4 * (s >> 1) + (s & 1);
+                    h[0] = __float2half_rn(hx);
+                    h[2] = __float2half_rn(hy);
+                    t.pl[s] = (uint32_t)(row * W + lx + 1) | (NO_SLOT << 16);
+                    if (mid && row >= 1 && row <= th_) {
+                        t.oslot[src[u] - (int)g0] = (uint16_t)s;
+                        vmax = max(vmax, max(xv[u].z & 0x7fffffffu, xv[u].w & 0x7fffffffu));
+                    }
+                    if (COUNT) t.cnt[s] = 0u;
+                }
+            }
+        }
+        vmax = __reduce_max_sync(0xffffffffu, vmax);
+        if ((tid & 31) == 0) atomicMax(&s_vmax, vmax);
+        __syncthreads();
+
+        // ---- pair forces (every row but the top halo row has forward runs)
+        pairs_mask<COUNT, TP::QLEN>(d, (uint32_t)s_lbeg[(th_ + 1) * W], t, s_rng,
+                                    __half2half2(__float2half_ru(d.near2)),
+                                    (uint32_t *)(smem + TP::queue_off(cap, NT, COUNT)) + TP::QLEN * (tid >> 5), s_lo,
+                                    s_hi);
+        __syncthreads();
+
+        // ---- integrate owned beads
+        ThermoQ th = thermo_q(s_vmax, (n_own + NT - 1) / NT, s_big);
+        RankLater later{-1, 0u};
+        for (int k = tid; k < n_own; k += NT) {
+            const int g = (int)g0 + k, s = min((int)t.oslot[k], total - 1);
+            const uint4 xv = t.xv[s];
+            const uint32_t id = t.id[s], ps = t.pl[s] >> 16;
+            if (id >= n) {
+                set_err_at(d, ERR_INTERNAL, 7, g, id, d.n);
+                continue;
+            }
+            uint2 xp = make_uint2(0u, 0u);
+            bool bond = true;
+            if (ps != NO_SLOT) xp = *reinterpret_cast<const uint2 *>(&t.xv[ps]);
+            else bond = partner_global(d, g, id, xp);
+            if (COUNT && d.pcnt) d.pcnt[id] = t.cnt[s];
+            integrate_bead_at<B>(d, g, xv, id, bond, xp, fq_load_s(&t.f[s], t.fs), fq_load_s(&t.f[2 * t.fs + s], t.fs),
+                                 flags, th, later);
+        }
+        if (flags & (F_ADVANCE | F_FINAL)) {
+            __syncthreads();
+            thermo_flush_q(d, th, (int *)(smem + TP::queue_off(cap, NT, COUNT)));
+        }
+        later.store(d);
+    } else {
+        Thermo3 th{0.0, 0.0, 0.0};
+        force_tile_global<B, COUNT>(d, g0, n_own, s_lo, s_hi, flags, th);
+        if (flags & (F_ADVANCE | F_FINAL)) {
+            __syncthreads();
+            thermo_flush_tile(d, th, (double *)(smem + TP::bead_off(NT)));
+        }
+    }
+}
+
 // Fused force + integrate for one tile.  Pairs inside the tile are taken once
 // (Newton-3 through shared-memory atomics on the partner's slot), pairs with
 // halo beads are taken from the owned side only (the neighbouring tile takes
@@ -1157,6 +1731,10 @@ __device__ void force_tile_g(const Sys &d, int tile, int flags, unsigned char *s
 template <int B, bool COUNT, int VAR>
 __device__ void force_tile(const Sys &d, int tile, int flags, unsigned char *smem, Thermo3 &th)
 {
+    if constexpr (VAR == 2) {
+        force_tile_m<B, COUNT>(d, tile, flags, smem);
+        return;
+    }
     if constexpr (VAR == 3) {
         force_tile_g<B, COUNT>(d, tile, flags, smem, th);
         return;
@@ -1173,8 +1751,6 @@ __device__ void force_tile(const Sys &d, int tile, int flags, unsigned char *sme
     uint32_t *s_items = (uint32_t *)(s_nit + B * B);  // variant 4: the ranges
     const int cap = d.cap;
     const TileArrays t = tile_arrays<B, VAR>(smem, cap, NT, COUNT);
-    uint16_t *s_order = (uint16_t *)(smem + TP::order_off(cap, NT, COUNT));   // variant 2
-    uint32_t *s_desc = (uint32_t *)(smem + TP::desc_off(cap, NT, COUNT));     // variant 2
 
     const int ty = tile / d.ntx, tx = tile - ty * d.ntx;
     const int x0 = tx * B, y0 = ty * B;
@@ -1190,22 +1766,13 @@ __device__ void force_tile(const Sys &d, int tile, int flags, unsigned char *sme
     const uint32_t g1 = max(g0, min(d.cstart[base + tw * th_], n));
     const int n_own = (int)(g1 - g0);
 
-    // owned cell table (and, for variant 2, each owned cell's walk
-    // descriptor: local cell index, the neighbour cells the tile owns (the
-    // Newton-3 side) and the ones to visit (ahead always, behind only when
-    // halo))
+    // owned cell table
     for (int c = tid; c < tw * th_; c += NT) {
         const int ly = c / tw, lx = c - ly * tw;
         const uint32_t b = min(max(d.cstart[base + c], g0), g1), e = min(max(d.cstart[base + c + 1], b), g1);
         const int lc = (ly + 1) * (B + 2) + lx + 1;
         s_cbeg[lc] = (int)(b - g0);
         s_ccnt[lc] = (int)(e - b);
-        if constexpr (TP::DESC) {
-            const uint32_t px = lx < tw - 1, nx = lx > 0, py = ly < th_ - 1, ny = ly > 0;
-            const uint32_t own = 1u | (px << 1) | ((px & py) << 2) | (py << 3) | ((nx & py) << 4) | (nx << 5) |
-                                 ((nx & ny) << 6) | (ny << 7) | ((px & ny) << 8);
-            s_desc[ly * B + lx] = (uint32_t)lc | (own << 9) | ((0x1fu | (~own & 0x1e0u)) << 18);
-        }
     }
     // halo cell table
     for (int h = tid; h < nh; h += NT) {
@@ -1258,8 +1825,6 @@ __device__ void force_tile(const Sys &d, int tile, int flags, unsigned char *sme
             s_hbeg[nh] = n_own + incl;
             s_sc[0] = n_own + incl;
             s_sc[1] = 0;   // next owned bead for the pair queue
-            s_sc[2] = 0;   // variant 2 order: beads placed from the front
-            s_sc[3] = 0;   // and from the back
         }
     }
     __syncthreads();
@@ -1281,12 +1846,6 @@ __device__ void force_tile(const Sys &d, int tile, int flags, unsigned char *sme
             t.f[3 * t.fs + k] = 0;
             if (COUNT) t.cnt[k] = 0u;
             t.lc[k] = (unsigned char)(lx | (ly << 4));
-            if constexpr (TP::ORDER) {
-                // cells whose walk also visits halo cells behind them (left
-                // column, bottom row, right column) have the longest walks
-                if (lx == 0 || ly == 0 || lx == tw - 1) s_order[atomicAdd(&s_sc[2], 1)] = (uint16_t)k;
-                else s_order[n_own - 1 - atomicAdd(&s_sc[3], 1)] = (uint16_t)k;
-            }
         }
         for (int k = n_own + tid; k < total; k += NT) {
             int lo = 0, hi = nh - 1;   // last h with hbeg[h] <= k
@@ -1312,13 +1871,10 @@ __device__ void force_tile(const Sys &d, int tile, int flags, unsigned char *sme
             __syncthreads();
             pairs_flat<COUNT>(d, n_own, total, tw, t, s_nit, s_items, (uint4 *)wbuf, (uint32_t *)(wbuf + 16 * 32),
                               s_sc + 1, s_lo, s_hi);
-        } else if constexpr (VAR == 5) {
+        } else {
             flat_cell_items<B>(d, tw, th_, n_own, s_cbeg, s_ccnt, s_nit, s_items);
             __syncthreads();
             pairs_items<COUNT, 2>(d, n_own, total, tw, t, s_nit, s_items, (uint32_t *)wbuf, s_sc + 1, s_lo, s_hi);
-        } else {
-            pairs_queue<B, COUNT>(d, n_own, s_cbeg, s_ccnt, t, (uint32_t *)wbuf, s_sc + 1, s_lo, s_hi, s_desc,
-                                  s_order);
         }
         __syncthreads();
 
@@ -1340,31 +1896,9 @@ __device__ void force_tile(const Sys &d, int tile, int flags, unsigned char *sme
 template <int B, int VAR>
 __host__ __device__ inline size_t tile_flush_off()
 {
-    if constexpr (VAR == 3) return TilePlanG<B>::bead_off(TILE_THREADS);
+    if constexpr (VAR == 2) return TilePlanM<B>::bead_off(tile_threads<B, VAR>());
+    else if constexpr (VAR == 3) return TilePlanG<B>::bead_off(TILE_THREADS);
     else return TilePlan<B, VAR>::bead_off(TILE_THREADS);
-}
-
-// Block reduction of a tile's thermo partials into the FP64 ring slot of
-// `step` (FP64 throughout): every thread's partials to shared memory (buf,
-// 3 blockDim doubles), then warp q adds quantity q (blockDim / 32 values per
-// lane, then across its lanes) and adds it to the slot.  A third of the FP64
-// additions of a shuffle tree in every warp (the FP64 pipe is narrow on this
-// part).  buf is read by warps 0-2 after the call: the caller synchronises
-// before reusing it.
-__device__ __forceinline__ void thermo_flush_tile(const Sys &d, Thermo3 th, double *buf)
-{
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nt = blockDim.x;
-    buf[tid] = th.ke;
-    buf[nt + tid] = th.px;
-    buf[2 * nt + tid] = th.py;
-    __syncthreads();
-    if (wid < 3) {
-        double a = 0.0;
-        for (int i = lane; i < nt; i += 32) a += buf[wid * nt + i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) atomicAdd(&d.thermo[4 * (size_t)(*d.step % THERMO_CAP) + wid], a);
-    }
 }
 
 // Block reduction of the thermo partials into the FP64 ring slot of `step`
