@@ -21,6 +21,7 @@
 
 #include "dpd.h"
 #include "obs_common.cuh"
+#include "vcf.cuh"
 #include "sim_host.h"
 
 namespace dpd {
@@ -103,99 +104,6 @@ __global__ void k_shells(const double2 *Z, int M, double scale, double *E)
     }
 }
 
-__global__ void k_vmeans(const double2 *v, int na, double *acc)
-{
-    double sx = 0, sy = 0, s2 = 0;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < na; k += gridDim.x * blockDim.x) {
-        const double2 a = v[k];
-        sx += a.x;
-        sy += a.y;
-        s2 += a.x * a.x + a.y * a.y;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sy += __shfl_xor_sync(0xffffffffu, sy, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&acc[0], sx);
-        atomicAdd(&acc[1], sy);
-        atomicAdd(&acc[2], s2);
-    }
-}
-
-// All pairs a < b of agents: separation bin floor(r / dr) (IEEE double, as
-// written), accumulate v_a . v_b and the pair count per bin in shared memory.
-constexpr int VCF_TILE = 256;
-__global__ void __launch_bounds__(VCF_TILE) k_vcf(const double2 *c, const double2 *v, int na, double L, double dr,
-                                                  int nbins, double *gnum, unsigned long long *gcnt)
-{
-    extern __shared__ unsigned char smem[];
-    double *snum = (double *)smem;
-    unsigned long long *scnt = (unsigned long long *)(snum + nbins);
-    double2 *sc = (double2 *)(scnt + nbins);
-    double2 *sv = sc + VCF_TILE;
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x) { snum[b] = 0.0; scnt[b] = 0ull; }
-    const int ntile = (na + VCF_TILE - 1) / VCF_TILE;
-    // block -> (row tile ti, column tile tj >= ti) over the upper triangle
-    // row ti starts at S(ti) = ti*ntile - ti*(ti-1)/2; invert with a square
-    // root and correct by one step either way
-    const long long bid = blockIdx.x, nt = ntile;
-    const double disc = (2.0 * nt + 1.0) * (2.0 * nt + 1.0) - 8.0 * (double)bid;
-    long long ti = (long long)floor(((2.0 * nt + 1.0) - sqrt(fmax(disc, 0.0))) * 0.5);
-    ti = ti < 0 ? 0 : (ti > nt - 1 ? nt - 1 : ti);
-    while (ti > 0 && ti * nt - ti * (ti - 1) / 2 > bid) --ti;
-    while (ti < nt - 1 && (ti + 1) * nt - (ti + 1) * ti / 2 <= bid) ++ti;
-    const int tj = (int)(ti + (bid - (ti * nt - ti * (ti - 1) / 2)));
-    const int a = (int)ti * VCF_TILE + threadIdx.x;
-    const int jb = tj * VCF_TILE;
-    for (int q = threadIdx.x; q < VCF_TILE; q += blockDim.x) {
-        const int j = jb + q;
-        sc[q] = j < na ? c[j] : make_double2(0.0, 0.0);
-        sv[q] = j < na ? v[j] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    if (a < na) {
-        const double2 ca = c[a], va = v[a];
-        const int jn = min(VCF_TILE, na - jb);
-        const double hL = 0.5 * L;
-        const double rmax2 = (double)nbins * dr * (double)nbins * dr * (1.0 + 1e-9);
-        const float inv_drf = (float)(1.0 / dr), nbf = (float)nbins;
-        for (int q = 0; q < jn; ++q) {
-            const int j = jb + q;
-            if (j <= a) continue;
-            // minimum image: agent centres lie on the L / 2^33 grid, so d / L never
-            // rounds onto +-1/2 and the comparison equals d - L rint(d / L)
-            double dx = __dsub_rn(ca.x, sc[q].x), dy = __dsub_rn(ca.y, sc[q].y);
-            dx = dx > hL ? __dsub_rn(dx, L) : (dx < -hL ? __dadd_rn(dx, L) : dx);
-            dy = dy > hL ? __dsub_rn(dy, L) : (dy < -hL ? __dadd_rn(dy, L) : dy);
-            const double r2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
-            if (!(r2 < rmax2)) continue;   // beyond the last bin (a margin above it)
-            // bin floor(sqrt(r2) / dr): FP32 where the value is at least 1e-3 from
-            // a bin edge (its error here is ~1e-4), else the FP64 expression
-            const float tf = sqrtf((float)r2) * inv_drf;
-            const float fl = floorf(tf);
-            int b;
-            if (tf - fl > 1e-3f && fl + 1.0f - tf > 1e-3f && tf < nbf - 1e-3f) {
-                b = (int)fl;
-            } else {
-                const double bf = floor(__ddiv_rn(sqrt(r2), dr));
-                if (!(bf < (double)nbins)) continue;
-                b = (int)bf;
-            }
-            atomicAdd(&snum[b], __dadd_rn(__dmul_rn(va.x, sv[q].x), __dmul_rn(va.y, sv[q].y)));
-            atomicAdd(&scnt[b], 1ull);
-        }
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
-        if (scnt[b]) {
-            atomicAdd(&gnum[b], snum[b]);
-            atomicAdd(&gcnt[b], scnt[b]);
-        }
-    }
-}
-
 // Sum over agents of |v_COM| with v_COM = (v_head + v_tail) / 2, FP64.
 __global__ void k_agent_speed(const uint4 *__restrict__ xv, int na, double *acc)
 {
@@ -208,135 +116,6 @@ __global__ void k_agent_speed(const uint4 *__restrict__ xv, int na, double *acc)
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(acc, s);
-}
-
-// ---- velocity correlation limited to r < r_max = nbins dr ------------------
-// Agents are counting-sorted into a periodic grid of ncv x ncv cells of side
-// L / ncv >= r_max, so every pair inside r_max lies in the same or an
-// adjacent cell.  One block per cell takes its own agents against the agents
-// of the cell itself (b after a) and of its four forward neighbours (E, NE,
-// N, NW), each neighbour cell staged in shared memory in chunks.  Separations
-// are taken in FP32 from offsets to the block's cell corner (error below
-// 1e-5); a pair whose r / dr lies within 1e-3 of a shell edge or of r_max is
-// decided by the FP64 expressions of k_vcf instead, so the shell of every
-// pair, and hence the counts, equal the all-pairs kernel's; the products
-// v_a . v_b are FP64 as there.
-constexpr int VCFC_THREADS = 128, VCFC_CHUNK = 512, VCFC_WARPS = VCFC_THREADS / 32;
-
-__device__ __forceinline__ int vcf_cell_of(double x, double cw, int ncv)
-{
-    const int c = (int)floor(__ddiv_rn(x, cw));
-    return c < 0 ? 0 : (c >= ncv ? ncv - 1 : c);
-}
-
-__global__ void k_vcf_count(const double2 *c, int na, double cw, int ncv, unsigned *cnt, unsigned *rank)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= na) return;
-    const double2 p = c[k];
-    const int cell = vcf_cell_of(p.y, cw, ncv) * ncv + vcf_cell_of(p.x, cw, ncv);
-    rank[k] = atomicAdd(&cnt[cell], 1u);
-}
-
-__global__ void k_vcf_scatter(const double2 *c, const double2 *v, int na, double cw, int ncv, const unsigned *start,
-                              const unsigned *rank, double2 *sc, double2 *sv)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= na) return;
-    const double2 p = c[k];
-    const int cell = vcf_cell_of(p.y, cw, ncv) * ncv + vcf_cell_of(p.x, cw, ncv);
-    const unsigned dst = start[cell] + rank[k];
-    if (dst < (unsigned)na) {
-        sc[dst] = p;
-        sv[dst] = v[k];
-    }
-}
-
-__global__ void __launch_bounds__(VCFC_THREADS) k_vcf_cells(const double2 *sc, const double2 *sv,
-                                                            const unsigned *start, int ncv, double L, double cw,
-                                                            double dr, int nbins, double *gnum,
-                                                            unsigned long long *gcnt)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    double *snum = (double *)smem;                                          // [VCFC_WARPS][nbins]
-    unsigned long long *scnt = (unsigned long long *)(snum + VCFC_WARPS * nbins);
-    double2 *bc = (double2 *)(scnt + VCFC_WARPS * nbins);                   // [VCFC_CHUNK]
-    double2 *bv = bc + VCFC_CHUNK;
-    float2 *bo = (float2 *)(bv + VCFC_CHUNK);
-    const int warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < VCFC_WARPS * nbins; i += blockDim.x) { snum[i] = 0.0; scnt[i] = 0ull; }
-    const int cell = blockIdx.x, cy = cell / ncv, cx = cell - cy * ncv;
-    const unsigned a0 = start[cell], a1 = start[cell + 1];
-    const double ox = cx * cw, oy = cy * cw, hL = 0.5 * L;
-    const double rmax2 = (double)nbins * dr * (double)nbins * dr * (1.0 + 1e-9);
-    const float rscr = (float)(nbins * dr) * 1.0001f + 1e-4f * (float)cw, rscr2 = rscr * rscr;
-    const float inv_drf = (float)(1.0 / dr), nbf = (float)nbins;
-    double *wnum = snum + warp * nbins;
-    unsigned long long *wcnt = scnt + warp * nbins;
-    for (int nb = 0; nb < 5; ++nb) {
-        // own cell, then E, NE, N, NW; periodic images carry their shift
-        const int dxc = nb == 0 ? 0 : (nb <= 2 ? 1 : (nb == 3 ? 0 : -1));
-        const int dyc = nb <= 1 ? 0 : 1;
-        int nx = cx + dxc, ny = cy + dyc;
-        double sx = 0.0, sy = 0.0;
-        if (nx >= ncv) { nx -= ncv; sx = L; } else if (nx < 0) { nx += ncv; sx = -L; }
-        if (ny >= ncv) { ny -= ncv; sy = L; }
-        const int nc = ny * ncv + nx;
-        const unsigned b0 = start[nc], b1 = start[nc + 1];
-        for (unsigned c0 = b0; c0 < b1; c0 += VCFC_CHUNK) {
-            const int m = (int)min((unsigned)VCFC_CHUNK, b1 - c0);
-            __syncthreads();
-            for (int q = threadIdx.x; q < m; q += blockDim.x) {
-                const double2 p = sc[c0 + q];
-                bc[q] = p;
-                bv[q] = sv[c0 + q];
-                bo[q] = make_float2((float)(p.x + sx - ox), (float)(p.y + sy - oy));
-            }
-            __syncthreads();
-            for (unsigned a = a0 + threadIdx.x; a < a1; a += blockDim.x) {
-                const double2 ca = sc[a], va = sv[a];
-                const float ax = (float)(ca.x - ox), ay = (float)(ca.y - oy);
-                const int q0 = nb == 0 ? (int)max(0ll, (long long)a + 1 - (long long)c0) : 0;
-                for (int q = q0; q < m; ++q) {
-                    const float fx = ax - bo[q].x, fy = ay - bo[q].y;
-                    const float r2f = fx * fx + fy * fy;
-                    if (r2f >= rscr2) continue;
-                    // the shell from the FP32 separation (error below 1e-5)
-                    // wherever r / dr lies at least 1e-3 from a shell edge
-                    // and from r_max; otherwise the FP64 expressions of k_vcf
-                    const float tf = sqrtf(r2f) * inv_drf;
-                    const float fl = floorf(tf);
-                    int bin;
-                    if (tf - fl > 1e-3f && fl + 1.0f - tf > 1e-3f && tf < nbf - 1e-3f) {
-                        bin = (int)fl;
-                    } else {
-                        const double2 cb = bc[q];
-                        double dx = __dsub_rn(ca.x, cb.x), dy = __dsub_rn(ca.y, cb.y);
-                        dx = dx > hL ? __dsub_rn(dx, L) : (dx < -hL ? __dadd_rn(dx, L) : dx);
-                        dy = dy > hL ? __dsub_rn(dy, L) : (dy < -hL ? __dadd_rn(dy, L) : dy);
-                        const double r2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
-                        if (!(r2 < rmax2)) continue;
-                        const double bf = floor(__ddiv_rn(sqrt(r2), dr));
-                        if (!(bf < (double)nbins)) continue;
-                        bin = (int)bf;
-                    }
-                    const double2 vb = bv[q];
-                    atomicAdd(&wnum[bin], __dadd_rn(__dmul_rn(va.x, vb.x), __dmul_rn(va.y, vb.y)));
-                    atomicAdd(&wcnt[bin], 1ull);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
-        double sn = 0.0;
-        unsigned long long cn = 0ull;
-        for (int w = 0; w < VCFC_WARPS; ++w) { sn += snum[w * nbins + b]; cn += scnt[w * nbins + b]; }
-        if (cn) {
-            atomicAdd(&gnum[b], sn);
-            atomicAdd(&gcnt[b], cn);
-        }
-    }
 }
 
 }  // namespace dpd
@@ -498,76 +277,25 @@ int dpd_velocity_correlation(dpd_ctx *c, double dr, int nbins, double *g, double
     if (!c->have_state) return DPD_ERR_STATE;
     const int na = c->d.n / 2;
     const double L = c->p.L;
-    // pairs within r_max = nbins dr only: a cell grid of side >= r_max when at
-    // least three cells fit per side (and the grid stays below 4 M cells),
-    // else all pairs; both evaluate a pair with the same arithmetic
+    // pairs within r_max = nbins dr only: a cell grid when at least three cells
+    // of side r_max fit per side, else all pairs; both give a pair the same shell
     const double rmax = (double)nbins * dr * (1.0 + 1e-9);
     const double ncv_d = std::floor(L / rmax);
-    const bool cells = ncv_d >= 3.0 && ncv_d <= 2048.0;
-    const int ncv = cells ? (int)ncv_d : 0, ncell = ncv * ncv;
-    const size_t a256 = 256;
-    auto up = [&](size_t x) { return (x + a256 - 1) & ~(a256 - 1); };
-    const size_t o_cc = 0, o_vv = up(o_cc + 16 * (size_t)na), o_num = up(o_vv + 16 * (size_t)na),
-                 o_cnt = up(o_num + 8 * (size_t)nbins), o_acc = up(o_cnt + 8 * (size_t)nbins),
-                 o_ccnt = up(o_acc + 64), o_cst = up(o_ccnt + 4 * (size_t)ncell),
-                 o_rnk = up(o_cst + 4 * ((size_t)ncell + 1)), o_scs = up(o_rnk + (cells ? 4 * (size_t)na : 0)),
-                 o_svs = up(o_scs + (cells ? 16 * (size_t)na : 0)), bytes = up(o_svs + (cells ? 16 * (size_t)na : 0));
-    ObsScratch *s = scratch_of(c, bytes);
+    const bool few = ncv_d >= 3.0 && ncv_d <= 2048.0, cells = few || (ncv_d > 2048.0 && nbins <= 2560);
+    const long long tiles = (na + 255) / 256;   // limits of the call: shells, and agents where r_max is no cell's side
+    if (few ? 64 * (size_t)nbins + 20480 > 200 * 1024
+            : 16 * (size_t)nbins + 8192 > 200 * 1024 || tiles * (tiles + 1) / 2 > 2147483647ll)
+        return DPD_ERR_INVALID_ARG;
+    int m = 0, n = 0;
+    if (cells) vcf::cells_for<2>(L, rmax, na, 2048, &m, &n);
+    ObsScratch *s = scratch_of(c, vcf::Layout((size_t)na, (size_t)nbins, vcf::cells_of<2>(n)).bytes);
     if (!s) return DPD_ERR_OOM;
-    char *b = (char *)s->buf;
-    double2 *cc = (double2 *)(b + o_cc), *vv = (double2 *)(b + o_vv);
-    double *gnum = (double *)(b + o_num);
-    unsigned long long *gcnt = (unsigned long long *)(b + o_cnt);
-    double *acc = (double *)(b + o_acc);
-    CUO(cudaMemsetAsync(gnum, 0, 8 * (size_t)nbins, c->st));
-    CUO(cudaMemsetAsync(gcnt, 0, 8 * (size_t)nbins, c->st));
-    CUO(cudaMemsetAsync(acc, 0, 64, c->st));
-    k_agent_com<<<(na + 255) / 256, 256, 0, c->st>>>(c->d.C_xv, na, L, c->d.ulen_d, cc, vv);
-    k_vmeans<<<64, 256, 0, c->st>>>(vv, na, acc);
-    if (cells) {
-        const double cw = L / ncv;
-        unsigned *ccnt = (unsigned *)(b + o_ccnt), *cst = (unsigned *)(b + o_cst), *rnk = (unsigned *)(b + o_rnk);
-        double2 *scs = (double2 *)(b + o_scs), *svs = (double2 *)(b + o_svs);
-        CUO(cudaMemsetAsync(ccnt, 0, 4 * (size_t)ncell, c->st));
-        k_vcf_count<<<(na + 255) / 256, 256, 0, c->st>>>(cc, na, cw, ncv, ccnt, rnk);
-        k_vcf_scan<<<1, 1024, 0, c->st>>>(ccnt, ncell, cst);
-        k_vcf_scatter<<<(na + 255) / 256, 256, 0, c->st>>>(cc, vv, na, cw, ncv, cst, rnk, scs, svs);
-        const size_t sm = (size_t)VCFC_WARPS * nbins * 16 + (size_t)VCFC_CHUNK * 40;
-        if (sm > 200 * 1024) return DPD_ERR_INVALID_ARG;
-        CUO(cudaFuncSetAttribute(k_vcf_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k_vcf_cells<<<ncell, VCFC_THREADS, sm, c->st>>>(scs, svs, cst, ncv, L, cw, dr, nbins, gnum, gcnt);
-    } else {
-        const int ntile = (na + VCF_TILE - 1) / VCF_TILE;
-        const long long nblk = (long long)ntile * (ntile + 1) / 2;
-        const size_t sm = 16 * (size_t)nbins + 32 * VCF_TILE;
-        if (sm > 200 * 1024 || nblk > 2147483647ll) return DPD_ERR_INVALID_ARG;
-        CUO(cudaFuncSetAttribute(k_vcf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k_vcf<<<(unsigned)nblk, VCF_TILE, sm, c->st>>>(cc, vv, na, L, dr, nbins, gnum, gcnt);
-    }
-    CUO(cudaGetLastError());
-    std::vector<double> hn(nbins), ha(3);
-    std::vector<unsigned long long> hc(nbins);
-    CUO(cudaMemcpyAsync(hn.data(), gnum, 8 * (size_t)nbins, cudaMemcpyDeviceToHost, c->st));
-    CUO(cudaMemcpyAsync(hc.data(), gcnt, 8 * (size_t)nbins, cudaMemcpyDeviceToHost, c->st));
-    CUO(cudaMemcpyAsync(ha.data(), acc, 24, cudaMemcpyDeviceToHost, c->st));
-    const int rc = dpd_internal_latched(c);
-    const double mx = ha[0] / na, my = ha[1] / na, v2 = ha[2] / na, m2 = mx * mx + my * my;
-    const double den = v2 - m2;
-    double li = 0.0, rprev = 0.0, gprev = 1.0;
-    for (int k = 0; k < nbins; ++k) {
-        if (hc[k] > 0 && den > 0) {
-            g[k] = (hn[k] / (double)hc[k] - m2) / den;
-            const double r = (k + 0.5) * dr;
-            li += 0.5 * (g[k] + gprev) * (r - rprev);
-            rprev = r;
-            gprev = g[k];
-        } else {
-            g[k] = NAN;
-        }
-        if (num) num[k] = hn[k];
-        if (cnt) cnt[k] = (int64_t)hc[k];
-    }
-    if (L_int) *L_int = den > 0 ? li : NAN;
+    const vcf::State state{c->d.C_xv, nullptr, na, L, c->d.ulen_d};
+    std::vector<long long> host;
+    int rc = vcf::vcf_run<2>(state, dr, nbins, m, n, (char *)s->buf, c->st, host);
+    if (rc) return rc;
+    rc = dpd_internal_latched(c);
+    vcf::vcf_outputs(vcf::vcf_finish<2>(host, na, nbins), dr, nbins, g, L_int, num, cnt);
     return rc;
 }
 

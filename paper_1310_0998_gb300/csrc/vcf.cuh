@@ -1,0 +1,678 @@
+// Velocity correlation of agents (Sec. 5.3, Eqs. VCF, spatial01) in two and
+// three dimensions: sums of v_a . v_b and pair counts over the agent pairs
+// a < b by shell floor(r / dr) of their separation, and the means of v and |v|^2.
+//
+// The FP64 pipe of this part is one lane wide (32 cycles per warp instruction)
+// and its shared-memory FP64 add is a compare-and-swap loop, so the pass does
+// its arithmetic in FP32 and whole numbers:
+//   separation  from FP32 offsets inside the cells (or from the 32-bit centres
+//               of mass where no cells are used).  A pair whose r / dr lies
+//               within `mg` of a shell edge or of r_max, `mg` being above the
+//               FP32 error, is queued, and full warps of queued pairs take the
+//               FP64 expressions of the definition: every pair's shell, and
+//               hence every count, is that of the FP64 evaluation.
+//   products    v = (V + r) / k with k a power of two by the fastest agent
+//               (|V| < 2^28, |r| <= 1/2): V_a . V_b is exact in 64 bits, the
+//               cross terms V_a . r_b + r_a . V_b are FP32, rounded to whole
+//               numbers (2^-53 of the largest product at most).
+//   sums        three 19-bit limbs of a product and the count go to the warp's
+//               own histogram in shared memory by native 32-bit integer adds;
+//               it is emptied into 64-bit global sums before a word can
+//               overflow.  Whole-number sums do not depend on the order.
+// A warp takes 32 agents of a cell at a time, one per lane, against the agents of
+// a neighbour cell, whose data every lane reads at the same address.
+// Bound by instruction issue (54 warp instructions per 32 candidates, half of
+// them inside r_max).  1,572,864 agents, r < 16, 64 shells (9.5e8 pairs): 4.0 ms
+// against 27.7 with FP64 products and shared FP64 adds; a cube of 393,216, r < 4:
+// 1.4 against 6.0; all pairs of 1,382 agents (96 shells): 22 us against 410.
+#pragma once
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <vector>
+
+#include <cuda_runtime.h>
+
+#include "dpd.h"
+#include "obs_common.cuh"
+
+namespace dpd {
+namespace vcf {
+
+// Canonical state in id order; beads 2k and 2k + 1 are agent k.  In two
+// dimensions the velocity is in p.z, p.w and v is unused.
+struct State {
+    const uint4 *p;
+    const float4 *v;
+    int na;
+    double L, ulen;
+};
+
+template <int D>
+struct Agent {
+    unsigned long long c[D];   // centre of mass in units L 2^-33
+    float sh[D], sl[D];        // v_head + v_tail = sh + sl exactly
+};
+
+template <int D>
+__device__ __forceinline__ Agent<D> load_agent(const State &s, int k)
+{
+    const uint4 h = s.p[2 * (size_t)k], t = s.p[2 * (size_t)k + 1];
+    const uint32_t hx[3] = {h.x, h.y, h.z}, tx[3] = {t.x, t.y, t.z};
+    float hv[3], tv[3];
+    if constexpr (D == 2) {
+        hv[0] = __uint_as_float(h.z); hv[1] = __uint_as_float(h.w);
+        tv[0] = __uint_as_float(t.z); tv[1] = __uint_as_float(t.w);
+    } else {
+        const float4 a = s.v[2 * (size_t)k], b = s.v[2 * (size_t)k + 1];
+        hv[0] = a.x; hv[1] = a.y; hv[2] = a.z;
+        tv[0] = b.x; tv[1] = b.y; tv[2] = b.z;
+    }
+    Agent<D> g;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        g.c[i] = (2ull * tx[i] + (unsigned long long)(long long)(int)(hx[i] - tx[i])) & 0x1ffffffffull;
+        const float x = __fadd_rn(hv[i], tv[i]), bb = __fsub_rn(x, hv[i]);
+        g.sh[i] = x;
+        g.sl[i] = __fadd_rn(__fsub_rn(hv[i], __fsub_rn(x, bb)), __fsub_rn(tv[i], bb));
+    }
+    return g;
+}
+
+// log2 of the velocity scale k: |v| k < 2^28 for |v|^2 <= the value whose bits
+// are v2 (one bit spare for its rounding).
+__device__ __host__ __forceinline__ int scale_log2(uint32_t v2)
+{
+    const int e = (int)(v2 >> 23) - 127;            // |v|^2 < 2^(e + 1)
+    const int h = e >= 0 ? e / 2 + 1 : -((-e) / 2) + 1;   // |v| < 2^h
+    const int x = 27 - h;
+    return v2 == 0u ? 0 : (x < -100 ? -100 : (x > 100 ? 100 : x));
+}
+
+// V and r of one component from half the head and tail sum.
+__device__ __forceinline__ void split_v(float sh, float sl, float half_k, int &V, float &r)
+{
+    const float x = __fmul_rn(sh, half_k);
+    const int i = __float2int_rn(x);
+    const float y = __fadd_rn(__fsub_rn(x, (float)i), __fmul_rn(sl, half_k));
+    const float f = rintf(y);
+    V = i + (int)f;
+    r = __fsub_rn(y, f);
+}
+
+template <int D>
+__global__ void __launch_bounds__(256) k_vcf_max(State s, unsigned *vmax)
+{
+    unsigned m = 0u;
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < s.na; k += gridDim.x * 256) {
+        const Agent<D> g = load_agent<D>(s, k);
+        float v2 = 0.f;
+#pragma unroll
+        for (int i = 0; i < D; ++i) v2 = fmaf(0.5f * g.sh[i], 0.5f * g.sh[i], v2);
+        m = max(m, __float_as_uint(v2));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(vmax, m);
+}
+
+template <int D>
+__device__ __forceinline__ int cell_of(const Agent<D> &g, int n)
+{
+    int f = 0;
+#pragma unroll
+    for (int i = D - 1; i >= 0; --i) f = f * n + (int)((g.c[i] * (unsigned long long)n) >> 33);
+    return f;
+}
+
+// Sums over the agents (sum V, sum 2^20 r per component; V^2 in two 32-bit
+// halves and r (2 V + r)) and, with cells (n > 0), each agent's rank in its cell.
+template <int D>
+__global__ void __launch_bounds__(256) k_vcf_count(State s, int n, const unsigned *vmax, unsigned *cnt, unsigned *rank,
+                                                   long long *sums)
+{
+    constexpr int NS = 2 * D + 3;
+    const float half_k = __int_as_float((127 + scale_log2(*vmax) - 1) << 23);
+    long long a[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) a[i] = 0;
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < s.na; k += gridDim.x * 256) {
+        const Agent<D> g = load_agent<D>(s, k);
+        if (n > 0) rank[k] = atomicAdd(&cnt[cell_of<D>(g, n)], 1u);
+        unsigned long long q = 0;
+        float er = 0.f;
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            int V;
+            float r;
+            split_v(g.sh[i], g.sl[i], half_k, V, r);
+            a[2 * i] += V;
+            a[2 * i + 1] += __float2int_rn(r * 1048576.0f);
+            q += (unsigned long long)((long long)V * V);
+            er = fmaf(r, fmaf(2.0f, (float)V, r), er);
+        }
+        a[2 * D] += (long long)(q & 0xffffffffull);
+        a[2 * D + 1] += (long long)(q >> 32);
+        a[2 * D + 2] += __float2int_rn(er);
+    }
+    __shared__ long long red[8][NS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        long long x = a[i];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) red[warp][i] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x < NS) {
+        long long x = 0;
+        for (int w = 0; w < 8; ++w) x += red[w][threadIdx.x];
+        atomicAdd((unsigned long long *)&sums[threadIdx.x], (unsigned long long)x);
+    }
+}
+
+// Agents in cell order (n > 0: offset from the cell's corner in units of dr) or
+// as they come (n = 0: 32-bit centre of mass): P, Q = (Vx, Vy, rx, ry) or
+// (Vx, Vy, Vz, rz) with R = (rx, ry), and the agent's id.
+template <int D>
+__global__ void __launch_bounds__(256) k_vcf_place(State s, int n, float cell_dr, const unsigned *vmax,
+                                                   const unsigned *start, const unsigned *rank, float4 *P, int4 *Q,
+                                                   float2 *R, int *id)
+{
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    if (k >= s.na) return;
+    const float half_k = __int_as_float((127 + scale_log2(*vmax) - 1) << 23);
+    const Agent<D> g = load_agent<D>(s, k);
+    unsigned dst = (unsigned)k;
+    if (n > 0) dst = start[cell_of<D>(g, n)] + rank[k];
+    if (dst >= (unsigned)s.na) return;
+    float p[3] = {0.f, 0.f, 0.f}, r[3] = {0.f, 0.f, 0.f};
+    int v[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        if (n > 0) {
+            const unsigned long long f = (g.c[i] * (unsigned long long)n) & 0x1ffffffffull;   // offset in the cell, 2^-33
+            p[i] = (float)(uint32_t)(f >> 1) * 2.3283064365386963e-10f * cell_dr;
+        } else {
+            p[i] = __uint_as_float((uint32_t)(g.c[i] >> 1));
+        }
+        split_v(g.sh[i], g.sl[i], half_k, v[i], r[i]);
+    }
+    P[dst] = make_float4(p[0], p[1], p[2], 0.f);
+    if constexpr (D == 2) {
+        Q[dst] = make_int4(v[0], v[1], __float_as_int(r[0]), __float_as_int(r[1]));
+    } else {
+        Q[dst] = make_int4(v[0], v[1], v[2], __float_as_int(r[2]));
+        R[dst] = make_float2(r[0], r[1]);
+    }
+    id[dst] = k;
+}
+
+// Exclusive scan of n counts in one block, 4096 coalesced counts a turn.
+static __global__ void __launch_bounds__(1024) k_vcf_scan(const unsigned *cnt, int n, unsigned *start)
+{
+    __shared__ unsigned s_w[32];
+    __shared__ unsigned s_carry;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t == 0) s_carry = 0u;
+    for (int b = 0; b < n; b += 4096) {
+        unsigned c[4], sum = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = b + 4 * t + i;
+            c[i] = k < n ? cnt[k] : 0u;
+            sum += c[i];
+        }
+        unsigned incl = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) s_w[warp] = incl;
+        __syncthreads();
+        if (warp == 0) {
+            const unsigned w = s_w[lane];
+            unsigned wi = w;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(0xffffffffu, wi, o);
+                if (lane >= o) wi += v;
+            }
+            s_w[lane] = wi - w + s_carry;
+            __syncwarp();
+            if (lane == 31) s_carry += wi;
+        }
+        __syncthreads();
+        unsigned run = s_w[warp] + incl - sum;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = b + 4 * t + i;
+            if (k < n) start[k] = run;
+            run += c[i];
+        }
+        __syncthreads();
+    }
+    if (t == 0) start[n] = s_carry;
+}
+
+// What the pair passes share.
+struct Pass {
+    State s;
+    const float4 *P;
+    const int4 *Q;
+    const float2 *R;
+    const int *id;
+    double dr;
+    int nbins;
+    float lim2, mg;            // (nbins + mg)^2, and the distance from a shell edge that FP32 decides
+    long long *gsum;           // [3][nbins] limb sums
+    unsigned long long *gcnt;  // [nbins]
+};
+
+constexpr int LIMB = 19;
+constexpr int FULL_AT = 4000;   // adds to a histogram word after which it is emptied (it holds 2^13)
+constexpr int QUEUE = 160;
+constexpr int RUN = 128;        // candidates between two looks at the counts: 32 x 128 adds at most
+
+template <int D>
+struct Warp {
+    const Pass &p;
+    int *h;            // [4][nbins]: low, middle, high limb, count (this warp's)
+    uint2 *q;          // queued pairs near a shell edge (QUEUE: 31 and four candidates of 32 lanes)
+    int qn, lane;
+    int a;             // the lane's agent, -1 for none
+    float x[D];
+    struct Vel { int V[D]; float r[D]; } va;
+    float Fa[D];
+
+    __device__ Warp(const Pass &pass, int *hist, uint2 *queue)
+        : p(pass), h(hist), q(queue), qn(0), lane(threadIdx.x & 31), a(-1)
+    {
+        for (int i = lane; i < 4 * p.nbins; i += 32) h[i] = 0;
+        __syncwarp();
+    }
+    __device__ __forceinline__ Vel vel(int b) const
+    {
+        const int4 q = p.Q[b];
+        Vel v;
+        v.V[0] = q.x;
+        v.V[1] = q.y;
+        if constexpr (D == 2) {
+            v.r[0] = __int_as_float(q.z);
+            v.r[1] = __int_as_float(q.w);
+        } else {
+            const float2 r = p.R[b];
+            v.V[2] = q.z;
+            v.r[0] = r.x;
+            v.r[1] = r.y;
+            v.r[2] = __int_as_float(q.w);
+        }
+        return v;
+    }
+    __device__ __forceinline__ void load(int k, int end)
+    {
+        a = k < end ? k : -1;
+        const float4 P = p.P[max(a, 0)];
+        const float px[3] = {P.x, P.y, P.z};
+        va = vel(max(a, 0));
+#pragma unroll
+        for (int i = 0; i < D; ++i) { x[i] = px[i]; Fa[i] = (float)va.V[i]; }
+    }
+    __device__ __forceinline__ void add(int bin, long long d)
+    {
+        int *w = h + bin;
+        atomicAdd(w, (int)(d & ((1 << LIMB) - 1)));
+        atomicAdd(w + p.nbins, (int)((d >> LIMB) & ((1 << LIMB) - 1)));
+        atomicAdd(w + 2 * p.nbins, (int)(d >> (2 * LIMB)));
+        atomicAdd(w + 3 * p.nbins, 1);
+    }
+    // v . w in units k^-2 (the product of the rests, below one unit, is left out).
+    static __device__ __forceinline__ long long dot(const Vel &v, const float *F, const Vel &w)
+    {
+        long long d = 0;
+        float c = 0.f;
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            d += (long long)v.V[i] * w.V[i];
+            c = fmaf(F[i], w.r[i], c);
+            c = fmaf(v.r[i], (float)w.V[i], c);
+        }
+        return d + __float2int_rn(c);
+    }
+    // FP64 centre of mass, the operations of k_agent_com.
+    __device__ __forceinline__ void com(int id, double *c) const
+    {
+        const uint4 hd = p.s.p[2 * (size_t)id], tl = p.s.p[2 * (size_t)id + 1];
+        const uint32_t hx[3] = {hd.x, hd.y, hd.z}, tx[3] = {tl.x, tl.y, tl.z};
+        for (int i = 0; i < D; ++i) {
+            const double t = __dmul_rn((double)tx[i], p.s.ulen);
+            const double y = __dadd_rn(t, __dmul_rn(0.5, minimg_d(__dsub_rn(__dmul_rn((double)hx[i], p.s.ulen), t), p.s.L)));
+            c[i] = __dsub_rn(y, __dmul_rn(p.s.L, floor(__ddiv_rn(y, p.s.L))));
+        }
+    }
+    // The last queued pairs (up to 32 of them) by the FP64 definition of their shell.
+    __device__ __forceinline__ void drain()
+    {
+        __syncwarp();
+        const int first = max(qn - 32, 0);
+        if (first + lane < qn) {
+            const uint2 e = q[first + lane];
+            double ca[3], cb[3], d[3];
+            com(p.id[e.x], ca);
+            com(p.id[e.y], cb);
+            const double hL = 0.5 * p.s.L;
+            for (int i = 0; i < D; ++i) {
+                d[i] = __dsub_rn(ca[i], cb[i]);
+                d[i] = d[i] > hL ? __dsub_rn(d[i], p.s.L) : (d[i] < -hL ? __dadd_rn(d[i], p.s.L) : d[i]);
+            }
+            double r2 = __dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1]));
+            if constexpr (D == 3) r2 = __dadd_rn(r2, __dmul_rn(d[2], d[2]));
+            const double rmax2 = (double)p.nbins * p.dr * (double)p.nbins * p.dr * (1.0 + 1e-9);
+            const double bf = floor(__ddiv_rn(sqrt(r2), p.dr));
+            if (r2 < rmax2 && bf < (double)p.nbins) {
+                const Vel v = vel((int)e.x);
+                float F[D];
+                for (int i = 0; i < D; ++i) F[i] = (float)v.V[i];
+                add((int)bf, dot(v, F, vel((int)e.y)));
+            }
+        }
+        qn = first;
+        __syncwarp();
+    }
+    __device__ __forceinline__ void flush()
+    {
+        __syncwarp();
+        const int nb = p.nbins;
+        for (int b = lane; b < nb; b += 32) {
+            const int c = h[3 * nb + b];
+            if (c == 0) continue;
+            for (int w = 0; w < 3; ++w) {
+                atomicAdd((unsigned long long *)&p.gsum[w * nb + b], (unsigned long long)(long long)h[w * nb + b]);
+                h[w * nb + b] = 0;
+            }
+            atomicAdd(&p.gcnt[b], (unsigned long long)c);
+            h[3 * nb + b] = 0;
+        }
+        __syncwarp();
+    }
+    // The lane's agent, seen from `sh` (cells: the neighbour cell's corner; none:
+    // ALL), against the agents [s, e) after `after`.
+    template <bool ALL>
+    __device__ __forceinline__ void run(int s, int e, const float *sh, int after, float unit)
+    {
+        constexpr float M = 12582912.0f;   // 1.5 2^23: adding it rounds to a whole number in the low bits
+        float y[D];
+        uint32_t X[D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            y[i] = ALL ? 0.f : x[i] - sh[i];
+            X[i] = __float_as_uint(x[i]);
+        }
+        const float lim2 = a >= 0 ? p.lim2 : -1.0f, inside = 0.5f - p.mg, last = (float)p.nbins - p.mg;
+        while (s < e) {
+            const int stop = min(e, s + RUN);
+            for (; s < stop; s += 4) {
+                unsigned near = 0u;   // candidates whose shell FP32 does not decide
+                float t2[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float4 P = p.P[min(s + u, stop - 1)];
+                    const float px[3] = {P.x, P.y, P.z};
+                    t2[u] = 0.f;
+#pragma unroll
+                    for (int i = 0; i < D; ++i) {
+                        // whole-number difference: the periodic image nearest by wrapping
+                        const float dd = ALL ? (float)(int)(X[i] - __float_as_uint(px[i])) * unit : y[i] - px[i];
+                        t2[u] = fmaf(dd, dd, t2[u]);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int b = s + u;
+                    if ((b < stop) & (t2[u] < lim2) & (b > after)) {
+                        float t;
+                        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(t2[u]));
+                        // the shell's middle nearest to t
+                        const float w = t - 0.5f, z = w + M;
+                        if ((fabsf(w - (z - M)) < inside) & (t < last)) add(__float_as_int(z) - 0x4B400000, dot(va, Fa, vel(b)));
+                        else near |= 1u << u;
+                    }
+                }
+                if (__any_sync(0xffffffffu, near != 0u)) {
+#pragma unroll 1
+                    for (int u = 0; u < 4; ++u) {
+                        const bool on = (near >> u) & 1u;
+                        const unsigned m = __ballot_sync(0xffffffffu, on);
+                        if (on) q[qn + __popc(m & ((1u << lane) - 1u))] = make_uint2((unsigned)a, (unsigned)(s + u));
+                        qn += __popc(m);
+                    }
+                    while (qn >= 32) drain();
+                }
+            }
+            __syncwarp();
+            int most = 0;
+            for (int b = lane; b < p.nbins; b += 32) most = max(most, h[3 * p.nbins + b]);
+            if (__any_sync(0xffffffffu, most >= FULL_AT)) flush();
+        }
+    }
+    __device__ __forceinline__ void finish()
+    {
+        while (qn > 0) drain();
+        flush();
+    }
+};
+
+__host__ __device__ inline size_t warp_smem(int nbins) { return (size_t)nbins * 16 + QUEUE * sizeof(uint2); }
+
+// Cells: task (cell, row of neighbour cells), rows 0 .. of the forward half
+// stencil of m cells each way (row 0: the own cell and those east of it), taken
+// from a counter.
+template <int D>
+__global__ void __launch_bounds__(128) k_vcf_cells(Pass p, const unsigned *start, int n, int m, int rows, int tasks,
+                                                   float cell_dr, unsigned *next)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned char *mine = smem + warp_smem(p.nbins) * (threadIdx.x >> 5);
+    Warp<D> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
+    while (true) {
+        unsigned t = 0;
+        if (w.lane == 0) t = atomicAdd(next, 1u);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= (unsigned)tasks) break;
+        const int cell = (int)t / rows, row = (int)t - cell * rows;
+        int c[3] = {cell % n, (cell / n) % n, D == 3 ? cell / (n * n) : 0};
+        // row r > 0: forward rows in (dz, dy) order after (0, 0)
+        int dy = row, dz = 0;
+        if (D == 3 && row > m) {
+            dz = 1 + (row - m - 1) / (2 * m + 1);
+            dy = (row - m - 1) % (2 * m + 1) - m;
+        }
+        const int yy = c[1] + dy, zz = c[2] + dz;
+        const int ny = yy < 0 ? yy + n : (yy >= n ? yy - n : yy), nz = zz >= n ? zz - n : zz;
+        const int a0 = (int)start[cell], a1 = (int)start[cell + 1];
+        for (int g = a0; g < a1; g += 32) {
+            w.load(g + w.lane, a1);
+            for (int dx = row == 0 ? 0 : -m; dx <= m; ++dx) {
+                const int xx = c[0] + dx, nx = xx < 0 ? xx + n : (xx >= n ? xx - n : xx);
+                const int nb = (nz * n + ny) * n + nx;
+                const float sh[3] = {dx * cell_dr, dy * cell_dr, dz * cell_dr};
+                w.template run<false>((int)start[nb], (int)start[nb + 1], sh, row == 0 && dx == 0 ? w.a : -1, 0.f);
+            }
+        }
+    }
+    w.finish();
+}
+
+// All pairs: a warp's 32 agents against a stretch of `cols` agents after them.
+template <int D>
+__global__ void __launch_bounds__(128) k_vcf_all(Pass p, int cols, float unit)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int a0 = ((int)blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5)) * 32;
+    const int s = max(a0, (int)blockIdx.y * cols), e = min(p.s.na, ((int)blockIdx.y + 1) * cols);
+    if (a0 >= p.s.na || s >= e) return;   // a whole warp at a time; no block barrier below
+    unsigned char *mine = smem + warp_smem(p.nbins) * (threadIdx.x >> 5);
+    Warp<D> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
+    w.load(a0 + w.lane, p.s.na);
+    w.template run<true>(s, e, nullptr, w.a, unit);
+    w.finish();
+}
+
+// Host results of a pass.
+struct Out {
+    std::vector<double> num;
+    std::vector<unsigned long long> cnt;
+    double mean[3], v2;
+};
+
+// Scratch of a pass: fixed offsets for na agents, nbins shells, ncell cells.
+struct Layout {
+    size_t P, Q, R, id, rank, cnt, start, zero, words, bytes;   // [zero, bytes): cleared words
+    Layout(size_t na, size_t nbins, size_t ncell)
+    {
+        auto up = [](size_t o) { return (o + 255) & ~size_t(255); };
+        P = 0;
+        Q = up(P + 16 * na);
+        R = up(Q + 16 * na);
+        id = up(R + 8 * na);
+        rank = up(id + 4 * na);
+        start = up(rank + (ncell ? 4 * na : 0));
+        zero = up(start + 4 * (ncell + 1));
+        words = zero;                    // [0] vmax, [1] task counter, then 16 sums
+        cnt = up(words + 256);           // cell counts
+        bytes = up(cnt + 4 * ncell) + 8 * 4 * nbins;
+    }
+    size_t sums() const { return words + 64; }
+    size_t gsum(size_t nbins) const { return bytes - 8 * 4 * nbins; }
+};
+
+#define VCF_CU(x)                                                                   \
+    do {                                                                            \
+        const cudaError_t e_ = (x);                                                 \
+        if (e_ != cudaSuccess) return e_ == cudaErrorMemoryAllocation ? DPD_ERR_OOM : DPD_ERR_CUDA; \
+    } while (0)
+
+// Cells per r_max (m) and per side (n) for a box with room for n1 >= 3 cells of
+// side r_max: half cells where they still hold warps of agents (candidates
+// inside r_max: half instead of a third of them in two dimensions).
+template <int D>
+static void cells_for(double L, double rmax, int na, int limit, int *m, int *n)
+{
+    const int n1 = (int)std::min<double>(std::floor(L / rmax), limit);
+    const int n2 = (int)std::floor(2.0 * L / rmax);
+    const bool half = n2 <= limit && na / std::pow((double)n2, D) >= 48.0;
+    *m = half ? 2 : 1;
+    *n = half ? n2 : n1;
+}
+
+template <int D>
+static size_t cells_of(int n) { return D == 2 ? (size_t)n * n : (size_t)n * n * n; }
+
+// One pass on `st`; buf holds Layout(na, nbins, n^D).bytes.  n = 0: all pairs.
+// Asynchronous up to the copies into the caller's host buffers, which are
+// complete after the caller's synchronisation; vcf_finish then makes Out.
+template <int D>
+static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf, cudaStream_t st, std::vector<long long> &host)
+{
+    const size_t ncell = cells_of<D>(n);
+    const Layout l((size_t)s.na, (size_t)nbins, ncell);
+    unsigned *vmax = (unsigned *)(buf + l.words), *next = vmax + 1;
+    long long *sums = (long long *)(buf + l.sums());
+    Pass p;
+    p.s = s;
+    p.P = (const float4 *)(buf + l.P);
+    p.Q = (const int4 *)(buf + l.Q);
+    p.R = (const float2 *)(buf + l.R);
+    p.id = (const int *)(buf + l.id);
+    p.dr = dr;
+    p.nbins = nbins;
+    // FP32 error of r / dr.  Cells: offsets up to 2.7 nbins from a corner, ten
+    // half-ulps of nbins a component, the square and its root: below 24 nbins
+    // 2^-24.  All pairs: the centres' 32 bits on top of three half-ulps.
+    p.mg = (float)(nbins * 2e-6 + 2e-6 + (n > 0 ? 0.0 : s.L / dr * std::ldexp(1.0, -31)));
+    p.lim2 = ((float)nbins + p.mg) * ((float)nbins + p.mg) * 1.000001f;
+    p.gsum = (long long *)(buf + l.gsum((size_t)nbins));
+    p.gcnt = (unsigned long long *)(p.gsum + 3 * (size_t)nbins);
+    VCF_CU(cudaMemsetAsync(buf + l.zero, 0, l.bytes - l.zero, st));
+    int dev = 0, nsm = 0;
+    VCF_CU(cudaGetDevice(&dev));
+    VCF_CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int g = std::min((s.na + 255) / 256, 8 * nsm), gp = (s.na + 255) / 256;
+    const float cell_dr = n > 0 ? (float)(s.L / n / dr) : 0.f;
+    unsigned *cnt = (unsigned *)(buf + l.cnt), *rank = (unsigned *)(buf + l.rank), *start = (unsigned *)(buf + l.start);
+    k_vcf_max<D><<<g, 256, 0, st>>>(s, vmax);
+    k_vcf_count<D><<<g, 256, 0, st>>>(s, n, vmax, cnt, rank, sums);
+    if (n > 0) k_vcf_scan<<<1, 1024, 0, st>>>(cnt, (int)ncell, start);
+    k_vcf_place<D><<<gp, 256, 0, st>>>(s, n, cell_dr, vmax, start, rank, (float4 *)p.P, (int4 *)p.Q, (float2 *)p.R, (int *)p.id);
+    // warps per block: four, or one where the histograms are large
+    const int wpb = warp_smem(nbins) * 4 <= 96 * 1024 ? 4 : 1;
+    const size_t sm = warp_smem(nbins) * wpb;
+    if (n > 0) {
+        VCF_CU(cudaFuncSetAttribute(k_vcf_cells<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        const int rows = D == 2 ? m + 1 : m + 1 + m * (2 * m + 1);
+        int occ = 0;
+        VCF_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_vcf_cells<D>, 32 * wpb, sm));
+        const long long tasks = (long long)ncell * rows;
+        const long long blocks = std::min<long long>((tasks + wpb - 1) / wpb, (long long)nsm * std::max(occ, 1));
+        if (tasks > 2000000000ll) return DPD_ERR_INVALID_ARG;
+        k_vcf_cells<D><<<(unsigned)blocks, 32 * wpb, sm, st>>>(p, start, n, m, rows, (int)tasks, cell_dr, next);
+    } else {
+        VCF_CU(cudaFuncSetAttribute(k_vcf_all<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        // stretches long enough that emptying the histograms does not matter,
+        // short enough for a few thousand warps
+        const long long tiles = (s.na + 31) / 32;
+        long long cols = tiles * s.na / 2 / (32ll * nsm) / 32 * 32;
+        cols = std::min<long long>(std::max<long long>(cols, 32), 1 << 20);
+        while ((s.na + cols - 1) / cols > 65535) cols *= 2;
+        const dim3 grid((unsigned)((tiles + wpb - 1) / wpb), (unsigned)((s.na + cols - 1) / cols));
+        k_vcf_all<D><<<grid, 32 * wpb, sm, st>>>(p, (int)cols, (float)(std::ldexp(s.L, -32) / dr));
+    }
+    VCF_CU(cudaGetLastError());
+    host.resize(32 + 4 * (size_t)nbins);
+    VCF_CU(cudaMemcpyAsync(host.data(), buf + l.words, 256, cudaMemcpyDeviceToHost, st));
+    VCF_CU(cudaMemcpyAsync(host.data() + 32, p.gsum, 8 * 4 * (size_t)nbins, cudaMemcpyDeviceToHost, st));
+    return DPD_OK;
+}
+
+template <int D>
+static Out vcf_finish(const std::vector<long long> &host, int na, int nbins)
+{
+    Out o;
+    const uint32_t vmax = (uint32_t)((unsigned long long)host[0] & 0xffffffffull);
+    const int k = scale_log2(vmax);
+    const long long *s = host.data() + 8, *g = host.data() + 32;
+    for (int i = 0; i < 3; ++i)
+        o.mean[i] = i < D ? std::ldexp((double)s[2 * i] + std::ldexp((double)s[2 * i + 1], -20), -k) / na : 0.0;
+    const __int128 q = ((__int128)s[2 * D + 1] << 32) + s[2 * D] + s[2 * D + 2];
+    o.v2 = std::ldexp((double)q, -2 * k) / na;
+    o.num.resize(nbins);
+    o.cnt.resize(nbins);
+    for (int b = 0; b < nbins; ++b) {
+        const __int128 t = ((__int128)g[2 * nbins + b] << (2 * LIMB)) + ((__int128)g[nbins + b] << LIMB) + g[b];
+        o.num[b] = std::ldexp((double)t, -2 * k);
+        o.cnt[b] = (unsigned long long)g[3 * nbins + b];
+    }
+    return o;
+}
+
+// g, L_int, num, cnt of Eqs. (VCF), (spatial01) from the sums.
+static inline void vcf_outputs(const Out &o, double dr, int nbins, double *g, double *L_int, double *num, int64_t *cnt)
+{
+    const double m2 = o.mean[0] * o.mean[0] + o.mean[1] * o.mean[1] + o.mean[2] * o.mean[2], den = o.v2 - m2;
+    double li = 0.0, rprev = 0.0, gprev = 1.0;
+    for (int k = 0; k < nbins; ++k) {
+        if (o.cnt[k] > 0 && den > 0) {
+            g[k] = (o.num[k] / (double)o.cnt[k] - m2) / den;
+            const double r = (k + 0.5) * dr;
+            li += 0.5 * (g[k] + gprev) * (r - rprev);
+            rprev = r;
+            gprev = g[k];
+        } else {
+            g[k] = NAN;
+        }
+        if (num) num[k] = o.num[k];
+        if (cnt) cnt[k] = (int64_t)o.cnt[k];
+    }
+    if (L_int) *L_int = den > 0 ? li : NAN;
+}
+
+}  // namespace vcf
+}  // namespace dpd
