@@ -246,6 +246,13 @@ __global__ void __launch_bounds__(tile_threads<B, 2>(), tile_ctas<B, 2>())
     if (busy) add_busy(busy, t0);
 }
 
+// Overflow count and error flag of every replica.
+__global__ void k_ens_status(const Sys *__restrict__ sys, int R, ulonglong2 *out)
+{
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < R) out[r] = make_ulonglong2(*sys[r].ovf, (unsigned long long)(unsigned)*sys[r].err);
+}
+
 // Self-test of the bounded barrier: block 0 never arrives, every other block
 // must give up after the spin limit and latch DPD_ERR_TIMEOUT.
 __global__ void k_barrier_selftest(unsigned *bar, int *berr)
@@ -272,7 +279,8 @@ struct dpd_batch {
     size_t smem = 0;
     cudaGraphExec_t g = nullptr;
     int64_t g_steps = -1;
-    int *h_pin = nullptr;
+    ulonglong2 *h_pin = nullptr;   // page-locked: [0] the batch's error word, [1 + r] replica r
+    ulonglong2 *d_status = nullptr;
     // variant 2: the force items by classes of threads per tile, each launched
     // on a stream of its own beside the others, and the step graphs
     struct Class { int nt, cap, first, n, slots; size_t smem; };
@@ -538,13 +546,15 @@ static int ens_build_tables(dpd_batch *b)
     b->n_scat = (int)scat.size();
     b->n_tiles = (int)tiles.size();
     if (b->pool) cudaFree(b->pool);
-    const size_t bytes = sizeof(Sys) * (size_t)b->R + 4 * scan.size() + 4 * scat.size() + 4 * tiles.size() + 256 * 5;
+    const size_t bytes = sizeof(Sys) * (size_t)b->R + 4 * scan.size() + 4 * scat.size() + 4 * tiles.size() +
+                         sizeof(ulonglong2) * (size_t)b->R + 256 * 6;
     CUB(cudaMalloc(&b->pool, bytes));
     char *p = (char *)b->pool;
     b->d_sys = (Sys *)p; p += (sizeof(Sys) * (size_t)b->R + 255) & ~size_t(255);
     b->d_scan = (uint32_t *)p; p += (4 * scan.size() + 255) & ~size_t(255);
     b->d_scat = (uint32_t *)p; p += (4 * scat.size() + 255) & ~size_t(255);
     b->d_tiles = (uint32_t *)p; p += (4 * tiles.size() + 255) & ~size_t(255);
+    b->d_status = (ulonglong2 *)p; p += (sizeof(ulonglong2) * (size_t)b->R + 255) & ~size_t(255);
     b->d_bar = (unsigned *)p;          // 2 words
     b->d_err = (int *)(b->d_bar + 8);  // 1 word
     b->d_ctr = (unsigned long long *)(b->d_bar + 16);
@@ -648,7 +658,7 @@ int dpd_batch_create(const dpd_params *p, int R, void *stream, dpd_batch **out)
         rc = dpd_create(&q[r], b->st, &b->reps[r]);
         if (rc == DPD_OK) b->reps[r]->batch_owned = true;
     }
-    if (rc == DPD_OK && cudaMallocHost((void **)&b->h_pin, 64) != cudaSuccess) rc = DPD_ERR_OOM;
+    if (rc == DPD_OK && cudaMallocHost((void **)&b->h_pin, sizeof(ulonglong2) * (size_t)(R + 1)) != cudaSuccess) rc = DPD_ERR_OOM;
     if (rc == DPD_OK && b->var == 2) {
         bool ok = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
         for (int i = 0; i < dpd_batch::MAX_CLASSES - 1; ++i)
@@ -749,14 +759,21 @@ int dpd_batch_step(dpd_batch *b, int64_t n)
 int dpd_batch_sync(dpd_batch *b)
 {
     if (!b) return DPD_ERR_INVALID_ARG;
+    // every replica's status in one copy (two copies and a wait per replica took
+    // 4 ms for 256)
+    k_ens_status<<<(b->R + 127) / 128, 128, 0, b->st>>>(b->d_sys, b->R, b->d_status);
+    CUB(cudaGetLastError());
     CUB(cudaMemcpyAsync(b->h_pin, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->st));
+    CUB(cudaMemcpyAsync(b->h_pin + 1, b->d_status, sizeof(ulonglong2) * (size_t)b->R, cudaMemcpyDeviceToHost, b->st));
     CUB(cudaStreamSynchronize(b->st));
     int status = DPD_OK;
-    if (b->h_pin[0] & ERR_TIMEOUT) status = DPD_ERR_TIMEOUT;
+    if (*(const int *)b->h_pin & ERR_TIMEOUT) status = DPD_ERR_TIMEOUT;
     bool grown = false;
-    for (dpd_ctx *c : b->reps) {
-        const unsigned long long seen = c->ovf_seen;
-        const int rc = dpd_internal_latched(c);
+    for (int r = 0; r < b->R; ++r) {
+        dpd_ctx *c = b->reps[r];
+        const unsigned long long seen = c->ovf_seen, e = b->h_pin[1 + r].y;
+        c->ovf_seen = std::max(seen, b->h_pin[1 + r].x);
+        const int rc = e & ERR_NONFINITE ? DPD_ERR_NONFINITE : e & ERR_TIMEOUT ? DPD_ERR_TIMEOUT : e & ERR_INTERNAL ? DPD_ERR_INTERNAL : DPD_OK;
         if (rc && status == DPD_OK) status = rc;
         // tiles of this replica took the global-memory path: a quarter more
         // room for its class, as a single system's
@@ -785,7 +802,7 @@ int dpd_batch_barrier_selftest(dpd_batch *b)
     CUB(cudaGetLastError());
     CUB(cudaMemcpyAsync(b->h_pin, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->st));
     CUB(cudaStreamSynchronize(b->st));
-    const int seen = b->h_pin[0];
+    const int seen = *(const int *)b->h_pin;
     // leave the batch usable: clear the error word and the barrier state
     CUB(cudaMemsetAsync(b->d_bar, 0, 64, b->st));
     CUB(cudaStreamSynchronize(b->st));

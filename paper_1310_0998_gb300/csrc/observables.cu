@@ -31,50 +31,13 @@ struct ObsScratch {
     size_t bytes = 0;
 };
 
-// Positions enter as the exact doubles X L / 2^32 of the fixed-point state.
-__global__ void k_agent_com(const uint4 *__restrict__ xv, int na, double L, double ulen, double2 *c, double2 *v)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= na) return;
-    const uint4 h = xv[2 * k], t = xv[2 * k + 1];
-    const double hx = __dmul_rn((double)h.x, ulen), hy = __dmul_rn((double)h.y, ulen);
-    const double tx = __dmul_rn((double)t.x, ulen), ty = __dmul_rn((double)t.y, ulen);
-    const double dx = minimg_d(__dsub_rn(hx, tx), L);
-    const double dy = minimg_d(__dsub_rn(hy, ty), L);
-    double cx = __dadd_rn(tx, __dmul_rn(0.5, dx));
-    double cy = __dadd_rn(ty, __dmul_rn(0.5, dy));
-    cx = __dsub_rn(cx, __dmul_rn(L, floor(__ddiv_rn(cx, L))));
-    cy = __dsub_rn(cy, __dmul_rn(L, floor(__ddiv_rn(cy, L))));
-    c[k] = make_double2(cx, cy);
-    const double hvx = (double)__uint_as_float(h.z), hvy = (double)__uint_as_float(h.w);
-    const double tvx = (double)__uint_as_float(t.z), tvy = (double)__uint_as_float(t.w);
-    v[k] = make_double2(__dmul_rn(0.5, __dadd_rn(hvx, tvx)), __dmul_rn(0.5, __dadd_rn(hvy, tvy)));
-}
-
-__global__ void k_deposit(const double2 *c, const double2 *v, int na, double L, double dxg, double half, int M,
-                          double *sx, double *sy, double *cnt)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= na) return;
-    int ix[64], iy[64];
-    const double2 ck = c[k], vk = v[k];
-    const int nx = window_hits(ck.x, L, dxg, half, M, ix, 64);
-    const int ny = window_hits(ck.y, L, dxg, half, M, iy, 64);
-    for (int a = 0; a < ny; ++a)
-        for (int b = 0; b < nx; ++b) {
-            const size_t g = (size_t)iy[a] * M + ix[b];
-            atomicAdd(&sx[g], vk.x);
-            atomicAdd(&sy[g], vk.y);
-            atomicAdd(&cnt[g], 1.0);
-        }
-}
-
+// u = window mean, 0 if empty, from the window sums (2 v_x, 2 v_y, count).
 __global__ void k_field_finish(const double *sx, const double *sy, const double *cnt, int MM, double2 *z)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= MM) return;
     const double n = cnt[g];
-    z[g] = n > 0.0 ? make_double2(sx[g] / n, sy[g] / n) : make_double2(0.0, 0.0);
+    z[g] = n > 0.0 ? make_double2(0.5 * sx[g] / n, 0.5 * sy[g] / n) : make_double2(0.0, 0.0);
 }
 
 // Scalar vorticity of the field, omega = du_y/dx - du_x/dy (Sec. 5.3), by
@@ -97,7 +60,7 @@ __global__ void k_shells(const double2 *Z, int M, double scale, double *E)
     if (g >= M * M) return;
     const int iy = g / M, ix = g - iy * M;
     const int ky = iy < M / 2 ? iy : iy - M, kx = ix < M / 2 ? ix : ix - M;
-    const int sh = (int)rint(sqrt((double)(kx * kx + ky * ky)));
+    const int sh = shell_of(kx * kx + ky * ky);
     if (sh >= 1 && sh <= M / 2) {
         const double2 a = Z[g];
         atomicAdd(&E[sh - 1], (a.x * a.x + a.y * a.y) * scale);
@@ -110,8 +73,8 @@ __global__ void k_agent_speed(const uint4 *__restrict__ xv, int na, double *acc)
     double s = 0.0;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < na; k += gridDim.x * blockDim.x) {
         const uint4 h = xv[2 * k], t = xv[2 * k + 1];
-        const double vx = __dmul_rn(0.5, __dadd_rn((double)__uint_as_float(h.z), (double)__uint_as_float(t.z)));
-        const double vy = __dmul_rn(0.5, __dadd_rn((double)__uint_as_float(h.w), (double)__uint_as_float(t.w)));
+        const double vx = __dmul_rn(0.5, __dadd_rn(to_double(__uint_as_float(h.z)), to_double(__uint_as_float(t.z))));
+        const double vy = __dmul_rn(0.5, __dadd_rn(to_double(__uint_as_float(h.w)), to_double(__uint_as_float(t.w))));
         s += sqrt(__dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)));
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -157,8 +120,22 @@ void dpd_internal_free_obs(dpd_ctx *c)
             return e_ == cudaErrorMemoryAllocation ? DPD_ERR_OOM : DPD_ERR_CUDA; \
     } while (0)
 
+// A result of a few values to the caller and the latched status: through the
+// context's page-locked buffer, since a copy to pageable memory waits by itself.
+static int small_out(dpd_ctx *c, void *to, const void *from, size_t bytes)
+{
+    if (bytes > H_PIN_SMALL) {
+        CUO(cudaMemcpyAsync(to, from, bytes, cudaMemcpyDeviceToHost, c->st));
+        return dpd_internal_latched(c);
+    }
+    CUO(cudaMemcpyAsync(c->h_pin, from, bytes, cudaMemcpyDeviceToHost, c->st));
+    const int rc = dpd_internal_latched(c);
+    std::memcpy(to, c->h_pin, bytes);
+    return rc;
+}
+
 // Field on the device: z [M*M] double2 (u_x, u_y), cnt [M*M], and a tail of
-// at least tail_bytes for the caller.  Every sub-buffer starts on a 256-byte
+// tail_bytes (cleared) for the caller.  Every sub-buffer starts on a 256-byte
 // boundary (z is read as double2, which needs 16; an odd M*M must not shift it).
 static int field_device(dpd_ctx *c, int M, double eps, size_t tail_bytes, double2 **z_out, double **cnt_out,
                         char **tail)
@@ -166,21 +143,17 @@ static int field_device(dpd_ctx *c, int M, double eps, size_t tail_bytes, double
     const int na = c->d.n / 2;
     const size_t MM = (size_t)M * M;
     auto up = [](size_t o) { return (o + 255) & ~size_t(255); };
-    const size_t o_cc = 0, o_vv = up(o_cc + 16 * (size_t)na), o_s = up(o_vv + 16 * (size_t)na);
-    const size_t o_z = up(o_s + 24 * MM), o_tail = up(o_z + 16 * MM);
-    ObsScratch *s = scratch_of(c, o_tail + tail_bytes + 256);
+    const size_t o_tail = up(24 * MM), o_z = up(o_tail + tail_bytes);
+    ObsScratch *s = scratch_of(c, o_z + 16 * MM + 256);
     if (!s) return DPD_ERR_OOM;
     char *b = (char *)s->buf;
-    double2 *cc = (double2 *)(b + o_cc);
-    double2 *vv = (double2 *)(b + o_vv);
-    double *sx = (double *)(b + o_s), *sy = sx + MM, *cn = sy + MM;   // contiguous: one clear
+    double *sum = (double *)b, *cn = sum + 2 * MM;
     double2 *z = (double2 *)(b + o_z);
     const double L = c->p.L;
     if (eps <= 0.0) eps = L * std::sqrt(10.0 / (double)na);
-    CUO(cudaMemsetAsync(sx, 0, 8 * MM * 3, c->st));
-    k_agent_com<<<(na + 255) / 256, 256, 0, c->st>>>(c->d.C_xv, na, L, c->d.ulen_d, cc, vv);
-    k_deposit<<<(na + 127) / 128, 128, 0, c->st>>>(cc, vv, na, L, L / M, 0.5 * eps, M, sx, sy, cn);
-    k_field_finish<<<(int)((MM + 255) / 256), 256, 0, c->st>>>(sx, sy, cn, (int)MM, z);
+    CUO(cudaMemsetAsync(b, 0, o_z, c->st));
+    deposit<2>(ObsState{c->d.C_xv, nullptr, na, L, c->d.ulen_d}, M, eps, sum, c->st);
+    k_field_finish<<<(int)((MM + 255) / 256), 256, 0, c->st>>>(sum, sum + MM, cn, (int)MM, z);
     CUO(cudaGetLastError());
     *z_out = z;
     *cnt_out = cn;
@@ -219,17 +192,13 @@ int dpd_energy_spectrum(dpd_ctx *c, int M, double eps, double *E)
     if (rc) return rc;
     int logM = 0;
     while ((1 << logM) < M) ++logM;
-    const size_t sm = 16 * (size_t)M;
-    const int thr = M / 2 < 512 ? M / 2 : 512;
-    k_fft<<<M, thr, sm, c->st>>>(z, M, logM, 1, M, M, 0);   // rows (along x)
-    k_fft<<<M, thr, sm, c->st>>>(z, M, logM, M, M, 1, 0);   // columns (along y)
+    fft_axis(z, M, logM, 1, M, M, 0, M, c->st);   // rows (along x)
+    fft_axis(z, M, logM, M, M, 1, 0, M, c->st);   // columns (along y)
     double *dE = (double *)tail;
-    CUO(cudaMemsetAsync(dE, 0, 8 * (size_t)(M / 2), c->st));
     const double M2 = (double)M * (double)M;
     k_shells<<<(M * M + 255) / 256, 256, 0, c->st>>>(z, M, 0.5 / (M2 * M2), dE);
     CUO(cudaGetLastError());
-    CUO(cudaMemcpyAsync(E, dE, 8 * (size_t)(M / 2), cudaMemcpyDeviceToHost, c->st));
-    return dpd_internal_latched(c);
+    return small_out(c, E, dE, 8 * (size_t)(M / 2));
 }
 
 int dpd_vorticity(dpd_ctx *c, int M, double eps, double *omega)
@@ -264,8 +233,7 @@ int dpd_agent_speed(dpd_ctx *c, double *mean_speed)
     k_agent_speed<<<std::min((na + 255) / 256, 1024), 256, 0, c->st>>>(c->d.C_xv, na, acc);
     CUO(cudaGetLastError());
     double h = 0.0;
-    CUO(cudaMemcpyAsync(&h, acc, 8, cudaMemcpyDeviceToHost, c->st));
-    const int rc = dpd_internal_latched(c);
+    const int rc = small_out(c, &h, acc, 8);
     *mean_speed = h / na;
     return rc;
 }
@@ -291,10 +259,11 @@ int dpd_velocity_correlation(dpd_ctx *c, double dr, int nbins, double *g, double
     ObsScratch *s = scratch_of(c, vcf::Layout((size_t)na, (size_t)nbins, vcf::cells_of<2>(n)).bytes);
     if (!s) return DPD_ERR_OOM;
     const vcf::State state{c->d.C_xv, nullptr, na, L, c->d.ulen_d};
-    std::vector<long long> host;
-    int rc = vcf::vcf_run<2>(state, dr, nbins, m, n, (char *)s->buf, c->st, host);
+    std::vector<long long> host(vcf::result_words(nbins));
+    const void *res = nullptr;
+    int rc = vcf::vcf_run<2>(state, dr, nbins, m, n, (char *)s->buf, c->st, &res);
     if (rc) return rc;
-    rc = dpd_internal_latched(c);
+    rc = small_out(c, host.data(), res, 8 * host.size());
     vcf::vcf_outputs(vcf::vcf_finish<2>(host, na, nbins), dr, nbins, g, L_int, num, cnt);
     return rc;
 }
@@ -313,13 +282,10 @@ int dpd_velocity_correlation(dpd_ctx *c, double dr, int nbins, double *g, double
 // synchronise the whole device and stall the other streams.  This variant
 // keeps its scratch in one fixed static device array instead.
 //
-// How.  The agent centres of mass and velocities, which the allocating path
-// stages in a per-agent buffer, are recomputed inside the deposit kernel
-// (k_deposit_state, the same IEEE operations as k_agent_com), so the scratch
-// no longer grows with the number of agents; what remains is the grid:
-// per point the window sums of u_x and u_y, the window count and the complex
-// field (5 doubles), plus M/2 shell sums: 2,622,464 bytes at the maximum
-// M = 256.  Larger M is rejected.
+// How.  The window sums come straight from the state (k_deposit), so the
+// scratch does not grow with the number of agents: per grid point the window
+// sums of u_x and u_y, the window count and the complex field (5 doubles), plus
+// M/2 shell sums: 2,622,464 bytes at the maximum M = 256.  Larger M is rejected.
 //
 // What must start at zero.  The three window sums and the shell sums are
 // accumulated with atomics; every call clears them (cudaMemsetAsync on the
@@ -366,41 +332,6 @@ static int spectrum_scratch(int ctx_dev, double **out)
     return DPD_OK;
 }
 
-namespace dpd {
-
-// k_agent_com followed by k_deposit for one agent, without staging the
-// centres of mass and velocities in memory.
-__global__ void k_deposit_state(const uint4 *__restrict__ xv, int na, double L, double ulen, double dxg,
-                                double half, int M, double *sx, double *sy, double *cnt)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= na) return;
-    const uint4 h = xv[2 * k], t = xv[2 * k + 1];
-    const double hx = __dmul_rn((double)h.x, ulen), hy = __dmul_rn((double)h.y, ulen);
-    const double tx = __dmul_rn((double)t.x, ulen), ty = __dmul_rn((double)t.y, ulen);
-    const double dx = minimg_d(__dsub_rn(hx, tx), L);
-    const double dy = minimg_d(__dsub_rn(hy, ty), L);
-    double cx = __dadd_rn(tx, __dmul_rn(0.5, dx));
-    double cy = __dadd_rn(ty, __dmul_rn(0.5, dy));
-    cx = __dsub_rn(cx, __dmul_rn(L, floor(__ddiv_rn(cx, L))));
-    cy = __dsub_rn(cy, __dmul_rn(L, floor(__ddiv_rn(cy, L))));
-    const double hvx = (double)__uint_as_float(h.z), hvy = (double)__uint_as_float(h.w);
-    const double tvx = (double)__uint_as_float(t.z), tvy = (double)__uint_as_float(t.w);
-    const double vx = __dmul_rn(0.5, __dadd_rn(hvx, tvx)), vy = __dmul_rn(0.5, __dadd_rn(hvy, tvy));
-    int ix[64], iy[64];
-    const int nx = window_hits(cx, L, dxg, half, M, ix, 64);
-    const int ny = window_hits(cy, L, dxg, half, M, iy, 64);
-    for (int a = 0; a < ny; ++a)
-        for (int b = 0; b < nx; ++b) {
-            const size_t g = (size_t)iy[a] * M + ix[b];
-            atomicAdd(&sx[g], vx);
-            atomicAdd(&sy[g], vy);
-            atomicAdd(&cnt[g], 1.0);
-        }
-}
-
-}  // namespace dpd
-
 extern "C" int dpd_energy_spectrum_noalloc(dpd_ctx *c, int M, double eps, double *E)
 {
     if (!c || !E || M < 4 || M > NOALLOC_MAX_M || (M & (M - 1))) return DPD_ERR_INVALID_ARG;
@@ -418,18 +349,14 @@ extern "C" int dpd_energy_spectrum_noalloc(dpd_ctx *c, int M, double eps, double
     double *dE = (double *)(z + MM);
     CUO(cudaMemsetAsync(sx, 0, 8 * MM * 3, c->st));
     CUO(cudaMemsetAsync(dE, 0, 8 * (size_t)(M / 2), c->st));
-    k_deposit_state<<<(na + 127) / 128, 128, 0, c->st>>>(c->d.C_xv, na, L, c->d.ulen_d, L / M, 0.5 * eps, M, sx,
-                                                         sy, cn);
+    deposit<2>(ObsState{c->d.C_xv, nullptr, na, L, c->d.ulen_d}, M, eps, sx, c->st);
     k_field_finish<<<(int)((MM + 255) / 256), 256, 0, c->st>>>(sx, sy, cn, (int)MM, z);
     int logM = 0;
     while ((1 << logM) < M) ++logM;
-    const size_t sm = 16 * (size_t)M;
-    const int thr = M / 2 < 512 ? M / 2 : 512;
-    k_fft<<<M, thr, sm, c->st>>>(z, M, logM, 1, M, M, 0);
-    k_fft<<<M, thr, sm, c->st>>>(z, M, logM, M, M, 1, 0);
+    fft_axis(z, M, logM, 1, M, M, 0, M, c->st);
+    fft_axis(z, M, logM, M, M, 1, 0, M, c->st);
     const double M2 = (double)M * (double)M;
     k_shells<<<(M * M + 255) / 256, 256, 0, c->st>>>(z, M, 0.5 / (M2 * M2), dE);
     CUO(cudaGetLastError());
-    CUO(cudaMemcpyAsync(E, dE, 8 * (size_t)(M / 2), cudaMemcpyDeviceToHost, c->st));
-    return dpd_internal_latched(c);
+    return small_out(c, E, dE, 8 * (size_t)(M / 2));
 }

@@ -34,55 +34,6 @@
 
 namespace dpd {
 
-// Agent position or velocity, FP64 (x, y, z, padding), 32-byte aligned.
-struct __align__(32) D4 {
-    double x, y, z, w;
-};
-
-__global__ void k3_agent_com(const uint4 *__restrict__ p, const float4 *__restrict__ v, int na, double L, double ulen,
-                             D4 *c, D4 *vc)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= na) return;
-    const uint4 h = p[2 * k], t = p[2 * k + 1];
-    const double hx = __dmul_rn((double)h.x, ulen), hy = __dmul_rn((double)h.y, ulen), hz = __dmul_rn((double)h.z, ulen);
-    const double tx = __dmul_rn((double)t.x, ulen), ty = __dmul_rn((double)t.y, ulen), tz = __dmul_rn((double)t.z, ulen);
-    double cx = __dadd_rn(tx, __dmul_rn(0.5, minimg_d(__dsub_rn(hx, tx), L)));
-    double cy = __dadd_rn(ty, __dmul_rn(0.5, minimg_d(__dsub_rn(hy, ty), L)));
-    double cz = __dadd_rn(tz, __dmul_rn(0.5, minimg_d(__dsub_rn(hz, tz), L)));
-    cx = __dsub_rn(cx, __dmul_rn(L, floor(__ddiv_rn(cx, L))));
-    cy = __dsub_rn(cy, __dmul_rn(L, floor(__ddiv_rn(cy, L))));
-    cz = __dsub_rn(cz, __dmul_rn(L, floor(__ddiv_rn(cz, L))));
-    c[k] = D4{cx, cy, cz, 0.0};
-    const float4 a = v[2 * k], b = v[2 * k + 1];
-    vc[k] = D4{__dmul_rn(0.5, __dadd_rn((double)a.x, (double)b.x)), __dmul_rn(0.5, __dadd_rn((double)a.y, (double)b.y)),
-               __dmul_rn(0.5, __dadd_rn((double)a.z, (double)b.z)), 0.0};
-}
-
-constexpr int WIN3 = 32;   // window hits per axis (the host keeps eps / (L / M) <= 28)
-
-// Window sums: sum u_x, u_y, u_z and count per grid point (z-major [iz][iy][ix]).
-__global__ void k3_deposit(const D4 *c, const D4 *vc, int na, double L, double dxg, double half, int M,
-                           double *sx, double *sy, double *sz, double *cnt)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= na) return;
-    int ix[WIN3], iy[WIN3], iz[WIN3];
-    const D4 ck = c[k], vk = vc[k];
-    const int nx = window_hits(ck.x, L, dxg, half, M, ix, WIN3);
-    const int ny = window_hits(ck.y, L, dxg, half, M, iy, WIN3);
-    const int nz = window_hits(ck.z, L, dxg, half, M, iz, WIN3);
-    for (int a = 0; a < nz; ++a)
-        for (int b = 0; b < ny; ++b)
-            for (int q = 0; q < nx; ++q) {
-                const size_t g = ((size_t)iz[a] * M + iy[b]) * M + ix[q];
-                atomicAdd(&sx[g], vk.x);
-                atomicAdd(&sy[g], vk.y);
-                atomicAdd(&sz[g], vk.z);
-                atomicAdd(&cnt[g], 1.0);
-            }
-}
-
 // u = window mean (0 if empty), stored as z1 = u_x + i u_y and z2 = u_z + 0 i.
 __global__ void k3_field_finish(const double *sx, const double *sy, const double *sz, const double *cnt, long long MMM,
                                 double2 *z1, double2 *z2)
@@ -90,8 +41,8 @@ __global__ void k3_field_finish(const double *sx, const double *sy, const double
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= MMM) return;
     const double n = cnt[g];
-    z1[g] = n > 0.0 ? make_double2(sx[g] / n, sy[g] / n) : make_double2(0.0, 0.0);
-    z2[g] = make_double2(n > 0.0 ? sz[g] / n : 0.0, 0.0);
+    z1[g] = n > 0.0 ? make_double2(0.5 * sx[g] / n, 0.5 * sy[g] / n) : make_double2(0.0, 0.0);   // the sums hold 2 v
+    z2[g] = make_double2(n > 0.0 ? 0.5 * sz[g] / n : 0.0, 0.0);
 }
 
 __global__ void k3_field_out(const double2 *z1, const double2 *z2, long long MMM, double *u)
@@ -139,7 +90,7 @@ __global__ void k3_shells(const double2 *Z1, const double2 *Z2, int M, double sc
          g += (long long)gridDim.x * blockDim.x) {
         const int iz = (int)(g / MM), iy = (int)((g / M) % M), ix = (int)(g % M);
         const int kz = iz < M / 2 ? iz : iz - M, ky = iy < M / 2 ? iy : iy - M, kx = ix < M / 2 ? ix : ix - M;
-        const int sh = (int)rint(sqrt((double)(kx * kx + ky * ky + kz * kz)));
+        const int sh = shell_of(kx * kx + ky * ky + kz * kz);
         if (sh >= 1 && sh <= nsh) {
             const double2 a = Z1[g], b = Z2[g];
             atomicAdd(&es[sh - 1], (a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y) * scale);
@@ -186,17 +137,14 @@ static int field3_device(dpd3_ctx *c, int M, double eps, size_t tail_bytes, doub
     const int na = c->s.b.n / 2;
     const size_t MMM = (size_t)M * M * M;
     auto up = [](size_t o) { return (o + 255) & ~size_t(255); };
-    const size_t o_cc = 0, o_vv = up(o_cc + 32 * (size_t)na), o_s = up(o_vv + 32 * (size_t)na);
-    const size_t o_z = up(o_s + 32 * MMM), o_tail = up(o_z + 32 * MMM);
-    char *b = scratch3(c, o_tail + tail_bytes + 256);
+    const size_t o_tail = up(32 * MMM), o_z = up(o_tail + tail_bytes);
+    char *b = scratch3(c, o_z + 32 * MMM + 256);
     if (!b) return DPD_ERR_OOM;
-    D4 *cc = (D4 *)(b + o_cc), *vv = (D4 *)(b + o_vv);
-    double *sx = (double *)(b + o_s), *sy = sx + MMM, *sz = sy + MMM, *cn = sz + MMM;   // one clear
+    double *sx = (double *)b, *sy = sx + MMM, *sz = sy + MMM, *cn = sz + MMM;
     double2 *z = (double2 *)(b + o_z);
     const double L = c->p.L;
-    CUO3(cudaMemsetAsync(sx, 0, 32 * MMM, c->st));
-    k3_agent_com<<<(na + 255) / 256, 256, 0, c->st>>>(c->s.C_p, c->s.C_v, na, L, c->s.b.ulen_d, cc, vv);
-    k3_deposit<<<(na + 127) / 128, 128, 0, c->st>>>(cc, vv, na, L, L / M, 0.5 * eps, M, sx, sy, sz, cn);
+    CUO3(cudaMemsetAsync(b, 0, 32 * MMM, c->st));
+    deposit<3>(ObsState{c->s.C_p, c->s.C_v, na, L, c->s.b.ulen_d}, M, eps, sx, c->st);
     k3_field_finish<<<(unsigned)((MMM + 255) / 256), 256, 0, c->st>>>(sx, sy, sz, cn, (long long)MMM, z, z + MMM);
     CUO3(cudaGetLastError());
     *z_out = z;
@@ -247,12 +195,10 @@ int dpd3_energy_spectrum(dpd3_ctx *c, int M, double eps, double *E)
     if (rc) return rc;
     int logM = 0;
     while ((1 << logM) < M) ++logM;
-    const size_t sm = 16 * (size_t)M;
-    const int thr = M / 2;
-    const unsigned lines = (unsigned)(2 * MM);   // M^2 lines per axis in each of z1, z2
-    k_fft<<<lines, thr, sm, c->st>>>(z, M, logM, 1, (int)(2 * MM), M, 0);    // along x
-    k_fft<<<lines, thr, sm, c->st>>>(z, M, logM, M, M, 1, MM);               // along y
-    k_fft<<<lines, thr, sm, c->st>>>(z, M, logM, MM, (int)MM, 1, MMM);       // along z
+    const int lines = (int)(2 * MM);   // M^2 lines per axis in each of z1, z2
+    fft_axis(z, M, logM, 1, lines, M, 0, lines, c->st);          // along x
+    fft_axis(z, M, logM, M, M, 1, MM, lines, c->st);             // along y
+    fft_axis(z, M, logM, MM, (int)MM, 1, MMM, lines, c->st);     // along z
     double *dE = (double *)tail;
     CUO3(cudaMemsetAsync(dE, 0, 8 * (size_t)(M / 2), c->st));
     const double M3 = (double)MMM;
@@ -302,9 +248,11 @@ int dpd3_velocity_correlation(dpd3_ctx *c, double dr, int nbins, double *g, doub
     char *buf = scratch3(c, vcf::Layout((size_t)na, (size_t)nbins, vcf::cells_of<3>(n)).bytes);
     if (!buf) return DPD_ERR_OOM;
     const vcf::State state{c->s.C_p, c->s.C_v, na, L, c->s.b.ulen_d};
-    std::vector<long long> host;
-    int rc = vcf::vcf_run<3>(state, dr, nbins, m, n, buf, c->st, host);
+    std::vector<long long> host(vcf::result_words(nbins));
+    const void *res = nullptr;
+    int rc = vcf::vcf_run<3>(state, dr, nbins, m, n, buf, c->st, &res);
     if (rc) return rc;
+    CUO3(cudaMemcpyAsync(host.data(), res, 8 * host.size(), cudaMemcpyDeviceToHost, c->st));
     rc = dpd3_internal_latched(c);
     vcf::vcf_outputs(vcf::vcf_finish<3>(host, na, nbins), dr, nbins, g, L_int, num, cnt);
     return rc;

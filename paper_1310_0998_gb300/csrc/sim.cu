@@ -519,7 +519,7 @@ static int ensure_graphs(dpd_ctx *c)
     return DPD_OK;
 }
 
-constexpr int H_PIN_STATUS = 510;   // h_pin holds 512 doubles; [510], [511]: error flag, overflow count
+constexpr int H_PIN_STATUS = 476;   // h_pin holds 512 doubles; the status words' slots begin here
 
 // A tile that did not fit in shared memory ran the global-memory path: raise
 // the capacity by a quarter (within the shared-memory limit) and re-capture
@@ -541,11 +541,14 @@ int dpd_internal_latched(dpd_ctx *c)
     int e = 0;
     unsigned long long ovf = 0;
     double *st = c->h_pin + H_PIN_STATUS;
-    CU(cudaMemcpyAsync(st, c->d.err, sizeof(int), cudaMemcpyDeviceToHost, c->st));
-    CU(cudaMemcpyAsync(st + 1, c->d.ovf, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->st));
+    // the overflow count and the error flag sit in neighbouring slices of the
+    // pool: one copy takes both
+    const size_t gap = (size_t)((const char *)c->d.err - (const char *)c->d.ovf);
+    static_assert(H_PIN_STATUS * sizeof(double) >= H_PIN_SMALL && (H_PIN_STATUS + 33) * sizeof(double) <= 4096, "pinned slots");
+    CU(cudaMemcpyAsync(st, c->d.ovf, gap + sizeof(int), cudaMemcpyDeviceToHost, c->st));
     CU(cudaStreamSynchronize(c->st));
-    std::memcpy(&e, st, sizeof(int));
-    std::memcpy(&ovf, st + 1, sizeof(ovf));
+    std::memcpy(&ovf, st, sizeof(ovf));
+    std::memcpy(&e, (const char *)st + gap, sizeof(int));
     if (ovf > c->ovf_seen) {
         c->ovf_seen = ovf;
         if (!c->batch_owned) grow_capacity(c);

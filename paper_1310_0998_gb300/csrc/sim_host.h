@@ -25,6 +25,7 @@ void launch_bin(const Sys &d, int B, cudaStream_t st);
 void launch_kick_bin(const Sys &d, int B, cudaStream_t st);
 int host_cell_of(int B, int nc, int cx, int cy);
 bool tuned_shape(const dpd_params *p, int R, int *tile, int *variant);
+constexpr size_t H_PIN_SMALL = 3584;   // bytes at the start of a context's page-locked buffer for small results
 constexpr int DEFAULT_TILE = 8, DEFAULT_VARIANT = 2;
 }  // namespace dpd
 

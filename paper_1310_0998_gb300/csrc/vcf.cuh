@@ -39,14 +39,7 @@
 namespace dpd {
 namespace vcf {
 
-// Canonical state in id order; beads 2k and 2k + 1 are agent k.  In two
-// dimensions the velocity is in p.z, p.w and v is unused.
-struct State {
-    const uint4 *p;
-    const float4 *v;
-    int na;
-    double L, ulen;
-};
+using State = ObsState;
 
 template <int D>
 struct Agent {
@@ -57,24 +50,14 @@ struct Agent {
 template <int D>
 __device__ __forceinline__ Agent<D> load_agent(const State &s, int k)
 {
-    const uint4 h = s.p[2 * (size_t)k], t = s.p[2 * (size_t)k + 1];
-    const uint32_t hx[3] = {h.x, h.y, h.z}, tx[3] = {t.x, t.y, t.z};
-    float hv[3], tv[3];
-    if constexpr (D == 2) {
-        hv[0] = __uint_as_float(h.z); hv[1] = __uint_as_float(h.w);
-        tv[0] = __uint_as_float(t.z); tv[1] = __uint_as_float(t.w);
-    } else {
-        const float4 a = s.v[2 * (size_t)k], b = s.v[2 * (size_t)k + 1];
-        hv[0] = a.x; hv[1] = a.y; hv[2] = a.z;
-        tv[0] = b.x; tv[1] = b.y; tv[2] = b.z;
-    }
+    const AgentBeads<D> a = load_beads<D>(s, k);
     Agent<D> g;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        g.c[i] = (2ull * tx[i] + (unsigned long long)(long long)(int)(hx[i] - tx[i])) & 0x1ffffffffull;
-        const float x = __fadd_rn(hv[i], tv[i]), bb = __fsub_rn(x, hv[i]);
+        g.c[i] = com33(a.hx[i], a.tx[i]);
+        const float x = __fadd_rn(a.hv[i], a.tv[i]), bb = __fsub_rn(x, a.hv[i]);
         g.sh[i] = x;
-        g.sl[i] = __fadd_rn(__fsub_rn(hv[i], __fsub_rn(x, bb)), __fsub_rn(tv[i], bb));
+        g.sl[i] = __fadd_rn(__fsub_rn(a.hv[i], __fsub_rn(x, bb)), __fsub_rn(a.tv[i], bb));
     }
     return g;
 }
@@ -337,16 +320,10 @@ struct Warp {
         }
         return d + __float2int_rn(c);
     }
-    // FP64 centre of mass, the operations of k_agent_com.
     __device__ __forceinline__ void com(int id, double *c) const
     {
-        const uint4 hd = p.s.p[2 * (size_t)id], tl = p.s.p[2 * (size_t)id + 1];
-        const uint32_t hx[3] = {hd.x, hd.y, hd.z}, tx[3] = {tl.x, tl.y, tl.z};
-        for (int i = 0; i < D; ++i) {
-            const double t = __dmul_rn((double)tx[i], p.s.ulen);
-            const double y = __dadd_rn(t, __dmul_rn(0.5, minimg_d(__dsub_rn(__dmul_rn((double)hx[i], p.s.ulen), t), p.s.L)));
-            c[i] = __dsub_rn(y, __dmul_rn(p.s.L, floor(__ddiv_rn(y, p.s.L))));
-        }
+        const AgentBeads<D> g = load_beads<D>(p.s, id);
+        for (int i = 0; i < D; ++i) c[i] = com_d(g.hx[i], g.tx[i], p.s.L, p.s.ulen);
     }
     // The last queued pairs (up to 32 of them) by the FP64 definition of their shell.
     __device__ __forceinline__ void drain()
@@ -536,13 +513,15 @@ struct Layout {
         rank = up(id + 4 * na);
         start = up(rank + (ncell ? 4 * na : 0));
         zero = up(start + 4 * (ncell + 1));
-        words = zero;                    // [0] vmax, [1] task counter, then 16 sums
-        cnt = up(words + 256);           // cell counts
-        bytes = up(cnt + 4 * ncell) + 8 * 4 * nbins;
+        words = zero;                    // [0] vmax, [1] task counter, then 16 sums, then the shell sums
+        cnt = up(gsum() + 8 * 4 * nbins);   // cell counts
+        bytes = cnt + 4 * ncell;
     }
     size_t sums() const { return words + 64; }
-    size_t gsum(size_t nbins) const { return bytes - 8 * 4 * nbins; }
+    size_t gsum() const { return words + 256; }
 };
+// 64-bit words of a pass's results (from Layout::words on).
+static inline size_t result_words(int nbins) { return 32 + 4 * (size_t)nbins; }
 
 #define VCF_CU(x)                                                                   \
     do {                                                                            \
@@ -567,10 +546,10 @@ template <int D>
 static size_t cells_of(int n) { return D == 2 ? (size_t)n * n : (size_t)n * n * n; }
 
 // One pass on `st`; buf holds Layout(na, nbins, n^D).bytes.  n = 0: all pairs.
-// Asynchronous up to the copies into the caller's host buffers, which are
-// complete after the caller's synchronisation; vcf_finish then makes Out.
+// Asynchronous; *res: the result words on the device, from which (copied to the
+// host) vcf_finish makes Out.
 template <int D>
-static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf, cudaStream_t st, std::vector<long long> &host)
+static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf, cudaStream_t st, const void **res)
 {
     const size_t ncell = cells_of<D>(n);
     const Layout l((size_t)s.na, (size_t)nbins, ncell);
@@ -589,7 +568,7 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     // 2^-24.  All pairs: the centres' 32 bits on top of three half-ulps.
     p.mg = (float)(nbins * 2e-6 + 2e-6 + (n > 0 ? 0.0 : s.L / dr * std::ldexp(1.0, -31)));
     p.lim2 = ((float)nbins + p.mg) * ((float)nbins + p.mg) * 1.000001f;
-    p.gsum = (long long *)(buf + l.gsum((size_t)nbins));
+    p.gsum = (long long *)(buf + l.gsum());
     p.gcnt = (unsigned long long *)(p.gsum + 3 * (size_t)nbins);
     VCF_CU(cudaMemsetAsync(buf + l.zero, 0, l.bytes - l.zero, st));
     int dev = 0, nsm = 0;
@@ -626,9 +605,7 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
         k_vcf_all<D><<<grid, 32 * wpb, sm, st>>>(p, (int)cols, (float)(std::ldexp(s.L, -32) / dr));
     }
     VCF_CU(cudaGetLastError());
-    host.resize(32 + 4 * (size_t)nbins);
-    VCF_CU(cudaMemcpyAsync(host.data(), buf + l.words, 256, cudaMemcpyDeviceToHost, st));
-    VCF_CU(cudaMemcpyAsync(host.data() + 32, p.gsum, 8 * 4 * (size_t)nbins, cudaMemcpyDeviceToHost, st));
+    *res = buf + l.words;
     return DPD_OK;
 }
 
