@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "dpd.h"
+#include "launch.cuh"
 #include "sim_host.h"
 #include "sim3d_host.h"
 #include "sim_kernels.cuh"
@@ -51,7 +52,9 @@ __device__ __forceinline__ int cell3(const Sys &d, uint32_t X, uint32_t Y, uint3
 __global__ void __launch_bounds__(SCAN_NT) k3_scan(Sys d, int nblocks)
 {
     __shared__ uint32_t s_buf[SCAN_BUF];
+    wait_for_previous();
     scan_decoupled_t<SCAN_NT>(d, nblocks, s_buf);
+    let_next_start();
 }
 
 __global__ void k3_bin(Sys3 s)
@@ -64,6 +67,7 @@ __global__ void k3_bin(Sys3 s)
 
 __global__ void k3_scatter(Sys3 s)
 {
+    wait_for_previous();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= s.b.n) return;
     const uint4 p = s.U_p[k];
@@ -204,6 +208,7 @@ __global__ void __launch_bounds__(PAIRS3_THREADS, 8) k3_pairs(Sys3 s)
     __shared__ uint32_t s_l[NW][10][32];      // and its length
     __shared__ long long s_r[NW][96];         // reactions of an evaluation, three words a pair
     __shared__ uint32_t s_rq[NW][32];         // and their slots (n: none)
+    wait_for_previous();
     __shared__ uint16_t s_q[NW][PAIRS3_Q];    // queued pairs: owner lane | slot in the run << 5 | run << 10
     const bool active = g < d.n;
     const long long step = *d.step;
@@ -375,6 +380,7 @@ __global__ void __launch_bounds__(256) k3_integrate(Sys3 s, int flags)
     __shared__ double s_big[4];
     if (threadIdx.x < 4) s_big[threadIdx.x] = 0.0;
     if (threadIdx.x == 0) s_vmax = 0u;
+    wait_for_previous();
     __syncthreads();
     float tv[3] = {0.f, 0.f, 0.f};   // v_s
     const uint32_t n = (uint32_t)d.n;
@@ -521,10 +527,10 @@ int dpd3_internal_latched(dpd3_ctx *c) { return latched3(c); }
 static void iteration3(dpd3_ctx *c, int flags)
 {
     const int g = (c->s.b.n + 255) / 256;
-    k3_scan<<<c->nscan, SCAN_NT, 0, c->st>>>(c->s.b, c->nscan);
-    k3_scatter<<<g, 256, 0, c->st>>>(c->s);
-    k3_pairs<<<(c->s.b.n + PAIRS3_THREADS - 1) / PAIRS3_THREADS, PAIRS3_THREADS, 0, c->st>>>(c->s);
-    k3_integrate<<<g, 256, 0, c->st>>>(c->s, flags);
+    launch_step(k3_scan, c->nscan, SCAN_NT, 0, c->st, c->s.b, c->nscan);
+    launch_step(k3_scatter, g, 256, 0, c->st, c->s);
+    launch_step(k3_pairs, (c->s.b.n + PAIRS3_THREADS - 1) / PAIRS3_THREADS, PAIRS3_THREADS, 0, c->st, c->s);
+    launch_step(k3_integrate, g, 256, 0, c->st, c->s, flags);
 }
 
 extern "C" {

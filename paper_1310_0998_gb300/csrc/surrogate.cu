@@ -28,8 +28,13 @@
 #include <cuda_runtime.h>
 
 #include "dpd.h"
+#include "launch.cuh"
 
 namespace sur {
+
+using dpd::launch_step;
+using dpd::let_next_start;
+using dpd::wait_for_previous;
 
 constexpr int NIN = 4, NIN_P = 16, NH = 256, NOUT = 40, NOUT_P = 48;
 
@@ -610,17 +615,6 @@ struct Rows {
 constexpr int GT_KC = 256, GT_THREADS = 256, GT_NT = 32;
 constexpr int GT_SMEM = (TC_M + GT_NT) * GT_KC * 2;
 
-// Programmatic launch order of a step's kernels.  Each kernel waits for the one
-// before it (which has waited for its own predecessor) and only then lets the
-// next one start, whose set-up and staging of weights so pass behind this
-// kernel's work; what runs before the wait reads nothing that the kernel before
-// writes, and writes nothing that it reads.
-__device__ __forceinline__ void wait_for_previous()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // Input c of row r, standardised (the operations of k_inputs).
 __device__ __forceinline__ float std_input(const Rows &b, int r, int c)
 {
@@ -685,6 +679,7 @@ __device__ __forceinline__ void gemm_tile(const __nv_bfloat16 *A, int M, int m0,
     if (EARLY == 1) stage_a(sa, 0, min(GT_KC, K));
     if (EARLY == 2) stage_tile(sb, B, n0, NT, N, 0, min(GT_KC, K), K);
     wait_for_previous();
+    let_next_start();
     uint32_t parity = 0;
     bool ok = true;
     for (int k0 = 0; k0 < K && ok; k0 += GT_KC) {
@@ -844,6 +839,7 @@ template <typename GET>
 __device__ __forceinline__ void colsum(int c, int M, float *out, GET get)
 {
     wait_for_previous();
+    let_next_start();
     const int lane = threadIdx.x & 31;
     float t = 0.f;
     for (int w = 0; w < 8 && 32 * w < M; ++w) {
@@ -907,6 +903,7 @@ __global__ void __launch_bounds__(256) k_adam_all(const Member *mem, float lr, f
 {
     const Member &m = mem[blockIdx.y];
     wait_for_previous();
+    let_next_start();
     int i = blockIdx.x * 256 + threadIdx.x;
     auto weights = [&](int l, int rows, int cols) {
         const float wi = adam_one(m.w[l], m.mw[l], m.vw[l], m.gw[l], i, lr, b1, b2, eps, c1, c2);
@@ -1015,23 +1012,6 @@ static int ensure_acts(sur_ctx *s, int M)
     s->extra_rows = M;
     s->group = group;
     return DPD_OK;
-}
-
-// Launch in programmatic order (see wait_for_previous).
-template <typename... P, typename... A>
-static void launch_step(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
-{
-    cudaLaunchConfig_t c{};
-    c.gridDim = grid;
-    c.blockDim = dim3(threads);
-    c.dynamicSmemBytes = smem;
-    c.stream = st;
-    cudaLaunchAttribute a{};
-    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    a.val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = &a;
-    c.numAttrs = 1;
-    cudaLaunchKernelEx(&c, kernel, args...);
 }
 
 // Forward pass of members [k, k + g) (g <= group) on the rows b; outputs in
