@@ -22,7 +22,6 @@ void launch_scatter(const Sys &d, int B, cudaStream_t st);
 int set_force_smem(int B, int var, int cap, int nt);
 int max_dynamic_smem();
 void launch_bin(const Sys &d, int B, cudaStream_t st);
-void launch_kick_bin(const Sys &d, int B, cudaStream_t st);
 int host_cell_of(int B, int nc, int cx, int cy);
 bool tuned_shape(const dpd_params *p, int R, int *tile, int *variant);
 constexpr size_t H_PIN_SMALL = 3584;   // bytes at the start of a context's page-locked buffer for small results
