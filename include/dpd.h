@@ -80,7 +80,7 @@ typedef struct dpd_params {
     int32_t exclude_bonded;/* 1 (paper): no pair force inside an agent       */
     int32_t noise;         /* 0: uniform alpha, 1: Gaussian alpha            */
     int32_t tile;          /* cell-block side in cells: 0 = default (by the
-                              number of blocks), else one of 4, 8, 16        */
+                              blocks' number and beads), else 4, 8 or 16     */
     int32_t variant;       /* pair-kernel variant: 0 = default (fastest),
                               1 = thread-per-bead, 2 = candidate masks and
                               pair queue, 3 = grid-order pair queue, 4 = flat

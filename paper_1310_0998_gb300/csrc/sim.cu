@@ -338,6 +338,17 @@ long long blocks_of(const dpd_params *p, int B)
     return nt * nt;
 }
 
+// A box alone on the chip: where 8 x 8 blocks leave SMs idle (152 or fewer of
+// them) and hold more than 64 beads, four times as many 4 x 4 blocks are each
+// done sooner (us a step with 4 x 4 / 8 x 8: 64 x 64 cells 13.7 / 17.0 at
+// density 3, 12.0 / 12.3 at 1.2, 12.3 / 12.2 at 0.8; 96 x 96 cells 15.3 / 18.2,
+// 12.7 / 12.9, 13.0 / 12.5; 128 x 128 cells, 256 blocks, 14.1 / 13.5 at 1.6).
+static int default_tile_alone(const dpd_params *p)
+{
+    if (blocks_of(p, 8) <= 152 && mean_owned(p, 8) > 64.0) return 4;
+    return default_tile(blocks_of(p, 16));
+}
+
 // Threads per tile: about two owned beads each where the blocks fill the chip
 // (16 x 16 blocks of 1024 x 1024 cells, us a step at 128 / 192 / 256 / 384
 // threads: 394 / 322 / 296 / 278 at density 3, 145 / 131 / 134 / 151 at 1.6,
@@ -653,7 +664,7 @@ int dpd_create(const dpd_params *p, void *stream, dpd_ctx **out)
     if (cudaGetDevice(&c->dev) != cudaSuccess) { delete c; return DPD_ERR_CUDA; }
     c->p = *p;
     c->var = p->variant ? p->variant : DEFAULT_VARIANT;
-    c->B = p->tile ? p->tile : c->var == DEFAULT_VARIANT ? default_tile(blocks_of(p, 16)) : DEFAULT_TILE;
+    c->B = p->tile ? p->tile : c->var == DEFAULT_VARIANT ? default_tile_alone(p) : DEFAULT_TILE;
     if (!p->tile && !p->variant) {
         int t = 0, v = 0;
         if (tuned_shape(p, 1, &t, &v)) { c->B = t; c->var = v; }
