@@ -207,7 +207,7 @@ def ensemble_leg(R, steps, warmup, seed=0, variant=0, tile=0, seq_steps=500):
     """C4: R replicas drawn from the uneven distribution (box side U(32, 192),
     area fraction U(0.05, 0.6), gamma log-U(0.5, 50), zeta log-U(0.005, 2),
     f_p U(0.5, 2)).  The kernel shape is tuned for this replica mix (unless
-    given), then `steps` steps of the batched persistent kernel are timed, and
+    given), then `steps` steps of the batched ensemble are timed, and
     `seq_steps` steps of every replica run alone through the single-system
     path (scaled to `steps`: the per-step cost of a replica is steady)."""
     import torch
@@ -251,8 +251,8 @@ def ensemble_leg(R, steps, warmup, seed=0, variant=0, tile=0, seq_steps=500):
            "batched_particle_steps_per_s": beads * steps / t_batch, "grid": info["grid"],
            "work_tiles": info["work_tiles"], "tile": shape.tile, "variant": shape.variant,
            "phases_ms_per_step": phases,
-           "timing": "wall clock around each synchronised leg; batched: the full step count in one persistent "
-                     "launch per call; sequential: each replica alone, one after another, for "
+           "timing": "wall clock around each synchronised leg; batched: the full step count in one "
+                     "call; sequential: each replica alone, one after another, for "
                      f"{seq_steps} steps, scaled to {steps}"}
     if tuning is not None:
         out["tuning"] = tuning
@@ -264,7 +264,7 @@ def sweep_leg(steps=20000, snaps=5, every=2000, M=128, seq_steps=2000, seed=0, s
     gamma {1, 4.5, 20} x zeta {0.01, 0.1, 1}, 54 points, f_p = 1), each point
     `steps` steps from the paper's initial condition with the FP64 E(k) on
     M^2 averaged over `snaps` snapshots `every` steps apart at the end of the
-    run.  Batched: all points in the persistent ensemble kernel (shape tuned
+    run.  Batched: all points in one ensemble (shape tuned
     for the mix).  Plain: every point alone through the single-system path,
     one after another (context creation, initial state, `seq_steps` steps
     scaled to `steps`, and all its snapshots, timed).  With a trained
@@ -327,7 +327,7 @@ def sweep_leg(steps=20000, snaps=5, every=2000, M=128, seq_steps=2000, seed=0, s
            "plain_s": t_seq, "plain_steps_timed_per_point": seq_steps,
            "speedup": t_seq / (t_setup + t_run), "tile": shape.tile, "variant": shape.variant,
            "spectra_finite": bool(np.all(np.isfinite(E)) and np.all(E > 0)), "tuning": tuning,
-           "timing": "wall clock; batched: set-up, then all steps in persistent launches of up to 1e4 steps and "
+           "timing": "wall clock; batched: set-up, then all steps in calls of up to 1e4 steps and "
                      "the E(k) of every point at each snapshot; plain: per point set-up, seq_steps steps scaled "
                      "to the full count, and every snapshot's E(k)"}
     if sur is not None:
