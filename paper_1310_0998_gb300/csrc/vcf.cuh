@@ -251,7 +251,7 @@ struct Pass {
 };
 
 constexpr int LIMB = 19;
-constexpr int FULL_AT = 4000;   // adds to a histogram word after which it is emptied (it holds 2^13)
+constexpr int FULL_AT = 4000;   // adds to a histogram word after which it is emptied (unsigned it holds 2^13)
 constexpr int QUEUE = 160;
 constexpr int RUN = 128;        // candidates between two looks at the counts: 32 x 128 adds at most
 
@@ -362,7 +362,9 @@ struct Warp {
             const int c = h[3 * nb + b];
             if (c == 0) continue;
             for (int w = 0; w < 3; ++w) {
-                atomicAdd((unsigned long long *)&p.gsum[w * nb + b], (unsigned long long)(long long)h[w * nb + b]);
+                // the low two limbs are never negative and fill their words to 2^32
+                const long long x = w < 2 ? (long long)(unsigned)h[w * nb + b] : (long long)h[w * nb + b];
+                atomicAdd((unsigned long long *)&p.gsum[w * nb + b], (unsigned long long)x);
                 h[w * nb + b] = 0;
             }
             atomicAdd(&p.gcnt[b], (unsigned long long)c);

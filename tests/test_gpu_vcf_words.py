@@ -1,0 +1,87 @@
+"""The velocity correlation's sums where its histogram words fill to their last
+bit: agents that move alike (every product has the same limbs) and slow opposed
+streams beside one fast agent (small negative products, whose low limbs are all
+ones), in one and two shells that take most pairs, with cells and without."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _state(D, L, na, seed):
+    """Agents with both beads at one place, on the grid L 2^-16."""
+    c = np.random.default_rng(seed).integers(0, 1 << 16, (na, D)) * (L / 65536.0)
+    return c, np.repeat(c, 2, axis=0)
+
+
+def _run(D, L, x, v, dr, nbins):
+    from paper_1310_0998_gb300 import Sim, Sim3
+    if D == 2:
+        with Sim(L, len(x), dt=1e-6) as s:
+            s.set_state(x, v, np.zeros_like(v))
+            return s.velocity_correlation(dr, nbins)
+    with Sim3(L, len(x), dt=1e-6, a=0.0, gamma=0.0, kBT=0.0, k_bond=0.0, f_p=0.0, zeta=0.0) as s:
+        s.set_positions(x, v)
+        return s.velocity_correlation(dr, nbins)
+
+
+def _pair_sums(c, v, L, dr, nbins):
+    """Counts and sums of v_a . v_b by shell, pair by pair (FP64, 80-bit sums)."""
+    num, cnt = np.zeros(nbins, np.longdouble), np.zeros(nbins, np.int64)
+    for a in range(len(c) - 1):
+        d = c[a] - c[a + 1:]
+        d -= L * np.rint(d / L)
+        b = np.floor(np.sqrt((d * d).sum(1)) / dr).astype(np.int64)
+        w = (v[a].astype(np.longdouble) * v[a + 1:]).sum(1)
+        for k in range(nbins):
+            m = b == k
+            cnt[k] += m.sum()
+            num[k] += w[m].sum()
+    return num, cnt
+
+
+@pytest.mark.parametrize("D,L,na,dr,nbins", [
+    (2, 32.0, 10000, 40.0, 1), (2, 32.0, 10000, 13.0, 2), (2, 32.0, 4096, 10.0, 1), (2, 32.0, 6000, 5.0, 2),
+    (3, 12.0, 10000, 16.0, 1), (3, 12.0, 4096, 4.0, 1)])
+def test_one_velocity(D, L, na, dr, nbins):
+    c, x = _state(D, L, na, na)
+    cnt0 = None
+    for u in ((0.3, 0.0, 0.1), (0.6, 0.8, 0.0), (1.1, 0.3, 0.7), (0.33, 0.81, 0.25), (-0.5, 0.0, 0.0)):
+        u = np.array(u[:D], np.float32)
+        v = np.tile(u, (2 * na, 1))
+        _, _, num, cnt = _run(D, L, x, v, dr, nbins)
+        if cnt0 is None:
+            cnt0 = cnt
+            if nbins == 1 and dr > L:
+                assert cnt[0] == na * (na - 1) // 2
+        np.testing.assert_array_equal(cnt, cnt0)
+        want = cnt * float((u.astype(np.float64) ** 2).sum())
+        # a product is good to 2^-48 of the largest, which it is here; a word that
+        # loses its top bit is off by 3e-5
+        np.testing.assert_allclose(num, want, rtol=2.0**-48)
+
+
+@pytest.mark.parametrize("D,L,na,dr,nbins", [(2, 32.0, 4096, 40.0, 1), (2, 32.0, 4096, 10.0, 1), (3, 12.0, 4096, 4.0, 1)])
+def test_crossing_streams(D, L, na, dr, nbins):
+    """Half of the products just below zero: a high limb of -1 over ones."""
+    c, x = _state(D, L, na, na + 2)
+    vc = np.zeros((na, D), np.float32)
+    vc[::2, 0] = 1.0
+    vc[1::2, :2] = (-2.0**-33, 1.0)
+    _, _, num, cnt = _run(D, L, x, np.repeat(vc, 2, axis=0), dr, nbins)
+    want, wcnt = _pair_sums(c, vc.astype(np.float64), L, dr, nbins)
+    np.testing.assert_array_equal(cnt, wcnt)
+    np.testing.assert_allclose(num, want.astype(np.float64), rtol=2.0**-48)
+
+
+@pytest.mark.parametrize("D,L,na,dr,nbins", [(2, 32.0, 4096, 40.0, 1), (2, 32.0, 4096, 10.0, 1), (3, 12.0, 4096, 4.0, 1)])
+def test_slow_opposed_streams_and_one_fast_agent(D, L, na, dr, nbins):
+    c, x = _state(D, L, na, na + 1)
+    vc = np.zeros((na, D), np.float32)
+    vc[:, 0] = np.where(np.arange(na) % 64 == 0, -2.0**-9, 2.0**-13)
+    vc[7] = 1.0
+    _, _, num, cnt = _run(D, L, x, np.repeat(vc, 2, axis=0), dr, nbins)
+    want, wcnt = _pair_sums(c, vc.astype(np.float64), L, dr, nbins)
+    np.testing.assert_array_equal(cnt, wcnt)
+    # the products are whole multiples of 2^-26, their sums below 2^53 of them: exact
+    np.testing.assert_array_equal(num, want.astype(np.float64))
