@@ -565,10 +565,14 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     p.id = (const int *)(buf + l.id);
     p.dr = dr;
     p.nbins = nbins;
-    // FP32 error of r / dr.  Cells: offsets up to 2.7 nbins from a corner, ten
-    // half-ulps of nbins a component, the square and its root: below 24 nbins
-    // 2^-24.  All pairs: the centres' 32 bits on top of three half-ulps.
-    p.mg = (float)(nbins * 2e-6 + 2e-6 + (n > 0 ? 0.0 : s.L / dr * std::ldexp(1.0, -31)));
+    // FP32 error of r / dr in half-ulps u = 2^-24.  Cells of side c (in dr): a
+    // component has 2 c u from each offset, (m + 1) c u from the shift and
+    // 2 nbins u from the difference and c's own rounding (m = 2: c is below 0.6
+    // nbins), the square and its root 4 nbins u: in all below 22 u max(nbins,
+    // 0.75 c).  Cells are wider than r_max where r_max is small beside the
+    // box.  All pairs: the centres' 32 bits on top of three half-ulps.
+    const double side = n > 0 ? s.L / n / dr : 0.0;
+    p.mg = (float)(std::max((double)nbins, 0.75 * side) * 2e-6 + 2e-6 + (n > 0 ? 0.0 : s.L / dr * std::ldexp(1.0, -31)));
     p.lim2 = ((float)nbins + p.mg) * ((float)nbins + p.mg) * 1.000001f;
     p.gsum = (long long *)(buf + l.gsum());
     p.gcnt = (unsigned long long *)(p.gsum + 3 * (size_t)nbins);
