@@ -11,11 +11,12 @@
 //               FP32 error, is queued, and full warps of queued pairs take the
 //               FP64 expressions of the definition: every pair's shell, and
 //               hence every count, is that of the FP64 evaluation.
-//   products    v = (V + r) / k with k a power of two by the fastest agent
-//               (|V| < 2^28, |r| <= 1/2): V_a . V_b is exact in 64 bits, the
-//               cross terms V_a . r_b + r_a . V_b are FP32, rounded to whole
-//               numbers (2^-53 of the largest product at most).
-//   sums        three 19-bit limbs of a product and the count go to the warp's
+//   products    v = (V + R 2^-32) / k, V and R whole numbers and k a power of
+//               two by the fastest agent (2^29 <= |V| < 2^30 there): a component
+//               is held to 2^-59 of the fastest speed.  v_a . v_b by 32 x 32 ->
+//               64 bit products in units k^-2, rounded once and without
+//               R_a . R_b: good to 2^-55 of the largest |v|^2.
+//   sums        three 21-bit limbs of a product and the count go to the warp's
 //               own histogram in shared memory by native 32-bit integer adds;
 //               it is emptied into 64-bit global sums before a word can
 //               overflow.  Whole-number sums do not depend on the order.
@@ -62,26 +63,27 @@ __device__ __forceinline__ Agent<D> load_agent(const State &s, int k)
     return g;
 }
 
-// log2 of the velocity scale k: |v| k < 2^28 for |v|^2 <= the value whose bits
-// are v2 (one bit spare for its rounding).
+// log2 of the velocity scale k: |v| k < 2^30 (1 + 2^-22) for the largest |v|^2,
+// whose FP32 value has the bits v2, and at least 2^29 there.
 __device__ __host__ __forceinline__ int scale_log2(uint32_t v2)
 {
     const int e = (int)(v2 >> 23) - 127;            // |v|^2 < 2^(e + 1)
-    const int h = e >= 0 ? e / 2 + 1 : -((-e) / 2) + 1;   // |v| < 2^h
-    const int x = 27 - h;
-    return v2 == 0u ? 0 : (x < -100 ? -100 : (x > 100 ? 100 : x));
+    return v2 == 0u ? 0 : 30 - ((e + 2) >> 1);      // |v| < 2^((e + 2) >> 1)
 }
 
-// V and r of one component from half the head and tail sum.
-__device__ __forceinline__ void split_v(float sh, float sl, float half_k, int &V, float &r)
+// V and R of one component from half the head and tail sum, R to a multiple of 4:
+// what sh k / 2 and sl k / 2 leave beside their nearest whole numbers is exact.
+__device__ __forceinline__ void split_v(float sh, float sl, float half_k, int &V, int &R)
 {
-    const float x = __fmul_rn(sh, half_k);
+    const float x = __fmul_rn(sh, half_k), z = __fmul_rn(sl, half_k), f = rintf(z);
     const int i = __float2int_rn(x);
-    const float y = __fadd_rn(__fsub_rn(x, (float)i), __fmul_rn(sl, half_k));
-    const float f = rintf(y);
-    V = i + (int)f;
-    r = __fsub_rn(y, f);
+    const int r = __float2int_rn(__fmul_rn(__fsub_rn(x, (float)i), 1073741824.0f)) +
+                  __float2int_rn(__fmul_rn(__fsub_rn(z, f), 1073741824.0f));
+    const int up = (r + (1 << 29)) >> 30;           // r - up 2^30 lies in [-2^29, 2^29)
+    V = i + (int)f + up;
+    R = (r - up * (1 << 30)) * 4;
 }
+constexpr long long HALF32 = 1ll << 31;   // rounds a following shift by 32
 
 template <int D>
 __global__ void __launch_bounds__(256) k_vcf_max(State s, unsigned *vmax)
@@ -107,8 +109,8 @@ __device__ __forceinline__ int cell_of(const Agent<D> &g, int n)
     return f;
 }
 
-// Sums over the agents (sum V, sum 2^20 r per component; V^2 in two 32-bit
-// halves and r (2 V + r)) and, with cells (n > 0), each agent's rank in its cell.
+// Sums over the agents (sum V, sum R per component; V^2 in two 32-bit halves and
+// the rest of |v|^2) and, with cells (n > 0), each agent's rank in its cell.
 template <int D>
 __global__ void __launch_bounds__(256) k_vcf_count(State s, int n, const unsigned *vmax, unsigned *cnt, unsigned *rank,
                                                    long long *sums)
@@ -122,20 +124,19 @@ __global__ void __launch_bounds__(256) k_vcf_count(State s, int n, const unsigne
         const Agent<D> g = load_agent<D>(s, k);
         if (n > 0) rank[k] = atomicAdd(&cnt[cell_of<D>(g, n)], 1u);
         unsigned long long q = 0;
-        float er = 0.f;
+        long long er = HALF32;   // 2^-32
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            int V;
-            float r;
-            split_v(g.sh[i], g.sl[i], half_k, V, r);
+            int V, R;
+            split_v(g.sh[i], g.sl[i], half_k, V, R);
             a[2 * i] += V;
-            a[2 * i + 1] += __float2int_rn(r * 1048576.0f);
+            a[2 * i + 1] += R;
             q += (unsigned long long)((long long)V * V);
-            er = fmaf(r, fmaf(2.0f, (float)V, r), er);
+            er += 2 * (long long)V * R + __mulhi(R, R);
         }
         a[2 * D] += (long long)(q & 0xffffffffull);
         a[2 * D + 1] += (long long)(q >> 32);
-        a[2 * D + 2] += __float2int_rn(er);
+        a[2 * D + 2] += er >> 32;
     }
     __shared__ long long red[8][NS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -154,12 +155,12 @@ __global__ void __launch_bounds__(256) k_vcf_count(State s, int n, const unsigne
 }
 
 // Agents in cell order (n > 0: offset from the cell's corner in units of dr) or
-// as they come (n = 0: 32-bit centre of mass): P, Q = (Vx, Vy, rx, ry) or
-// (Vx, Vy, Vz, rz) with R = (rx, ry), and the agent's id.
+// as they come (n = 0: 32-bit centre of mass): P, Q = (Vx, Vy, Rx, Ry) or
+// (Vx, Vy, Vz, Rz) with R = (Rx, Ry), and the agent's id.
 template <int D>
 __global__ void __launch_bounds__(256) k_vcf_place(State s, int n, float cell_dr, const unsigned *vmax,
                                                    const unsigned *start, const unsigned *rank, float4 *P, int4 *Q,
-                                                   float2 *R, int *id)
+                                                   int2 *R, int *id)
 {
     const int k = blockIdx.x * 256 + threadIdx.x;
     if (k >= s.na) return;
@@ -168,8 +169,8 @@ __global__ void __launch_bounds__(256) k_vcf_place(State s, int n, float cell_dr
     unsigned dst = (unsigned)k;
     if (n > 0) dst = start[cell_of<D>(g, n)] + rank[k];
     if (dst >= (unsigned)s.na) return;
-    float p[3] = {0.f, 0.f, 0.f}, r[3] = {0.f, 0.f, 0.f};
-    int v[3] = {0, 0, 0};
+    float p[3] = {0.f, 0.f, 0.f};
+    int v[3] = {0, 0, 0}, r[3] = {0, 0, 0};
 #pragma unroll
     for (int i = 0; i < D; ++i) {
         if (n > 0) {
@@ -182,10 +183,10 @@ __global__ void __launch_bounds__(256) k_vcf_place(State s, int n, float cell_dr
     }
     P[dst] = make_float4(p[0], p[1], p[2], 0.f);
     if constexpr (D == 2) {
-        Q[dst] = make_int4(v[0], v[1], __float_as_int(r[0]), __float_as_int(r[1]));
+        Q[dst] = make_int4(v[0], v[1], r[0], r[1]);
     } else {
-        Q[dst] = make_int4(v[0], v[1], v[2], __float_as_int(r[2]));
-        R[dst] = make_float2(r[0], r[1]);
+        Q[dst] = make_int4(v[0], v[1], v[2], r[2]);
+        R[dst] = make_int2(r[0], r[1]);
     }
     id[dst] = k;
 }
@@ -241,7 +242,7 @@ struct Pass {
     State s;
     const float4 *P;
     const int4 *Q;
-    const float2 *R;
+    const int2 *R;
     const int *id;
     double dr;
     int nbins;
@@ -250,10 +251,12 @@ struct Pass {
     unsigned long long *gcnt;  // [nbins]
 };
 
-constexpr int LIMB = 19;
-constexpr int FULL_AT = 4000;   // adds to a histogram word after which it is emptied (unsigned it holds 2^13)
+constexpr int LIMB = 21;        // a histogram word takes 2^11 adds of a limb (the high one: of 2^18 in magnitude)
 constexpr int QUEUE = 160;
-constexpr int RUN = 128;        // candidates between two looks at the counts: 32 x 128 adds at most
+// Candidates (32 adds each at most) until the counts are looked at again, where
+// the largest is `most`; fewer than 32 pairs wait in the queue.
+__device__ __forceinline__ int room_after(int most) { return ((1 << 11) - 32 - most) / 32 & ~3; }
+constexpr int FULL_AT = 992;    // count from which the histogram is emptied at a look: room for 60 then, for 32 below
 
 template <int D>
 struct Warp {
@@ -262,12 +265,12 @@ struct Warp {
     uint2 *q;          // queued pairs near a shell edge (QUEUE: 31 and four candidates of 32 lanes)
     int qn, lane;
     int a;             // the lane's agent, -1 for none
+    int room;          // candidates until the next look at the counts
     float x[D];
-    struct Vel { int V[D]; float r[D]; } va;
-    float Fa[D];
+    struct Vel { int V[D], R[D]; } va;
 
     __device__ Warp(const Pass &pass, int *hist, uint2 *queue)
-        : p(pass), h(hist), q(queue), qn(0), lane(threadIdx.x & 31), a(-1)
+        : p(pass), h(hist), q(queue), qn(0), lane(threadIdx.x & 31), a(-1), room(room_after(0))
     {
         for (int i = lane; i < 4 * p.nbins; i += 32) h[i] = 0;
         __syncwarp();
@@ -279,14 +282,14 @@ struct Warp {
         v.V[0] = q.x;
         v.V[1] = q.y;
         if constexpr (D == 2) {
-            v.r[0] = __int_as_float(q.z);
-            v.r[1] = __int_as_float(q.w);
+            v.R[0] = q.z;
+            v.R[1] = q.w;
         } else {
-            const float2 r = p.R[b];
+            const int2 r = p.R[b];
             v.V[2] = q.z;
-            v.r[0] = r.x;
-            v.r[1] = r.y;
-            v.r[2] = __int_as_float(q.w);
+            v.R[0] = r.x;
+            v.R[1] = r.y;
+            v.R[2] = q.w;
         }
         return v;
     }
@@ -297,7 +300,7 @@ struct Warp {
         const float px[3] = {P.x, P.y, P.z};
         va = vel(max(a, 0));
 #pragma unroll
-        for (int i = 0; i < D; ++i) { x[i] = px[i]; Fa[i] = (float)va.V[i]; }
+        for (int i = 0; i < D; ++i) x[i] = px[i];
     }
     __device__ __forceinline__ void add(int bin, long long d)
     {
@@ -307,18 +310,18 @@ struct Warp {
         atomicAdd(w + 2 * p.nbins, (int)(d >> (2 * LIMB)));
         atomicAdd(w + 3 * p.nbins, 1);
     }
-    // v . w in units k^-2 (the product of the rests, below one unit, is left out).
-    static __device__ __forceinline__ long long dot(const Vel &v, const float *F, const Vel &w)
+    // v . w in units k^-2: the whole parts' product, and the cross terms (below
+    // 2^63: |V| < 2^30 and |R| <= 3^1/2 2^31) rounded.
+    static __device__ __forceinline__ long long dot(const Vel &v, const Vel &w)
     {
-        long long d = 0;
-        float c = 0.f;
+        long long d = 0, c = HALF32;
 #pragma unroll
         for (int i = 0; i < D; ++i) {
             d += (long long)v.V[i] * w.V[i];
-            c = fmaf(F[i], w.r[i], c);
-            c = fmaf(v.r[i], (float)w.V[i], c);
+            c += (long long)v.V[i] * w.R[i];
+            c += (long long)v.R[i] * w.V[i];
         }
-        return d + __float2int_rn(c);
+        return d + (c >> 32);
     }
     __device__ __forceinline__ void com(int id, double *c) const
     {
@@ -345,10 +348,7 @@ struct Warp {
             const double rmax2 = (double)p.nbins * p.dr * (double)p.nbins * p.dr * (1.0 + 1e-9);
             const double bf = floor(__ddiv_rn(sqrt(r2), p.dr));
             if (r2 < rmax2 && bf < (double)p.nbins) {
-                const Vel v = vel((int)e.x);
-                float F[D];
-                for (int i = 0; i < D; ++i) F[i] = (float)v.V[i];
-                add((int)bf, dot(v, F, vel((int)e.y)));
+                add((int)bf, dot(vel((int)e.x), vel((int)e.y)));
             }
         }
         qn = first;
@@ -387,7 +387,8 @@ struct Warp {
         }
         const float lim2 = a >= 0 ? p.lim2 : -1.0f, inside = 0.5f - p.mg, last = (float)p.nbins - p.mg;
         while (s < e) {
-            const int stop = min(e, s + RUN);
+            const int stop = min(e, s + room);
+            room -= (stop - s + 3) & ~3;
             for (; s < stop; s += 4) {
                 unsigned near = 0u;   // candidates whose shell FP32 does not decide
                 float t2[4];
@@ -411,7 +412,7 @@ struct Warp {
                         asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(t2[u]));
                         // the shell's middle nearest to t
                         const float w = t - 0.5f, z = w + M;
-                        if ((fabsf(w - (z - M)) < inside) & (t < last)) add(__float_as_int(z) - 0x4B400000, dot(va, Fa, vel(b)));
+                        if ((fabsf(w - (z - M)) < inside) & (t < last)) add(__float_as_int(z) - 0x4B400000, dot(va, vel(b)));
                         else near |= 1u << u;
                     }
                 }
@@ -426,10 +427,16 @@ struct Warp {
                     while (qn >= 32) drain();
                 }
             }
+            if (room > 0) continue;
             __syncwarp();
             int most = 0;
             for (int b = lane; b < p.nbins; b += 32) most = max(most, h[3 * p.nbins + b]);
-            if (__any_sync(0xffffffffu, most >= FULL_AT)) flush();
+            most = __reduce_max_sync(0xffffffffu, most);
+            if (most >= FULL_AT) {
+                flush();
+                most = 0;
+            }
+            room = room_after(most);
         }
     }
     __device__ __forceinline__ void finish()
@@ -561,7 +568,7 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     p.s = s;
     p.P = (const float4 *)(buf + l.P);
     p.Q = (const int4 *)(buf + l.Q);
-    p.R = (const float2 *)(buf + l.R);
+    p.R = (const int2 *)(buf + l.R);
     p.id = (const int *)(buf + l.id);
     p.dr = dr;
     p.nbins = nbins;
@@ -586,7 +593,7 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     k_vcf_max<D><<<g, 256, 0, st>>>(s, vmax);
     k_vcf_count<D><<<g, 256, 0, st>>>(s, n, vmax, cnt, rank, sums);
     if (n > 0) k_vcf_scan<<<1, 1024, 0, st>>>(cnt, (int)ncell, start);
-    k_vcf_place<D><<<gp, 256, 0, st>>>(s, n, cell_dr, vmax, start, rank, (float4 *)p.P, (int4 *)p.Q, (float2 *)p.R, (int *)p.id);
+    k_vcf_place<D><<<gp, 256, 0, st>>>(s, n, cell_dr, vmax, start, rank, (float4 *)p.P, (int4 *)p.Q, (int2 *)p.R, (int *)p.id);
     // warps per block: four, or one where the histograms are large
     const int wpb = warp_smem(nbins) * 4 <= 96 * 1024 ? 4 : 1;
     const size_t sm = warp_smem(nbins) * wpb;
@@ -623,7 +630,7 @@ static Out vcf_finish(const std::vector<long long> &host, int na, int nbins)
     const int k = scale_log2(vmax);
     const long long *s = host.data() + 8, *g = host.data() + 32;
     for (int i = 0; i < 3; ++i)
-        o.mean[i] = i < D ? std::ldexp((double)s[2 * i] + std::ldexp((double)s[2 * i + 1], -20), -k) / na : 0.0;
+        o.mean[i] = i < D ? std::ldexp((double)s[2 * i] + std::ldexp((double)s[2 * i + 1], -32), -k) / na : 0.0;
     const __int128 q = ((__int128)s[2 * D + 1] << 32) + s[2 * D] + s[2 * D + 2];
     o.v2 = std::ldexp((double)q, -2 * k) / na;
     o.num.resize(nbins);

@@ -1,7 +1,8 @@
 """The velocity correlation's sums where its histogram words fill to their last
 bit: agents that move alike (every product has the same limbs) and slow opposed
 streams beside one fast agent (small negative products, whose low limbs are all
-ones), in one and two shells that take most pairs, with cells and without."""
+ones), in one and two shells that take most pairs, with cells and without; and
+the accuracy of single products, in shells of few pairs."""
 import numpy as np
 import pytest
 
@@ -14,13 +15,13 @@ def _state(D, L, na, seed):
     return c, np.repeat(c, 2, axis=0)
 
 
-def _run(D, L, x, v, dr, nbins):
+def _run(D, L, x, v, dr, nbins, dt=1e-6):
     from paper_1310_0998_gb300 import Sim, Sim3
     if D == 2:
-        with Sim(L, len(x), dt=1e-6) as s:
+        with Sim(L, len(x), dt=dt) as s:
             s.set_state(x, v, np.zeros_like(v))
             return s.velocity_correlation(dr, nbins)
-    with Sim3(L, len(x), dt=1e-6, a=0.0, gamma=0.0, kBT=0.0, k_bond=0.0, f_p=0.0, zeta=0.0) as s:
+    with Sim3(L, len(x), dt=dt, a=0.0, gamma=0.0, kBT=0.0, k_bond=0.0, f_p=0.0, zeta=0.0) as s:
         s.set_positions(x, v)
         return s.velocity_correlation(dr, nbins)
 
@@ -85,3 +86,25 @@ def test_slow_opposed_streams_and_one_fast_agent(D, L, na, dr, nbins):
     np.testing.assert_array_equal(cnt, wcnt)
     # the products are whole multiples of 2^-26, their sums below 2^53 of them: exact
     np.testing.assert_array_equal(num, want.astype(np.float64))
+
+
+@pytest.mark.parametrize("D,L,na,dr,nbins", [(2, 32.0, 300, 16.0 / 4000, 4000), (2, 32.0, 1000, 8.0 / 2500, 2500), (2, 48.0, 40, 0.02, 600),
+                                             (3, 12.0, 300, 0.002, 3000), (3, 12.0, 700, 4.0 / 2000, 2000)])
+@pytest.mark.parametrize("kind", ["alike", "head"])
+def test_products(D, L, na, dr, nbins, kind):
+    """Shells of a pair or two.  kind "head": the tail's velocity 2^-1 to 2^-24 of
+    the head's, so that their sum needs more bits than FP32 has."""
+    c, x = _state(D, L, na, na + 3)
+    rng = np.random.default_rng(na)
+    v = rng.standard_normal((2 * na, D)).astype(np.float32)
+    if kind == "head":
+        v[1::2] *= np.exp2(-rng.integers(1, 25, (na, 1))).astype(np.float32)
+    _, _, num, cnt = _run(D, L, x, v, dr, nbins)
+    vc = 0.5 * (v[0::2].astype(np.longdouble) + v[1::2].astype(np.longdouble))
+    want, wcnt = _pair_sums(c, vc, L, dr, nbins)
+    np.testing.assert_array_equal(cnt, wcnt)
+    assert (cnt == 1).any()
+    # a product is good to 2^-55 of the largest |v|^2 at least; the result is rounded to FP64
+    v2 = (vc * vc).sum(1).max()
+    err = np.abs(num - want)
+    assert np.all(err <= cnt * 2.0**-55 * v2 + 2.0**-53 * np.abs(want)), float(err.max())
