@@ -15,7 +15,10 @@
 //               two by the fastest agent (2^29 <= |V| < 2^30 there): a component
 //               is held to 2^-59 of the fastest speed.  v_a . v_b by 32 x 32 ->
 //               64 bit products in units k^-2, rounded once and without
-//               R_a . R_b: good to 2^-55 of the largest |v|^2.
+//               R_a . R_b: good to 2^-55 of the largest |v|^2.  Where the
+//               fastest agent's |v|^2 is no FP32 number, or the mean |v|^2 lies
+//               so far below it (256 to 1024 times) that FP64 products would be
+//               the better ones, the same pass takes those, with FP64 sums.
 //   sums        three 21-bit limbs of a product and the count go to the warp's
 //               own histogram in shared memory by native 32-bit integer adds;
 //               it is emptied into 64-bit global sums before a word can
@@ -30,6 +33,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -84,6 +89,15 @@ __device__ __forceinline__ void split_v(float sh, float sl, float half_k, int &V
     R = (r - up * (1 << 30)) * 4;
 }
 constexpr long long HALF32 = 1ll << 31;   // rounds a following shift by 32
+
+// Whether the pass takes FP64 products: |v|^2 of the fastest agent (bits v2) zero,
+// denormal or infinite, or the mean V^2 below 2^52 (sums: as k_vcf_count's).
+template <int D>
+__device__ __host__ __forceinline__ bool wide_speeds(uint32_t v2, const long long *sums, int na)
+{
+    const uint32_t e = v2 >> 23;
+    return e == 0u || e == 255u || sums[2 * D + 1] + (sums[2 * D] >> 32) < ((long long)na << 20);
+}
 
 template <int D>
 __global__ void __launch_bounds__(256) k_vcf_max(State s, unsigned *vmax)
@@ -156,13 +170,30 @@ __global__ void __launch_bounds__(256) k_vcf_count(State s, int n, const unsigne
 
 // Agents in cell order (n > 0: offset from the cell's corner in units of dr) or
 // as they come (n = 0: 32-bit centre of mass): P, Q = (Vx, Vy, Rx, Ry) or
-// (Vx, Vy, Vz, Rz) with R = (Rx, Ry), and the agent's id.
+// (Vx, Vy, Vz, Rz) with R = (Rx, Ry), and the agent's id.  For FP64 products: Q
+// (and R) hold v, and wsum gets the sums of v (three) and |v|^2.
 template <int D>
 __global__ void __launch_bounds__(256) k_vcf_place(State s, int n, float cell_dr, const unsigned *vmax,
-                                                   const unsigned *start, const unsigned *rank, float4 *P, int4 *Q,
-                                                   int2 *R, int *id)
+                                                   const long long *sums, const unsigned *start, const unsigned *rank,
+                                                   float4 *P, int4 *Q, int2 *R, int *id, double *wsum)
 {
     const int k = blockIdx.x * 256 + threadIdx.x;
+    const bool wide = wide_speeds<D>(*vmax, sums, s.na);
+    double w[4] = {0.0, 0.0, 0.0, 0.0};
+    if (wide) {
+        if (k < s.na) {
+            const AgentBeads<D> g = load_beads<D>(s, k);
+            for (int i = 0; i < D; ++i) {
+                w[i] = __dmul_rn(0.5, __dadd_rn((double)g.hv[i], (double)g.tv[i]));
+                w[3] = fma(w[i], w[i], w[3]);
+            }
+        }
+        for (int i = 0; i < 4; ++i) {
+            double t = w[i];
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if ((threadIdx.x & 31) == 0) atomicAdd(&wsum[i], t);
+        }
+    }
     if (k >= s.na) return;
     const float half_k = __int_as_float((127 + scale_log2(*vmax) - 1) << 23);
     const Agent<D> g = load_agent<D>(s, k);
@@ -182,7 +213,10 @@ __global__ void __launch_bounds__(256) k_vcf_place(State s, int n, float cell_dr
         split_v(g.sh[i], g.sl[i], half_k, v[i], r[i]);
     }
     P[dst] = make_float4(p[0], p[1], p[2], 0.f);
-    if constexpr (D == 2) {
+    if (wide) {
+        reinterpret_cast<double2 *>(Q)[dst] = make_double2(w[0], w[1]);
+        if constexpr (D == 3) reinterpret_cast<double *>(R)[dst] = w[2];
+    } else if constexpr (D == 2) {
         Q[dst] = make_int4(v[0], v[1], r[0], r[1]);
     } else {
         Q[dst] = make_int4(v[0], v[1], v[2], r[2]);
@@ -246,8 +280,10 @@ struct Pass {
     const int *id;
     double dr;
     int nbins;
+    const unsigned *vmax;      // what wide_speeds takes
+    const long long *sums;
     float lim2, mg;            // (nbins + mg)^2, and the distance from a shell edge that FP32 decides
-    long long *gsum;           // [3][nbins] limb sums
+    long long *gsum;           // [3][nbins] limb sums (FP64 products: [nbins] doubles)
     unsigned long long *gcnt;  // [nbins]
 };
 
@@ -258,7 +294,9 @@ constexpr int QUEUE = 160;
 __device__ __forceinline__ int room_after(int most) { return ((1 << 11) - 32 - most) / 32 & ~3; }
 constexpr int FULL_AT = 992;    // count from which the histogram is emptied at a look: room for 60 then, for 32 below
 
-template <int D>
+// (WIDE: FP64 products and sums; the histogram is nbins doubles, and the counts
+// where they are otherwise.)
+template <int D, bool WIDE>
 struct Warp {
     const Pass &p;
     int *h;            // [4][nbins]: low, middle, high limb, count (this warp's)
@@ -267,7 +305,10 @@ struct Warp {
     int a;             // the lane's agent, -1 for none
     int room;          // candidates until the next look at the counts
     float x[D];
-    struct Vel { int V[D], R[D]; } va;
+    struct Whole { int V[D], R[D]; };
+    struct Real { double v[D]; };
+    using Vel = std::conditional_t<WIDE, Real, Whole>;
+    Vel va;
 
     __device__ Warp(const Pass &pass, int *hist, uint2 *queue)
         : p(pass), h(hist), q(queue), qn(0), lane(threadIdx.x & 31), a(-1), room(room_after(0))
@@ -277,21 +318,29 @@ struct Warp {
     }
     __device__ __forceinline__ Vel vel(int b) const
     {
-        const int4 q = p.Q[b];
         Vel v;
-        v.V[0] = q.x;
-        v.V[1] = q.y;
-        if constexpr (D == 2) {
-            v.R[0] = q.z;
-            v.R[1] = q.w;
+        if constexpr (WIDE) {
+            const double2 q = reinterpret_cast<const double2 *>(p.Q)[b];
+            v.v[0] = q.x;
+            v.v[1] = q.y;
+            if constexpr (D == 3) v.v[2] = reinterpret_cast<const double *>(p.R)[b];
+            return v;
         } else {
-            const int2 r = p.R[b];
-            v.V[2] = q.z;
-            v.R[0] = r.x;
-            v.R[1] = r.y;
-            v.R[2] = q.w;
+            const int4 q = p.Q[b];
+            v.V[0] = q.x;
+            v.V[1] = q.y;
+            if constexpr (D == 2) {
+                v.R[0] = q.z;
+                v.R[1] = q.w;
+            } else {
+                const int2 r = p.R[b];
+                v.V[2] = q.z;
+                v.R[0] = r.x;
+                v.R[1] = r.y;
+                v.R[2] = q.w;
+            }
+            return v;
         }
-        return v;
     }
     __device__ __forceinline__ void load(int k, int end)
     {
@@ -301,6 +350,11 @@ struct Warp {
         va = vel(max(a, 0));
 #pragma unroll
         for (int i = 0; i < D; ++i) x[i] = px[i];
+    }
+    __device__ __forceinline__ void add(int bin, double d)
+    {
+        atomicAdd(reinterpret_cast<double *>(h) + bin, d);
+        atomicAdd(h + 3 * p.nbins + bin, 1);
     }
     __device__ __forceinline__ void add(int bin, long long d)
     {
@@ -312,7 +366,13 @@ struct Warp {
     }
     // v . w in units k^-2: the whole parts' product, and the cross terms (below
     // 2^63: |V| < 2^30 and |R| <= 3^1/2 2^31) rounded.
-    static __device__ __forceinline__ long long dot(const Vel &v, const Vel &w)
+    static __device__ __forceinline__ double dot(const Real &v, const Real &w)
+    {
+        double d = __dadd_rn(__dmul_rn(v.v[0], w.v[0]), __dmul_rn(v.v[1], w.v[1]));
+        if constexpr (D == 3) d = __dadd_rn(d, __dmul_rn(v.v[2], w.v[2]));
+        return d;
+    }
+    static __device__ __forceinline__ long long dot(const Whole &v, const Whole &w)
     {
         long long d = 0, c = HALF32;
 #pragma unroll
@@ -361,11 +421,17 @@ struct Warp {
         for (int b = lane; b < nb; b += 32) {
             const int c = h[3 * nb + b];
             if (c == 0) continue;
-            for (int w = 0; w < 3; ++w) {
-                // the low two limbs are never negative and fill their words to 2^32
-                const long long x = w < 2 ? (long long)(unsigned)h[w * nb + b] : (long long)h[w * nb + b];
-                atomicAdd((unsigned long long *)&p.gsum[w * nb + b], (unsigned long long)x);
-                h[w * nb + b] = 0;
+            if constexpr (WIDE) {
+                double *sum = reinterpret_cast<double *>(h) + b;
+                atomicAdd(reinterpret_cast<double *>(p.gsum) + b, *sum);
+                *sum = 0.0;
+            } else {
+                for (int w = 0; w < 3; ++w) {
+                    // the low two limbs are never negative and fill their words to 2^32
+                    const long long x = w < 2 ? (long long)(unsigned)h[w * nb + b] : (long long)h[w * nb + b];
+                    atomicAdd((unsigned long long *)&p.gsum[w * nb + b], (unsigned long long)x);
+                    h[w * nb + b] = 0;
+                }
             }
             atomicAdd(&p.gcnt[b], (unsigned long long)c);
             h[3 * nb + b] = 0;
@@ -451,13 +517,13 @@ __host__ __device__ inline size_t warp_smem(int nbins) { return (size_t)nbins * 
 // Cells: task (cell, row of neighbour cells), rows 0 .. of the forward half
 // stencil of m cells each way (row 0: the own cell and those east of it), taken
 // from a counter.
-template <int D>
-__global__ void __launch_bounds__(128) k_vcf_cells(Pass p, const unsigned *start, int n, int m, int rows, int tasks,
-                                                   float cell_dr, unsigned *next)
+template <int D, bool WIDE>
+__device__ __forceinline__ void cells_pass(const Pass &p, const unsigned *start, int n, int m, int rows, int tasks,
+                                           float cell_dr, unsigned *next)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char *mine = smem + warp_smem(p.nbins) * (threadIdx.x >> 5);
-    Warp<D> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
+    Warp<D, WIDE> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
     while (true) {
         unsigned t = 0;
         if (w.lane == 0) t = atomicAdd(next, 1u);
@@ -486,20 +552,44 @@ __global__ void __launch_bounds__(128) k_vcf_cells(Pass p, const unsigned *start
     }
     w.finish();
 }
+template <int D>
+__device__ __noinline__ void cells_pass_wide(const Pass &p, const unsigned *start, int n, int m, int rows, int tasks,
+                                             float cell_dr, unsigned *next)
+{
+    cells_pass<D, true>(p, start, n, m, rows, tasks, cell_dr, next);
+}
+template <int D>
+__global__ void __launch_bounds__(128) k_vcf_cells(const __grid_constant__ Pass p, const unsigned *start, int n, int m,
+                                                   int rows, int tasks, float cell_dr, unsigned *next)
+{
+    if (wide_speeds<D>(*p.vmax, p.sums, p.s.na)) cells_pass_wide<D>(p, start, n, m, rows, tasks, cell_dr, next);
+    else cells_pass<D, false>(p, start, n, m, rows, tasks, cell_dr, next);
+}
 
 // All pairs: a warp's 32 agents against a stretch of `cols` agents after them.
-template <int D>
-__global__ void __launch_bounds__(128) k_vcf_all(Pass p, int cols, float unit)
+template <int D, bool WIDE>
+__device__ __forceinline__ void all_pass(const Pass &p, int cols, float unit)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int a0 = ((int)blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5)) * 32;
     const int s = max(a0, (int)blockIdx.y * cols), e = min(p.s.na, ((int)blockIdx.y + 1) * cols);
     if (a0 >= p.s.na || s >= e) return;   // a whole warp at a time; no block barrier below
     unsigned char *mine = smem + warp_smem(p.nbins) * (threadIdx.x >> 5);
-    Warp<D> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
+    Warp<D, WIDE> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
     w.load(a0 + w.lane, p.s.na);
     w.template run<true>(s, e, nullptr, w.a, unit);
     w.finish();
+}
+template <int D>
+__device__ __noinline__ void all_pass_wide(const Pass &p, int cols, float unit)
+{
+    all_pass<D, true>(p, cols, unit);
+}
+template <int D>
+__global__ void __launch_bounds__(128) k_vcf_all(const __grid_constant__ Pass p, int cols, float unit)
+{
+    if (wide_speeds<D>(*p.vmax, p.sums, p.s.na)) all_pass_wide<D>(p, cols, unit);
+    else all_pass<D, false>(p, cols, unit);
 }
 
 // Host results of a pass.
@@ -522,11 +612,12 @@ struct Layout {
         rank = up(id + 4 * na);
         start = up(rank + (ncell ? 4 * na : 0));
         zero = up(start + 4 * (ncell + 1));
-        words = zero;                    // [0] vmax, [1] task counter, then 16 sums, then the shell sums
+        words = zero;                    // [0] vmax, [1] task counter, 16 whole-number sums, 4 FP64 ones, the shell sums
         cnt = up(gsum() + 8 * 4 * nbins);   // cell counts
         bytes = cnt + 4 * ncell;
     }
     size_t sums() const { return words + 64; }
+    size_t wsum() const { return words + 192; }
     size_t gsum() const { return words + 256; }
 };
 // 64-bit words of a pass's results (from Layout::words on).
@@ -572,6 +663,8 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     p.id = (const int *)(buf + l.id);
     p.dr = dr;
     p.nbins = nbins;
+    p.vmax = vmax;
+    p.sums = sums;
     // FP32 error of r / dr in half-ulps u = 2^-24.  Cells of side c (in dr): a
     // component has 2 c u from each offset, (m + 1) c u from the shift and
     // 2 nbins u from the difference and c's own rounding (m = 2: c is below 0.6
@@ -593,7 +686,8 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     k_vcf_max<D><<<g, 256, 0, st>>>(s, vmax);
     k_vcf_count<D><<<g, 256, 0, st>>>(s, n, vmax, cnt, rank, sums);
     if (n > 0) k_vcf_scan<<<1, 1024, 0, st>>>(cnt, (int)ncell, start);
-    k_vcf_place<D><<<gp, 256, 0, st>>>(s, n, cell_dr, vmax, start, rank, (float4 *)p.P, (int4 *)p.Q, (int2 *)p.R, (int *)p.id);
+    k_vcf_place<D><<<gp, 256, 0, st>>>(s, n, cell_dr, vmax, sums, start, rank, (float4 *)p.P, (int4 *)p.Q, (int2 *)p.R, (int *)p.id,
+                                     (double *)(buf + l.wsum()));
     // warps per block: four, or one where the histograms are large
     const int wpb = warp_smem(nbins) * 4 <= 96 * 1024 ? 4 : 1;
     const size_t sm = warp_smem(nbins) * wpb;
@@ -629,16 +723,24 @@ static Out vcf_finish(const std::vector<long long> &host, int na, int nbins)
     const uint32_t vmax = (uint32_t)((unsigned long long)host[0] & 0xffffffffull);
     const int k = scale_log2(vmax);
     const long long *s = host.data() + 8, *g = host.data() + 32;
+    o.num.resize(nbins);
+    o.cnt.resize(nbins);
+    for (int b = 0; b < nbins; ++b) o.cnt[b] = (unsigned long long)g[3 * nbins + b];
+    if (wide_speeds<D>(vmax, s, na)) {
+        double w[4];
+        std::memcpy(w, host.data() + 24, sizeof w);
+        for (int i = 0; i < 3; ++i) o.mean[i] = w[i] / na;
+        o.v2 = w[3] / na;
+        std::memcpy(o.num.data(), g, 8 * (size_t)nbins);
+        return o;
+    }
     for (int i = 0; i < 3; ++i)
         o.mean[i] = i < D ? std::ldexp((double)s[2 * i] + std::ldexp((double)s[2 * i + 1], -32), -k) / na : 0.0;
     const __int128 q = ((__int128)s[2 * D + 1] << 32) + s[2 * D] + s[2 * D + 2];
     o.v2 = std::ldexp((double)q, -2 * k) / na;
-    o.num.resize(nbins);
-    o.cnt.resize(nbins);
     for (int b = 0; b < nbins; ++b) {
         const __int128 t = ((__int128)g[2 * nbins + b] << (2 * LIMB)) + ((__int128)g[nbins + b] << LIMB) + g[b];
         o.num[b] = std::ldexp((double)t, -2 * k);
-        o.cnt[b] = (unsigned long long)g[3 * nbins + b];
     }
     return o;
 }

@@ -108,3 +108,28 @@ def test_products(D, L, na, dr, nbins, kind):
     v2 = (vc * vc).sum(1).max()
     err = np.abs(num - want)
     assert np.all(err <= cnt * 2.0**-55 * v2 + 2.0**-53 * np.abs(want)), float(err.max())
+
+
+@pytest.mark.parametrize("D,L,na,dr,nbins", [(2, 32.0, 500, 16.0 / 100, 100), (2, 32.0, 2000, 8.0 / 30, 30), (3, 12.0, 500, 0.06, 100),
+                                             (3, 12.0, 2000, 4.0 / 20, 20), (2, 32.0, 2000, 40.0, 1)])
+@pytest.mark.parametrize("scale", [1.0, 1e-30, 1e25])
+def test_wide_speeds(D, L, na, dr, nbins, scale):
+    """One agent 2^12 times faster than the rest, and speeds whose squares are no
+    FP32 numbers: every product, the mean and the mean square to FP64."""
+    c, x = _state(D, L, na, na + 4)
+    v = np.random.default_rng(na).standard_normal((2 * na, D))
+    v[10:12] *= 4096.0
+    v = (v * scale).astype(np.float32)
+    g, _, num, cnt = _run(D, L, x, v, dr, nbins, dt=1e-35)
+    vc = 0.5 * (v[0::2].astype(np.longdouble) + v[1::2].astype(np.longdouble))
+    want, wcnt = _pair_sums(c, vc, L, dr, nbins)
+    size, _ = _pair_sums(c, np.abs(vc), L, dr, nbins)   # sum of |v_a . v_b| component by component
+    np.testing.assert_array_equal(cnt, wcnt)
+    # FP64 products (three roundings each) added one by one: a sum of n terms
+    # is off by n 2^-53 of their magnitudes at most
+    assert np.all(np.abs(num - want) <= (cnt + 3) * 2.0**-53 * size)
+    m2, v2 = (vc.mean(0) ** 2).sum(), (vc * vc).sum(1).mean()
+    on = cnt > 0
+    wg = (want[on] / cnt[on] - m2) / (v2 - m2)
+    tol = ((cnt + 3) * 2.0**-53 * size)[on] / cnt[on] / (v2 - m2) + na * 2.0**-51 * (1.0 + np.abs(wg))
+    assert np.all(np.abs(g[on] - wg) <= tol)
