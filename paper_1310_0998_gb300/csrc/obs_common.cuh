@@ -137,7 +137,8 @@ __device__ __noinline__ void deposit_exact(const ObsState &s, int k, double dxg,
 template <int D, int W>
 __global__ void __launch_bounds__(128) k_deposit(ObsState s, double dxg, double half, long long H, int M, double *sum)
 {
-    const int k = (blockIdx.x * 128 + threadIdx.x) / W, lane = threadIdx.x % W;
+    // (the threads of 2^27 agents on 32 lanes do not fit in 32 bits)
+    const int k = (int)(blockIdx.x * (128 / W) + threadIdx.x / W), lane = threadIdx.x % W;
     if (k >= s.na) return;
     const AgentBeads<D> g = load_beads<D>(s, k);
     int f[3] = {0, 0, 0}, n[3] = {1, 1, 1};
