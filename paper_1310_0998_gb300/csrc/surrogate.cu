@@ -1133,7 +1133,10 @@ static int set_weights_host(sur_ctx *s, int k, const float *const W[3], const fl
 }
 
 // Epochs of sur_train on the tensor cores: the table goes to the device once,
-// each epoch's row order after it, and a minibatch is launches only.
+// each epoch's row order after it, and a minibatch is launches only.  The host
+// runs ahead of the device, and a copy from its memory may be taken when the
+// stream reaches it: orders go from two buffers in turn, each rewritten once its
+// last copy is done.
 static int train_tc(sur_ctx *s, const float *X, const std::vector<float> &Ts, std::vector<int> &perm, int epochs, int batch,
                     float lr, float *final_loss)
 {
@@ -1151,6 +1154,18 @@ static int train_tc(sur_ctx *s, const float *X, const std::vector<float> &Ts, st
         if (cudaMalloc((void **)&s->train, bytes) != cudaSuccess) return DPD_ERR_OOM;
         s->train_bytes = bytes;
     }
+    std::vector<int> order[2];
+    struct InFlight {   // whatever ends the call: no copy reads the host's arrays after it
+        cudaStream_t st;
+        cudaEvent_t taken[2] = {};
+        ~InFlight()
+        {
+            cudaStreamSynchronize(st);
+            for (cudaEvent_t e : taken)
+                if (e) cudaEventDestroy(e);
+        }
+    } fly{s->st};
+    for (cudaEvent_t &e : fly.taken) CUS(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     char *t = (char *)s->train;
     const float *dX = (const float *)t, *dT = (const float *)(t + o_T);
     int *sel = (int *)(t + o_sel);
@@ -1162,8 +1177,10 @@ static int train_tc(sur_ctx *s, const float *X, const std::vector<float> &Ts, st
     uint64_t st = 0x5EEDull + (uint64_t)n;
     for (int e = 0; e < epochs; ++e) {
         for (int i = n - 1; i > 0; --i) std::swap(perm[i], perm[splitmix(st) % (uint64_t)(i + 1)]);
-        // the copy has taken perm from the host before it returns (pageable memory)
-        CUS(cudaMemcpyAsync(sel, perm.data(), 4 * (size_t)n, cudaMemcpyHostToDevice, s->st));
+        CUS(cudaEventSynchronize(fly.taken[e & 1]));   // (returns at once before the first record)
+        order[e & 1] = perm;
+        CUS(cudaMemcpyAsync(sel, order[e & 1].data(), 4 * (size_t)n, cudaMemcpyHostToDevice, s->st));
+        CUS(cudaEventRecord(fly.taken[e & 1], s->st));
         CUS(cudaMemsetAsync(loss, 0, 4 * (size_t)std::max(nb, 1), s->st));
         for (int q = 0; q < nb; ++q) {
             ++s->adam_t;
