@@ -271,6 +271,8 @@ struct dpd_batch {
     std::vector<dpd_ctx *> reps;
     void *pool = nullptr;
     Sys *d_sys = nullptr;
+    std::vector<Sys> sys;                  // what d_sys holds: the replicas as created, capacities as grown
+    std::vector<int> cls_of;               // variant 2: class of each replica
     uint32_t *d_scan = nullptr, *d_scat = nullptr, *d_tiles = nullptr;
     unsigned *d_bar = nullptr;
     int *d_err = nullptr;
@@ -421,11 +423,12 @@ static void ens_free_graphs(dpd_batch *b)
 // force items of each class in a row (d_tiles keeps the order of `tiles`).  The
 // capacity takes what shared memory the class's residency leaves (tiles that
 // cluster stay off the global-memory path), or cap_min if that is more.
-static void ens_classes(dpd_batch *b, std::vector<Sys> &sys, std::vector<uint32_t> &tiles)
+static void ens_classes(dpd_batch *b, std::vector<uint32_t> &tiles)
 {
+    std::vector<Sys> &sys = b->sys;
+    std::vector<int> &cls_of = b->cls_of;
     long long blocks = (long long)tiles.size();
-    std::vector<int> cls_of(b->R);
-    b->cls.clear();
+    cls_of.assign(b->R, 0);
     for (int k = dpd_batch::MAX_CLASSES; k >= 1; --k) {
         dpd_batch::Class c{0, 0, 0, 0, 0, 0};
         for (int r = 0; r < b->R; ++r) {
@@ -493,7 +496,8 @@ static void ens_dispatch_launch(dpd_batch *b, int nsteps, int final_last, unsign
 
 static int ens_build_tables(dpd_batch *b)
 {
-    std::vector<Sys> sys(b->R);
+    std::vector<Sys> &sys = b->sys;
+    sys.resize(b->R);
     std::vector<uint32_t> order(b->R), scan, scat, tiles;
     int cap = 0;
     for (int r = 0; r < b->R; ++r) {
@@ -532,7 +536,7 @@ static int ens_build_tables(dpd_batch *b)
     for (uint32_t r : order)
         for (int k = 0; k < (sys[r].ncells + SCAN_TILE - 1) / SCAN_TILE; ++k) scan.push_back(r);
     if (b->var == 2) {
-        ens_classes(b, sys, tiles);
+        ens_classes(b, tiles);
     } else {
         // every replica's tile plan fits the common shared-memory size; the
         // dynamic buffer also serves the scan phase's transpose
@@ -545,7 +549,6 @@ static int ens_build_tables(dpd_batch *b)
     b->n_scan = (int)scan.size();
     b->n_scat = (int)scat.size();
     b->n_tiles = (int)tiles.size();
-    if (b->pool) cudaFree(b->pool);
     const size_t bytes = sizeof(Sys) * (size_t)b->R + 4 * scan.size() + 4 * scat.size() + 4 * tiles.size() +
                          sizeof(ulonglong2) * (size_t)b->R + 256 * 6;
     CUB(cudaMalloc(&b->pool, bytes));
@@ -570,6 +573,36 @@ static int ens_build_tables(dpd_batch *b)
     }
     int rc = ens_dispatch_prepare(b);
     if (rc) return rc;
+    CUB(cudaStreamSynchronize(b->st));
+    return DPD_OK;
+}
+
+// A quarter more room for the tiles of class k (variant 2; the batch is idle):
+// the class's capacity and shared memory, and its replicas' rows of the table.
+// Nothing else of the batch changes, and a step that is not taken leaves it as
+// it was.
+static int ens_grow(dpd_batch *b, int k)
+{
+    auto &c = b->cls[k];
+    const auto old = c;
+    c.cap = std::min(4096, ((c.cap * 5 / 4) + 31) & ~31);
+    while (force_smem(b->B, 2, c.cap, tile_threads<16, 2>(), true) > 200 * 1024) c.cap -= 32;
+    c.smem = force_smem(b->B, 2, c.cap, c.nt, false);
+    if (ens_dispatch_prepare(b) != DPD_OK) {
+        c = old;
+        return ens_dispatch_prepare(b);
+    }
+    // from here on the graphs are captured with the new size, before a row says so
+    ens_free_graphs(b);
+    for (int r = 0; r < b->R; ++r) {
+        if (b->cls_of[r] != k) continue;
+        b->sys[r].cap = c.cap;
+        dpd_ctx *x = b->reps[r];   // its own path, if that still is this variant's
+        if (x->var != 2) continue;
+        x->d.cap = c.cap;
+        x->smem = force_smem(b->B, 2, c.cap, x->d.nt, false);
+    }
+    CUB(cudaMemcpyAsync(b->d_sys, b->sys.data(), sizeof(Sys) * (size_t)b->R, cudaMemcpyHostToDevice, b->st));
     CUB(cudaStreamSynchronize(b->st));
     return DPD_OK;
 }
@@ -768,7 +801,7 @@ int dpd_batch_sync(dpd_batch *b)
     CUB(cudaStreamSynchronize(b->st));
     int status = DPD_OK;
     if (*(const int *)b->h_pin & ERR_TIMEOUT) status = DPD_ERR_TIMEOUT;
-    bool grown = false;
+    bool grown[dpd_batch::MAX_CLASSES] = {};
     for (int r = 0; r < b->R; ++r) {
         dpd_ctx *c = b->reps[r];
         const unsigned long long seen = c->ovf_seen, e = b->h_pin[1 + r].y;
@@ -777,17 +810,13 @@ int dpd_batch_sync(dpd_batch *b)
         if (rc && status == DPD_OK) status = rc;
         // tiles of this replica took the global-memory path: a quarter more
         // room for its class, as a single system's
-        if (b->var == 2 && c->ovf_seen > seen) {
-            c->d.cap = std::min(4096, ((c->d.cap * 5 / 4) + 31) & ~31);
-            while (force_smem(b->B, 2, c->d.cap, tile_threads<16, 2>(), true) > 200 * 1024) c->d.cap -= 32;
-            grown = true;
+        if (b->var == 2 && c->ovf_seen > seen) grown[b->cls_of[r]] = true;
+    }
+    for (int k = 0; k < dpd_batch::MAX_CLASSES; ++k)
+        if (grown[k]) {
+            const int rc = ens_grow(b, k);
+            if (rc && status == DPD_OK) status = rc;
         }
-    }
-    if (grown) {
-        ens_free_graphs(b);
-        const int rc = ens_build_tables(b);
-        if (rc && status == DPD_OK) status = rc;
-    }
     return status;
 }
 

@@ -1,0 +1,57 @@
+"""A batch whose tiles outgrow their class's capacity: what growth changes, and
+what it leaves alone."""
+import ctypes
+import time
+
+import numpy as np
+import pytest
+
+from paper_1310_0998_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+STILL = dict(a=0.0, gamma=0.0, kBT=0.0, k_bond=0.0, f_p=0.0, zeta=0.0, dt=1e-3)   # nothing moves
+L, N = 64.0, 4096
+
+
+def _clustered(k, side=6.0, seed=0):
+    """N beads, the first k of them inside a square of `side`, agents spread evenly."""
+    x, _ = synth.dimers(N // 2, L, 0.5, seed=seed)
+    c = np.random.default_rng(seed + 1).uniform(0.0, side, (k // 2, 2)) + 17.0
+    x[0:k:2] = c
+    x[1:k:2] = c + [0.25, 0.1]
+    return x
+
+
+def _overflows(ens, r):
+    return ens.replica(r).info().overflow_tiles
+
+
+def test_growth_keeps_parameters_and_bits():
+    """The tables keep the parameters that the replicas were created with (a
+    replica's own dpd_set_params is for its own steps), and every replica's
+    trajectory is that of a box alone."""
+    from paper_1310_0998_gb300 import Ensemble, Sim, _lib
+    from paper_1310_0998_gb300.sim import make_params
+    pts = [dict(L=L, n_beads=N, dt=1e-3, seed=3 + r) for r in range(3)]
+    x = [_clustered(2000 if r == 1 else 0, 14.0, seed=r) for r in range(3)]
+    v = synth.velocities(N, 0.5, seed=9)
+    with Ensemble(pts) as ens:
+        for r in range(3):
+            ens.replica(r).set_positions(x[r], v)
+        other = make_params(L, N, dt=1e-3, seed=4, f_p=7.0)
+        lib = _lib.lib()
+        assert lib.dpd_set_params(ens.replica(1)._h, ctypes.byref(other)) == 0
+        before = _overflows(ens, 1)
+        for _ in range(10):
+            ens.step(2)
+            ens.sync()
+        assert _overflows(ens, 1) > before     # there was something to grow for
+        got = [ens.replica(r).get_state() for r in range(3)]
+    for r in range(3):
+        with Sim(L, N, dt=1e-3, seed=3 + r) as s:
+            s.set_positions(x[r], v)
+            s.step(20)
+            want = s.get_state()
+        for a, b in zip(got[r][:3], want[:3]):
+            np.testing.assert_array_equal(a, b)
