@@ -579,14 +579,18 @@ static int ens_build_tables(dpd_batch *b)
 
 // A quarter more room for the tiles of class k (variant 2; the batch is idle):
 // the class's capacity and shared memory, and its replicas' rows of the table.
-// Nothing else of the batch changes, and a step that is not taken leaves it as
-// it was.
+// Nothing else of the batch changes, and growth that is not taken (the largest
+// capacity is reached) leaves it as it was, its graphs too.
 static int ens_grow(dpd_batch *b, int k)
 {
     auto &c = b->cls[k];
     const auto old = c;
     c.cap = std::min(4096, ((c.cap * 5 / 4) + 31) & ~31);
-    while (force_smem(b->B, 2, c.cap, tile_threads<16, 2>(), true) > 200 * 1024) c.cap -= 32;
+    while (c.cap > old.cap && force_smem(b->B, 2, c.cap, c.nt, true) > 200 * 1024) c.cap -= 32;
+    if (c.cap <= old.cap) {
+        c = old;
+        return DPD_OK;
+    }
     c.smem = force_smem(b->B, 2, c.cap, c.nt, false);
     if (ens_dispatch_prepare(b) != DPD_OK) {
         c = old;

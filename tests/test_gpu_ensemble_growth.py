@@ -55,3 +55,38 @@ def test_growth_keeps_parameters_and_bits():
             want = s.get_state()
         for a, b in zip(got[r][:3], want[:3]):
             np.testing.assert_array_equal(a, b)
+
+
+def test_growth_stops_at_the_largest_tile():
+    """A cluster that no tile can hold takes the global-memory path for good: a
+    synchronising call finds it there and leaves the graphs alone."""
+    from paper_1310_0998_gb300 import Ensemble
+
+    def sync_ms(k):
+        pts = [dict(STILL, L=L, n_beads=N + 4096 * (r == 0), seed=r) for r in range(24)]
+        with Ensemble(pts) as ens:
+            for r, pt in enumerate(pts):
+                n = pt["n_beads"]
+                x = np.random.default_rng(r).uniform(0.0, L, (n, 2))
+                if r == 0 and k:
+                    x[:k] = np.random.default_rng(50).uniform(17.0, 22.0, (k, 2))
+                ens.replica(r).set_positions(x)
+            for _ in range(15):          # up to the largest capacity: a quarter each
+                ens.step(1)
+                ens.sync()
+            a = _overflows(ens, 0)
+            took = []
+            for _ in range(20):
+                ens.step(1)
+                t = time.perf_counter()
+                ens.sync()
+                took.append(time.perf_counter() - t)
+            return 1e3 * min(took), _overflows(ens, 0) - a, ens.info()
+
+    base, none, _ = sync_ms(0)
+    full, some, info = sync_ms(7000)
+    assert none == 0 and some > 0        # overflows go on
+    assert info["grid"] > 0
+    # a step with the overflowing tile, and a copy of statuses: far below the tens
+    # of milliseconds that sorting the work lists and capturing graphs take
+    assert full < base + 4.0, (base, full)
