@@ -273,6 +273,7 @@ struct dpd_batch {
     Sys *d_sys = nullptr;
     std::vector<Sys> sys;                  // what d_sys holds: the replicas as created, capacities as grown
     std::vector<int> cls_of;               // variant 2: class of each replica
+    std::vector<unsigned long long> ovf;   // overflow counts that growth has answered (a replica's own calls keep their own)
     uint32_t *d_scan = nullptr, *d_scat = nullptr, *d_tiles = nullptr;
     unsigned *d_bar = nullptr;
     int *d_err = nullptr;
@@ -690,6 +691,7 @@ int dpd_batch_create(const dpd_params *p, int R, void *stream, dpd_batch **out)
     b->B = q[0].tile;
     b->var = q[0].variant;
     b->reps.assign(R, nullptr);
+    b->ovf.assign(R, 0ull);
     int rc = DPD_OK;
     for (int r = 0; r < R && rc == DPD_OK; ++r) {
         rc = dpd_create(&q[r], b->st, &b->reps[r]);
@@ -807,14 +809,13 @@ int dpd_batch_sync(dpd_batch *b)
     if (*(const int *)b->h_pin & ERR_TIMEOUT) status = DPD_ERR_TIMEOUT;
     bool grown[dpd_batch::MAX_CLASSES] = {};
     for (int r = 0; r < b->R; ++r) {
-        dpd_ctx *c = b->reps[r];
-        const unsigned long long seen = c->ovf_seen, e = b->h_pin[1 + r].y;
-        c->ovf_seen = std::max(seen, b->h_pin[1 + r].x);
+        const unsigned long long seen = b->ovf[r], e = b->h_pin[1 + r].y;
+        b->ovf[r] = std::max(seen, b->h_pin[1 + r].x);
         const int rc = e & ERR_NONFINITE ? DPD_ERR_NONFINITE : e & ERR_TIMEOUT ? DPD_ERR_TIMEOUT : e & ERR_INTERNAL ? DPD_ERR_INTERNAL : DPD_OK;
         if (rc && status == DPD_OK) status = rc;
         // tiles of this replica took the global-memory path: a quarter more
         // room for its class, as a single system's
-        if (b->var == 2 && c->ovf_seen > seen) grown[b->cls_of[r]] = true;
+        if (b->var == 2 && b->ovf[r] > seen) grown[b->cls_of[r]] = true;
     }
     for (int k = 0; k < dpd_batch::MAX_CLASSES; ++k)
         if (grown[k]) {

@@ -90,3 +90,22 @@ def test_growth_stops_at_the_largest_tile():
     # a step with the overflowing tile, and a copy of statuses: far below the tens
     # of milliseconds that sorting the work lists and capturing graphs take
     assert full < base + 4.0, (base, full)
+
+
+def test_growth_after_a_replicas_own_call():
+    """Overflows that a replica's own synchronising call sees first still grow the
+    batch: after a few steps none are left."""
+    from paper_1310_0998_gb300 import Ensemble
+    pts = [dict(STILL, L=L, n_beads=N, seed=r) for r in range(2)]
+    with Ensemble(pts) as ens:
+        for r in range(2):
+            ens.replica(r).set_positions(_clustered(2600 if r == 0 else 0, 7.0, seed=r))
+        for _ in range(12):
+            ens.step(1)
+            ens.replica(0).temperature()
+            ens.sync()
+        a = _overflows(ens, 0)
+        assert a > 0
+        ens.step(5)
+        ens.sync()
+        assert _overflows(ens, 0) == a
