@@ -60,6 +60,8 @@ def test_growth_keeps_parameters_and_bits():
 def test_growth_stops_at_the_largest_tile():
     """A cluster that no tile can hold takes the global-memory path for good: a
     synchronising call finds it there and leaves the graphs alone."""
+    import torch
+
     from paper_1310_0998_gb300 import Ensemble
 
     def sync_ms(k):
@@ -78,6 +80,7 @@ def test_growth_stops_at_the_largest_tile():
             took = []
             for _ in range(20):
                 ens.step(1)
+                torch.cuda.synchronize()
                 t = time.perf_counter()
                 ens.sync()
                 took.append(time.perf_counter() - t)
@@ -87,9 +90,9 @@ def test_growth_stops_at_the_largest_tile():
     full, some, info = sync_ms(7000)
     assert none == 0 and some > 0        # overflows go on
     assert info["grid"] > 0
-    # a step with the overflowing tile, and a copy of statuses: far below the tens
-    # of milliseconds that sorting the work lists and capturing graphs take
-    assert full < base + 4.0, (base, full)
+    # a copy of statuses, as without overflows: well below the time that sorting the
+    # work lists or rewriting a table takes, let alone the graphs of the next step
+    assert full < 2.0 * base + 0.05, (base, full)
 
 
 def test_growth_after_a_replicas_own_call():
