@@ -41,6 +41,7 @@
 
 #include "dpd.h"
 #include "obs_common.cuh"
+#include "sim_host.h"
 
 namespace dpd {
 namespace vcf {
@@ -688,11 +689,13 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     if (n > 0) k_vcf_scan<<<1, 1024, 0, st>>>(cnt, (int)ncell, start);
     k_vcf_place<D><<<gp, 256, 0, st>>>(s, n, cell_dr, vmax, sums, start, rank, (float4 *)p.P, (int4 *)p.Q, (int2 *)p.R, (int *)p.id,
                                      (double *)(buf + l.wsum()));
-    // warps per block: four, or one where the histograms are large
+    // warps per block: four, or one where the histograms are large.  The kernels'
+    // limit on shared memory is the process's: it is always set to the largest, so
+    // that no thread's call lowers it for another's.
     const int wpb = warp_smem(nbins) * 4 <= 96 * 1024 ? 4 : 1;
     const size_t sm = warp_smem(nbins) * wpb;
     if (n > 0) {
-        VCF_CU(cudaFuncSetAttribute(k_vcf_cells<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        VCF_CU(cudaFuncSetAttribute(k_vcf_cells<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dynamic_smem()));
         const int rows = D == 2 ? m + 1 : m + 1 + m * (2 * m + 1);
         int occ = 0;
         VCF_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_vcf_cells<D>, 32 * wpb, sm));
@@ -701,7 +704,7 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
         if (tasks > 2000000000ll) return DPD_ERR_INVALID_ARG;
         k_vcf_cells<D><<<(unsigned)blocks, 32 * wpb, sm, st>>>(p, start, n, m, rows, (int)tasks, cell_dr, next);
     } else {
-        VCF_CU(cudaFuncSetAttribute(k_vcf_all<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        VCF_CU(cudaFuncSetAttribute(k_vcf_all<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dynamic_smem()));
         // stretches long enough that emptying the histograms does not matter,
         // short enough for a few thousand warps
         const long long tiles = (s.na + 31) / 32;
