@@ -11,6 +11,8 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "dpd.h"
 #include "launch.cuh"
 #include "sim_kernels.cuh"
@@ -609,21 +611,39 @@ int dpd_internal_latched(dpd_ctx *c)
     return DPD_OK;
 }
 
+// Number of the allocation or registration that holds p, unique in the process; 0
+// where there is none.
+static unsigned long long buffer_of(const void *p)
+{
+    using Query = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
+    static const Query query = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &r) != cudaSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (Query)f;
+    }();
+    unsigned long long id = 0;
+    return query && query(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS ? id : 0;
+}
+
 // Page-locked host memory as kernels address it, if it starts on a multiple of
-// `align`: they read and write it at the host link's rate (209 and 192 GB/s, as
-// the copy engine), with no pass over device memory before or after.  Null for
-// other memory, which is copied.
+// `align` and one allocation or registration holds all of it (between two of them
+// there may be memory that kernels must not touch): they read and write it at the
+// host link's rate (209 and 192 GB/s, as the copy engine), with no pass over
+// device memory before or after.  Null for other memory, which is copied.
 static void *kernel_view(const void *p, size_t bytes, size_t align)
 {
-    cudaPointerAttributes a{}, e{};
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&e, (const char *)p + bytes - 1) != cudaSuccess) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    const bool host = a.type == cudaMemoryTypeHost && e.type == cudaMemoryTypeHost && a.devicePointer &&
-                      (char *)a.devicePointer + bytes - 1 == (char *)e.devicePointer;
-    return host && (uintptr_t)a.devicePointer % align == 0 ? a.devicePointer : nullptr;
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer || (uintptr_t)a.devicePointer % align != 0) return nullptr;
+    const unsigned long long id = buffer_of(p);
+    return id && buffer_of((const char *)p + bytes - 1) == id ? a.devicePointer : nullptr;
 }
 
 // What kernels read for the host array p: the array itself, or its copy in `to`.
