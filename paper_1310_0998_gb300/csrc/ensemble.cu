@@ -669,6 +669,7 @@ int dpd_batch_create(const dpd_params *p, int R, void *stream, dpd_batch **out)
     }
     // one shape for every replica: the caller's, the tuned one, or the default
     std::vector<dpd_params> q(p, p + R);
+    bool tuned = false;
     {
         int v = p[0].variant ? p[0].variant : DEFAULT_VARIANT, t = p[0].tile ? p[0].tile : DEFAULT_TILE;
         if (!p[0].tile && v == DEFAULT_VARIANT) {
@@ -676,7 +677,7 @@ int dpd_batch_create(const dpd_params *p, int R, void *stream, dpd_batch **out)
             for (int r = 0; r < R; ++r) blocks16 += blocks_of(&p[r], 16);
             t = default_tile(blocks16);
         }
-        if (!p[0].tile && !p[0].variant) tuned_shape(p, R, &t, &v);
+        tuned = !p[0].tile && !p[0].variant && tuned_shape(p, R, &t, &v);
         for (auto &e : q) { e.tile = t; e.variant = v; }
     }
     dpd_batch *b = new (std::nothrow) dpd_batch();
@@ -695,7 +696,10 @@ int dpd_batch_create(const dpd_params *p, int R, void *stream, dpd_batch **out)
     int rc = DPD_OK;
     for (int r = 0; r < R && rc == DPD_OK; ++r) {
         rc = dpd_create(&q[r], b->st, &b->reps[r]);
-        if (rc == DPD_OK) b->reps[r]->batch_owned = true;
+        if (rc == DPD_OK) {
+            b->reps[r]->batch_owned = true;
+            if (!p[0].tile && !tuned) b->reps[r]->tile_arg = DEFAULT_TILE;
+        }
     }
     if (rc == DPD_OK && cudaMallocHost((void **)&b->h_pin, sizeof(ulonglong2) * (size_t)(R + 1)) != cudaSuccess) rc = DPD_ERR_OOM;
     if (rc == DPD_OK && b->var == 2) {

@@ -685,9 +685,10 @@ int dpd_create(const dpd_params *p, void *stream, dpd_ctx **out)
     c->p = *p;
     c->var = p->variant ? p->variant : DEFAULT_VARIANT;
     c->B = p->tile ? p->tile : c->var == DEFAULT_VARIANT ? default_tile_alone(p) : DEFAULT_TILE;
+    c->tile_arg = p->tile ? p->tile : DEFAULT_TILE;
     if (!p->tile && !p->variant) {
         int t = 0, v = 0;
-        if (tuned_shape(p, 1, &t, &v)) { c->B = t; c->var = v; }
+        if (tuned_shape(p, 1, &t, &v)) { c->B = c->tile_arg = t; c->var = v; }
     }
     if (stream) {
         c->st = (cudaStream_t)stream;
@@ -776,8 +777,8 @@ int dpd_set_params(dpd_ctx *c, const dpd_params *p)
     int rc = validate(p);
     if (rc) return rc;
     if (p->n_beads != c->p.n_beads || p->L != c->p.L || p->rc != c->p.rc) return DPD_ERR_STATE;
-    const int B = p->tile ? p->tile : c->B;
-    if (B != c->B) return DPD_ERR_STATE;
+    // a tile named here is the context's, or the one that stands for the default
+    if (p->tile && p->tile != c->B && p->tile != c->tile_arg) return DPD_ERR_STATE;
     const int var = p->variant ? p->variant : c->var;
     if (var != c->var) {   // another variant's shared-memory plan
         const int nt = tile_nt(mean_owned(p, c->B), (long long)c->d.ntx * c->d.ntx, c->B, var);

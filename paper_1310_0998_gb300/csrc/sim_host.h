@@ -34,6 +34,7 @@ struct dpd_ctx {
     cudaStream_t st = nullptr;
     bool own_stream = false;
     int B = 8, var = 2, nscan = 1;
+    int tile_arg = 8;          // the tile that a caller may name for a default one (B is what it became)
     size_t smem = 0;
     void *pool = nullptr;
     size_t pool_bytes = 0;

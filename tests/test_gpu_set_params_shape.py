@@ -1,0 +1,39 @@
+"""dpd_set_params with the kernel shape named: what a caller of the default shape
+may name, and a change of variant whose tile plan is larger."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_1310_0998_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+STATE = -6
+
+
+def _set(s, **kw):
+    from paper_1310_0998_gb300 import _lib
+    from paper_1310_0998_gb300.sim import make_params
+    p = make_params(s.L, s.n, **kw)
+    return _lib.lib().dpd_set_params(s._h, ctypes.byref(p))
+
+
+@pytest.mark.parametrize("L,rho", [(24.0, 3.0), (64.0, 1.0), (300.0, 1.0)])
+def test_tile_named_for_the_default_one(L, rho):
+    """8 stands for the default tile, whatever the box made of it; the tile that
+    dpd_get_info reports can be named too, another cannot."""
+    from paper_1310_0998_gb300 import Ensemble, Sim
+    n = int(rho * L * L) // 2 * 2
+    with Sim(L, n) as s:
+        tile = s.info().tile
+        for t in (4, 8, 16):
+            assert _set(s, tile=t) == (0 if t in (8, tile) else STATE)
+        s.init_random(1)
+        s.step(2)
+    with Sim(L, n, tile=4) as s:
+        assert [_set(s, tile=t) for t in (4, 8, 16)] == [0, STATE, STATE]
+    with Ensemble([dict(L=L, n_beads=n)]) as ens:
+        r = ens.replica(0)
+        tile = r.info().tile
+        for t in (4, 8, 16):
+            assert _set(r, tile=t) == (0 if t in (8, tile) else STATE)
