@@ -782,7 +782,7 @@ int dpd_set_params(dpd_ctx *c, const dpd_params *p)
     const int var = p->variant ? p->variant : c->var;
     if (var != c->var) {   // another variant's shared-memory plan
         const int nt = tile_nt(mean_owned(p, c->B), (long long)c->d.ntx * c->d.ntx, c->B, var);
-        if (force_smem(c->B, var, c->d.cap, nt, true) > 200 * 1024) return DPD_ERR_INVALID_ARG;
+        while (force_smem(c->B, var, c->d.cap, nt, true) > 200 * 1024) c->d.cap -= 32;
         c->var = var;
         c->d.nt = nt;
         c->smem = force_smem(c->B, var, c->d.cap, nt, false);

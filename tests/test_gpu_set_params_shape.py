@@ -37,3 +37,24 @@ def test_tile_named_for_the_default_one(L, rho):
         tile = r.info().tile
         for t in (4, 8, 16):
             assert _set(r, tile=t) == (0 if t in (8, tile) else STATE)
+
+
+def test_variant_with_a_larger_tile_plan():
+    """A dense box whose capacity the new variant's plan cannot hold: its tiles get
+    a smaller one, and the bits stay."""
+    from paper_1310_0998_gb300 import Sim
+    L, nd = 64.0, 32768                       # 4096 beads and more in a 16 x 16 block
+    x, _ = synth.dimers(nd, L, 0.5, seed=1)
+    v = synth.velocities(2 * nd, 0.5, seed=2)
+    want = None
+    for first, then in ((2, 2), (1, 2), (1, 3), (3, 2), (2, 1)):
+        with Sim(L, 2 * nd, dt=1e-3, tile=16, variant=first) as s:
+            s.set_positions(x, v)
+            s.step(2)
+            assert _set(s, dt=1e-3, tile=16, variant=then) == 0
+            s.step(2)
+            got = s.get_state()
+        if want is None:
+            want = got
+        for a, b in zip(got[:3], want[:3]):
+            np.testing.assert_array_equal(a, b)
