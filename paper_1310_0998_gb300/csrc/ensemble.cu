@@ -674,8 +674,19 @@ int dpd_batch_create(const dpd_params *p, int R, void *stream, dpd_batch **out)
         int v = p[0].variant ? p[0].variant : DEFAULT_VARIANT, t = p[0].tile ? p[0].tile : DEFAULT_TILE;
         if (!p[0].tile && v == DEFAULT_VARIANT) {
             long long blocks16 = 0;
-            for (int r = 0; r < R; ++r) blocks16 += blocks_of(&p[r], 16);
-            t = default_tile(blocks16);
+            double beads = 0.0, sum = 0.0, most = 0.0;
+            for (int r = 0; r < R; ++r) {
+                const double c = beads_per_cell(&p[r]);
+                blocks16 += blocks_of(&p[r], 16);
+                beads += (double)p[r].n_beads;
+                sum += (double)p[r].n_beads * c;
+                most = std::max(most, c);
+            }
+            t = default_tile(sum / beads, blocks16);
+            // no block that the densest replica would overflow (10 beads a cell fill
+            // a 16 x 16 block's tile, 30 an 8 x 8 block's)
+            if (t == 16 && most > 9.0) t = 8;
+            if (t == 8 && most > 28.0) t = 4;
         }
         tuned = !p[0].tile && !p[0].variant && tuned_shape(p, R, &t, &v);
         for (auto &e : q) { e.tile = t; e.variant = v; }

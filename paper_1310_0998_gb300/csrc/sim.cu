@@ -327,12 +327,29 @@ int tile_capacity(const dpd_params *p, int B)
     return std::min(std::max(cap, 256), 4096);   // queue entries pack bead slots in 12 bits
 }
 
-// Cell-block side when the caller and the tuner leave it open: 16 x 16 blocks
-// carry the smaller halo (1.27 staged beads per owned one instead of 1.56) and
-// win from two blocks per SM on (us a step at density 1.6: 512 x 512 cells 44.8
-// against 52.3, 256 x 256 cells 21.5 against 21.1; 1024 x 1024 at density 3: 278
-// against 303).
-int default_tile(long long blocks16) { return blocks16 >= 304 ? 16 : 8; }
+// Cell-block side when the caller and the tuner leave it open, by the beads per
+// cell (of a batch: their mean over the beads) and the 16 x 16 blocks.  16 x 16
+// blocks carry the smaller halo (1.27 staged beads per owned one instead of 1.56)
+// and win from two blocks per SM on (us a step at density 1.6: 512 x 512 cells
+// 44.8 against 52.3, 256 x 256 cells 21.5 against 21.1; 1024 x 1024 at density 3:
+// 278 against 303), while their tiles leave three to an SM: 300 x 300 and 512 x
+// 512 cells take with 4 x 4 / 8 x 8 / 16 x 16 blocks
+//   density 3     58 / 44 / 44      145 / 93 / 89
+//   density 4.5   80 / 73 / 83      202 / 165 / 161
+//   density 6    112 / 109 / 143    293 / 266 / 336
+//   density 8    166 / 189 / 229    440 / 460 / 542
+//   density 12   337 / 456 / 1525   934 / 1209 / 4367  (16 x 16 overflow)
+//   density 24  1391 / 3347 / 5860
+int default_tile(double per_cell, long long blocks16)
+{
+    return per_cell > 7.0 ? 4 : per_cell <= 4.0 && blocks16 >= 304 ? 16 : 8;
+}
+
+double beads_per_cell(const dpd_params *p)
+{
+    const double nc = n_cells_side(p->L, p->rc);
+    return (double)p->n_beads / (nc * nc);
+}
 
 long long blocks_of(const dpd_params *p, int B)
 {
@@ -348,7 +365,7 @@ long long blocks_of(const dpd_params *p, int B)
 static int default_tile_alone(const dpd_params *p)
 {
     if (blocks_of(p, 8) <= 152 && mean_owned(p, 8) > 64.0) return 4;
-    return default_tile(blocks_of(p, 16));
+    return default_tile(beads_per_cell(p), blocks_of(p, 16));
 }
 
 // Threads per tile: about two owned beads each where the blocks fill the chip

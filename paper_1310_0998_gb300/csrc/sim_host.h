@@ -12,7 +12,8 @@ void fill_physics(Sys &d, const dpd_params *p);
 void fill_geometry(Sys &d, const dpd_params *p, int B);
 int tile_capacity(const dpd_params *p, int B);
 double mean_owned(const dpd_params *p, int B);
-int default_tile(long long blocks16);
+int default_tile(double per_cell, long long blocks16);
+double beads_per_cell(const dpd_params *p);
 long long blocks_of(const dpd_params *p, int B);
 int tile_nt(double own, long long blocks, int B, int var);
 size_t force_smem(int B, int var, int cap, int nt, bool count);
