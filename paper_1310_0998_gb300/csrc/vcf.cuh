@@ -632,12 +632,19 @@ static inline size_t result_words(int nbins) { return 32 + 4 * (size_t)nbins; }
 
 // Cells per r_max (m) and per side (n) for a box with room for n1 >= 3 cells of
 // side r_max: half cells where they still hold warps of agents (candidates
-// inside r_max: half instead of a third of them in two dimensions).
+// inside r_max: half instead of a third of them in two dimensions).  Where more
+// than `limit` of them fit a side, wider cells of about two agents each: 20,000
+// agents on 2048 x 2048 cells spent 7.0 of 7.1 ms in the scan of the counts
+// (5.2 ms as all pairs).
 template <int D>
 static void cells_for(double L, double rmax, int na, int limit, int *m, int *n)
 {
-    const int n1 = (int)std::min<double>(std::floor(L / rmax), limit);
-    const int n2 = (int)std::floor(2.0 * L / rmax);
+    if (L / rmax >= limit + 1.0) {
+        *m = 1;
+        *n = std::min(std::max((int)std::pow(0.5 * na, 1.0 / D), 3), limit);
+        return;
+    }
+    const int n1 = (int)std::floor(L / rmax), n2 = (int)std::floor(2.0 * L / rmax);
     const bool half = n2 <= limit && na / std::pow((double)n2, D) >= 48.0;
     *m = half ? 2 : 1;
     *n = half ? n2 : n1;

@@ -44,3 +44,22 @@ def test_counts(D, L, na, dr, nbins):
         r2 = r2 + d[:, 2] * d[:, 2]
     b = np.floor(np.sqrt(r2) / dr)
     np.testing.assert_array_equal(cnt, [(b == k).sum() for k in range(nbins)])
+
+
+def test_few_agents_take_no_million_cells():
+    """300 agents out to L / 100,000: as many cells as agents at most, not the
+    4,194,304 that the box has room for (7 ms a call in the scan of their counts)."""
+    import time
+
+    from paper_1310_0998_gb300 import Sim
+    L, na = 1000.0, 300
+    x = _pairs(2, L, na, 0.01, 4)
+    v = np.random.default_rng(6).standard_normal(x.shape).astype(np.float32)
+    with Sim(L, len(x), dt=1e-6) as s:
+        s.set_state(x, v, np.zeros_like(v))
+        took = []
+        for _ in range(8):
+            t = time.perf_counter()
+            s.velocity_correlation(1e-3, 10)
+            took.append(time.perf_counter() - t)
+    assert min(took) < 2e-3, took
