@@ -515,11 +515,11 @@ struct Warp {
 
 __host__ __device__ inline size_t warp_smem(int nbins) { return (size_t)nbins * 16 + QUEUE * sizeof(uint2); }
 
-// Cells: task (cell, row of neighbour cells), rows 0 .. of the forward half
-// stencil of m cells each way (row 0: the own cell and those east of it), taken
-// from a counter.
+// Cells: task (cell, row of neighbour cells, one of `parts` shares of the cell's
+// agents), rows 0 .. of the forward half stencil of m cells each way (row 0: the own
+// cell and those east of it), taken from a counter.
 template <int D, bool WIDE>
-__device__ __forceinline__ void cells_pass(const Pass &p, const unsigned *start, int n, int m, int rows, int tasks,
+__device__ __forceinline__ void cells_pass(const Pass &p, const unsigned *start, int n, int m, int rows, int parts, int tasks,
                                            float cell_dr, unsigned *next)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -530,7 +530,7 @@ __device__ __forceinline__ void cells_pass(const Pass &p, const unsigned *start,
         if (w.lane == 0) t = atomicAdd(next, 1u);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= (unsigned)tasks) break;
-        const int cell = (int)t / rows, row = (int)t - cell * rows;
+        const int u = (int)t / parts, part = (int)t - u * parts, cell = u / rows, row = u - cell * rows;
         int c[3] = {cell % n, (cell / n) % n, D == 3 ? cell / (n * n) : 0};
         // row r > 0: forward rows in (dz, dy) order after (0, 0)
         int dy = row, dz = 0;
@@ -541,7 +541,7 @@ __device__ __forceinline__ void cells_pass(const Pass &p, const unsigned *start,
         const int yy = c[1] + dy, zz = c[2] + dz;
         const int ny = yy < 0 ? yy + n : (yy >= n ? yy - n : yy), nz = zz >= n ? zz - n : zz;
         const int a0 = (int)start[cell], a1 = (int)start[cell + 1];
-        for (int g = a0; g < a1; g += 32) {
+        for (int g = a0 + 32 * part; g < a1; g += 32 * parts) {
             w.load(g + w.lane, a1);
             for (int dx = row == 0 ? 0 : -m; dx <= m; ++dx) {
                 const int xx = c[0] + dx, nx = xx < 0 ? xx + n : (xx >= n ? xx - n : xx);
@@ -554,17 +554,17 @@ __device__ __forceinline__ void cells_pass(const Pass &p, const unsigned *start,
     w.finish();
 }
 template <int D>
-__device__ __noinline__ void cells_pass_wide(const Pass &p, const unsigned *start, int n, int m, int rows, int tasks,
+__device__ __noinline__ void cells_pass_wide(const Pass &p, const unsigned *start, int n, int m, int rows, int parts, int tasks,
                                              float cell_dr, unsigned *next)
 {
-    cells_pass<D, true>(p, start, n, m, rows, tasks, cell_dr, next);
+    cells_pass<D, true>(p, start, n, m, rows, parts, tasks, cell_dr, next);
 }
 template <int D>
 __global__ void __launch_bounds__(128) k_vcf_cells(const __grid_constant__ Pass p, const unsigned *start, int n, int m,
-                                                   int rows, int tasks, float cell_dr, unsigned *next)
+                                                   int rows, int parts, int tasks, float cell_dr, unsigned *next)
 {
-    if (wide_speeds<D>(*p.vmax, p.sums, p.s.na)) cells_pass_wide<D>(p, start, n, m, rows, tasks, cell_dr, next);
-    else cells_pass<D, false>(p, start, n, m, rows, tasks, cell_dr, next);
+    if (wide_speeds<D>(*p.vmax, p.sums, p.s.na)) cells_pass_wide<D>(p, start, n, m, rows, parts, tasks, cell_dr, next);
+    else cells_pass<D, false>(p, start, n, m, rows, parts, tasks, cell_dr, next);
 }
 
 // All pairs: a warp's 32 agents against a stretch of `cols` agents after them.
@@ -706,10 +706,15 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
         const int rows = D == 2 ? m + 1 : m + 1 + m * (2 * m + 1);
         int occ = 0;
         VCF_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_vcf_cells<D>, 32 * wpb, sm));
-        const long long tasks = (long long)ncell * rows;
+        // few cells: a cell's agents by shares of 32, for 24 warps an SM (400,000
+        // agents in 16 cells, 64 shells: 0.12 s against 2.29; 60,000 in 400 cells,
+        // 512 shells: 0.33 ms against 0.89)
+        const long long each = (s.na / (long long)ncell + 31) / 32, want = 24ll * nsm / ((long long)ncell * rows);
+        const int parts = (int)std::max<long long>(std::min(each, want), 1);
+        const long long tasks = (long long)ncell * rows * parts;
         const long long blocks = std::min<long long>((tasks + wpb - 1) / wpb, (long long)nsm * std::max(occ, 1));
         if (tasks > 2000000000ll) return DPD_ERR_INVALID_ARG;
-        k_vcf_cells<D><<<(unsigned)blocks, 32 * wpb, sm, st>>>(p, start, n, m, rows, (int)tasks, cell_dr, next);
+        k_vcf_cells<D><<<(unsigned)blocks, 32 * wpb, sm, st>>>(p, start, n, m, rows, parts, (int)tasks, cell_dr, next);
     } else {
         VCF_CU(cudaFuncSetAttribute(k_vcf_all<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dynamic_smem()));
         // stretches long enough that emptying the histograms does not matter,

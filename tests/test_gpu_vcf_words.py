@@ -133,3 +133,16 @@ def test_wide_speeds(D, L, na, dr, nbins, scale):
     wg = (want[on] / cnt[on] - m2) / (v2 - m2)
     tol = ((cnt + 3) * 2.0**-53 * size)[on] / cnt[on] / (v2 - m2) + na * 2.0**-51 * (1.0 + np.abs(wg))
     assert np.all(np.abs(g[on] - wg) <= tol)
+
+
+@pytest.mark.parametrize("D,L,na,dr,nbins", [(2, 32.0, 31, 5.0, 2), (2, 32.0, 290, 5.0, 2), (2, 32.0, 1200, 2.5, 4), (2, 32.0, 600, 0.02, 500),
+                                             (3, 12.0, 33, 1.0, 4), (3, 12.0, 1500, 1.9, 2)])
+def test_shares_of_few_cells(D, L, na, dr, nbins):
+    """Grids of 9 to 27 cells, whose agents are shared out by 32."""
+    c, x = _state(D, L, na, na + 9)
+    v = np.random.default_rng(na).standard_normal((2 * na, D)).astype(np.float32)
+    _, _, num, cnt = _run(D, L, x, v, dr, nbins)
+    vc = 0.5 * (v[0::2].astype(np.longdouble) + v[1::2].astype(np.longdouble))
+    want, wcnt = _pair_sums(c, vc, L, dr, nbins)
+    np.testing.assert_array_equal(cnt, wcnt)
+    assert np.all(np.abs(num - want) <= cnt * 2.0**-55 * (vc * vc).sum(1).max() + 2.0**-53 * np.abs(want))
