@@ -264,7 +264,7 @@ int dpd_velocity_correlation(dpd_ctx *c, double dr, int nbins, double *g, double
     int rc = vcf::vcf_run<2>(state, dr, nbins, m, n, (char *)s->buf, c->st, &res);
     if (rc) return rc;
     rc = small_out(c, host.data(), res, 8 * host.size());
-    vcf::vcf_outputs(vcf::vcf_finish<2>(host, na, nbins), dr, nbins, g, L_int, num, cnt);
+    vcf::vcf_outputs(vcf::vcf_finish<2>(host, na, nbins, n), dr, nbins, g, L_int, num, cnt);
     return rc;
 }
 

@@ -254,7 +254,7 @@ int dpd3_velocity_correlation(dpd3_ctx *c, double dr, int nbins, double *g, doub
     if (rc) return rc;
     CUO3(cudaMemcpyAsync(host.data(), res, 8 * host.size(), cudaMemcpyDeviceToHost, c->st));
     rc = dpd3_internal_latched(c);
-    vcf::vcf_outputs(vcf::vcf_finish<3>(host, na, nbins), dr, nbins, g, L_int, num, cnt);
+    vcf::vcf_outputs(vcf::vcf_finish<3>(host, na, nbins, n), dr, nbins, g, L_int, num, cnt);
     return rc;
 }
 

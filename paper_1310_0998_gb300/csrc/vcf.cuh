@@ -18,7 +18,8 @@
 //               R_a . R_b: good to 2^-55 of the largest |v|^2.  Where the
 //               fastest agent's |v|^2 is no FP32 number, or the mean |v|^2 lies
 //               so far below it (256 to 1024 times) that FP64 products would be
-//               the better ones, the same pass takes those, with FP64 sums.
+//               the better ones, the same pass takes those, with FP64 sums (so do
+//               all pairs of more than MANY shells).
 //   sums        three 21-bit limbs of a product and the count go to the warp's
 //               own histogram in shared memory by native 32-bit integer adds;
 //               it is emptied into 64-bit global sums before a word can
@@ -175,11 +176,11 @@ __global__ void __launch_bounds__(256) k_vcf_count(State s, int n, const unsigne
 // (and R) hold v, and wsum gets the sums of v (three) and |v|^2.
 template <int D>
 __global__ void __launch_bounds__(256) k_vcf_place(State s, int n, float cell_dr, const unsigned *vmax,
-                                                   const long long *sums, const unsigned *start, const unsigned *rank,
+                                                   const long long *sums, bool real, const unsigned *start, const unsigned *rank,
                                                    float4 *P, int4 *Q, int2 *R, int *id, double *wsum)
 {
     const int k = blockIdx.x * 256 + threadIdx.x;
-    const bool wide = wide_speeds<D>(*vmax, sums, s.na);
+    const bool wide = real || wide_speeds<D>(*vmax, sums, s.na);
     double w[4] = {0.0, 0.0, 0.0, 0.0};
     if (wide) {
         if (k < s.na) {
@@ -283,6 +284,7 @@ struct Pass {
     int nbins;
     const unsigned *vmax;      // what wide_speeds takes
     const long long *sums;
+    bool real;                 // FP64 products whatever the speeds
     float lim2, mg;            // (nbins + mg)^2, and the distance from a shell edge that FP32 decides
     long long *gsum;           // [3][nbins] limb sums (FP64 products: [nbins] doubles)
     unsigned long long *gcnt;  // [nbins]
@@ -295,9 +297,10 @@ constexpr int QUEUE = 160;
 __device__ __forceinline__ int room_after(int most) { return ((1 << 11) - 32 - most) / 32 & ~3; }
 constexpr int FULL_AT = 992;    // count from which the histogram is emptied at a look: room for 60 then, for 32 below
 
-// (WIDE: FP64 products and sums; the histogram is nbins doubles, and the counts
-// where they are otherwise.)
-template <int D, bool WIDE>
+// WIDE: FP64 products and sums; the histogram is nbins doubles, and the counts where
+// they are otherwise.  SHARED (and WIDE): the block's warps add to one histogram,
+// nbins doubles and nbins counts, which the block clears and empties.
+template <int D, bool WIDE, bool SHARED>
 struct Warp {
     const Pass &p;
     int *h;            // [4][nbins]: low, middle, high limb, count (this warp's)
@@ -314,7 +317,8 @@ struct Warp {
     __device__ Warp(const Pass &pass, int *hist, uint2 *queue)
         : p(pass), h(hist), q(queue), qn(0), lane(threadIdx.x & 31), a(-1), room(room_after(0))
     {
-        for (int i = lane; i < 4 * p.nbins; i += 32) h[i] = 0;
+        if (!SHARED)
+            for (int i = lane; i < 4 * p.nbins; i += 32) h[i] = 0;
         __syncwarp();
     }
     __device__ __forceinline__ Vel vel(int b) const
@@ -355,7 +359,7 @@ struct Warp {
     __device__ __forceinline__ void add(int bin, double d)
     {
         atomicAdd(reinterpret_cast<double *>(h) + bin, d);
-        atomicAdd(h + 3 * p.nbins + bin, 1);
+        atomicAdd(h + (SHARED ? 2 : 3) * p.nbins + bin, 1);
     }
     __device__ __forceinline__ void add(int bin, long long d)
     {
@@ -454,8 +458,8 @@ struct Warp {
         }
         const float lim2 = a >= 0 ? p.lim2 : -1.0f, inside = 0.5f - p.mg, last = (float)p.nbins - p.mg;
         while (s < e) {
-            const int stop = min(e, s + room);
-            room -= (stop - s + 3) & ~3;
+            const int stop = SHARED ? e : min(e, s + room);
+            if (!SHARED) room -= (stop - s + 3) & ~3;
             for (; s < stop; s += 4) {
                 unsigned near = 0u;   // candidates whose shell FP32 does not decide
                 float t2[4];
@@ -494,7 +498,7 @@ struct Warp {
                     while (qn >= 32) drain();
                 }
             }
-            if (room > 0) continue;
+            if (SHARED || room > 0) continue;
             __syncwarp();
             int most = 0;
             for (int b = lane; b < p.nbins; b += 32) most = max(most, h[3 * p.nbins + b]);
@@ -509,7 +513,7 @@ struct Warp {
     __device__ __forceinline__ void finish()
     {
         while (qn > 0) drain();
-        flush();
+        if (!SHARED) flush();
     }
 };
 
@@ -524,7 +528,7 @@ __device__ __forceinline__ void cells_pass(const Pass &p, const unsigned *start,
 {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char *mine = smem + warp_smem(p.nbins) * (threadIdx.x >> 5);
-    Warp<D, WIDE> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
+    Warp<D, WIDE, false> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
     while (true) {
         unsigned t = 0;
         if (w.lane == 0) t = atomicAdd(next, 1u);
@@ -568,7 +572,7 @@ __global__ void __launch_bounds__(128) k_vcf_cells(const __grid_constant__ Pass 
 }
 
 // All pairs: a warp's 32 agents against a stretch of `cols` agents after them.
-template <int D, bool WIDE>
+template <int D>
 __device__ __forceinline__ void all_pass(const Pass &p, int cols, float unit)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -576,22 +580,51 @@ __device__ __forceinline__ void all_pass(const Pass &p, int cols, float unit)
     const int s = max(a0, (int)blockIdx.y * cols), e = min(p.s.na, ((int)blockIdx.y + 1) * cols);
     if (a0 >= p.s.na || s >= e) return;   // a whole warp at a time; no block barrier below
     unsigned char *mine = smem + warp_smem(p.nbins) * (threadIdx.x >> 5);
-    Warp<D, WIDE> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
+    Warp<D, false, false> w(p, (int *)(mine + QUEUE * sizeof(uint2)), (uint2 *)mine);
     w.load(a0 + w.lane, p.s.na);
     w.template run<true>(s, e, nullptr, w.a, unit);
     w.finish();
 }
+// The same with FP64 products: one histogram per block (its shared FP64 adds are
+// compare-and-swap loops, which wait more than they collide), 12 bytes a shell.
+__host__ __device__ inline size_t block_smem(int nbins, int warps) { return (size_t)nbins * 12 + warps * QUEUE * sizeof(uint2); }
 template <int D>
 __device__ __noinline__ void all_pass_wide(const Pass &p, int cols, float unit)
 {
-    all_pass<D, true>(p, cols, unit);
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int warps = (int)(blockDim.x >> 5), warp = (int)(threadIdx.x >> 5), nb = p.nbins;
+    const int b0 = (int)blockIdx.x * warps * 32, a0 = b0 + 32 * warp, c0 = (int)blockIdx.y * cols;
+    const int e = min(p.s.na, c0 + cols);
+    if (b0 >= p.s.na || max(b0, c0) >= e) return;   // the whole block
+    int *h = (int *)(smem + warps * QUEUE * sizeof(uint2));
+    for (int i = threadIdx.x; i < 3 * nb; i += blockDim.x) h[i] = 0;
+    __syncthreads();
+    if (a0 < p.s.na && max(a0, c0) < e) {
+        Warp<D, true, true> w(p, h, (uint2 *)smem + warp * QUEUE);
+        w.load(a0 + w.lane, p.s.na);
+        w.template run<true>(max(a0, c0), e, nullptr, w.a, unit);
+        w.finish();
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+        if (h[2 * nb + b] == 0) continue;
+        atomicAdd(reinterpret_cast<double *>(p.gsum) + b, reinterpret_cast<const double *>(h)[b]);
+        atomicAdd(&p.gcnt[b], (unsigned long long)(unsigned)h[2 * nb + b]);
+    }
 }
 template <int D>
 __global__ void __launch_bounds__(128) k_vcf_all(const __grid_constant__ Pass p, int cols, float unit)
 {
-    if (wide_speeds<D>(*p.vmax, p.sums, p.s.na)) all_pass_wide<D>(p, cols, unit);
-    else all_pass<D, false>(p, cols, unit);
+    if (p.real || wide_speeds<D>(*p.vmax, p.sums, p.s.na)) all_pass_wide<D>(p, cols, unit);
+    else all_pass<D>(p, cols, unit);
 }
+
+// All pairs of more shells than this take FP64 products: a warp's whole-number
+// histogram of 8,192 shells leaves one warp to an SM (60,000 agents: 157 ms against 32
+// with a block's FP64 one).  Up to here the sums that no order changes are kept, at
+// 44 ms against 22 for 4,096 shells; below 2,500 they are the faster ones too (18
+// against 21 for 2,048, 9 against 20 for 1,024).
+constexpr int MANY = 4096;
 
 // Host results of a pass.
 struct Out {
@@ -671,6 +704,7 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     p.id = (const int *)(buf + l.id);
     p.dr = dr;
     p.nbins = nbins;
+    p.real = n == 0 && nbins > MANY;
     p.vmax = vmax;
     p.sums = sums;
     // FP32 error of r / dr in half-ulps u = 2^-24.  Cells of side c (in dr): a
@@ -694,13 +728,13 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
     k_vcf_max<D><<<g, 256, 0, st>>>(s, vmax);
     k_vcf_count<D><<<g, 256, 0, st>>>(s, n, vmax, cnt, rank, sums);
     if (n > 0) k_vcf_scan<<<1, 1024, 0, st>>>(cnt, (int)ncell, start);
-    k_vcf_place<D><<<gp, 256, 0, st>>>(s, n, cell_dr, vmax, sums, start, rank, (float4 *)p.P, (int4 *)p.Q, (int2 *)p.R, (int *)p.id,
+    k_vcf_place<D><<<gp, 256, 0, st>>>(s, n, cell_dr, vmax, sums, p.real, start, rank, (float4 *)p.P, (int4 *)p.Q, (int2 *)p.R, (int *)p.id,
                                      (double *)(buf + l.wsum()));
     // warps per block: four, or one where the histograms are large.  The kernels'
     // limit on shared memory is the process's: it is always set to the largest, so
     // that no thread's call lowers it for another's.
-    const int wpb = warp_smem(nbins) * 4 <= 96 * 1024 ? 4 : 1;
-    const size_t sm = warp_smem(nbins) * wpb;
+    int wpb = warp_smem(nbins) * 4 <= 96 * 1024 ? 4 : 1;
+    size_t sm = warp_smem(nbins) * wpb;
     if (n > 0) {
         VCF_CU(cudaFuncSetAttribute(k_vcf_cells<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dynamic_smem()));
         const int rows = D == 2 ? m + 1 : m + 1 + m * (2 * m + 1);
@@ -717,6 +751,10 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
         k_vcf_cells<D><<<(unsigned)blocks, 32 * wpb, sm, st>>>(p, start, n, m, rows, parts, (int)tasks, cell_dr, next);
     } else {
         VCF_CU(cudaFuncSetAttribute(k_vcf_all<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dynamic_smem()));
+        if (p.real) {
+            wpb = 4;
+            sm = block_smem(nbins, wpb);
+        }
         // stretches long enough that emptying the histograms does not matter,
         // short enough for a few thousand warps
         const long long tiles = (s.na + 31) / 32;
@@ -732,7 +770,7 @@ static int vcf_run(const State &s, double dr, int nbins, int m, int n, char *buf
 }
 
 template <int D>
-static Out vcf_finish(const std::vector<long long> &host, int na, int nbins)
+static Out vcf_finish(const std::vector<long long> &host, int na, int nbins, int n)
 {
     Out o;
     const uint32_t vmax = (uint32_t)((unsigned long long)host[0] & 0xffffffffull);
@@ -741,7 +779,7 @@ static Out vcf_finish(const std::vector<long long> &host, int na, int nbins)
     o.num.resize(nbins);
     o.cnt.resize(nbins);
     for (int b = 0; b < nbins; ++b) o.cnt[b] = (unsigned long long)g[3 * nbins + b];
-    if (wide_speeds<D>(vmax, s, na)) {
+    if ((n == 0 && nbins > MANY) || wide_speeds<D>(vmax, s, na)) {
         double w[4];
         std::memcpy(w, host.data() + 24, sizeof w);
         for (int i = 0; i < 3; ++i) o.mean[i] = w[i] / na;
@@ -753,9 +791,11 @@ static Out vcf_finish(const std::vector<long long> &host, int na, int nbins)
         o.mean[i] = i < D ? std::ldexp((double)s[2 * i] + std::ldexp((double)s[2 * i + 1], -32), -k) / na : 0.0;
     const __int128 q = ((__int128)s[2 * D + 1] << 32) + s[2 * D] + s[2 * D + 2];
     o.v2 = std::ldexp((double)q, -2 * k) / na;
+    const double unit = std::ldexp(1.0, -2 * k);   // (a power of two: exact)
     for (int b = 0; b < nbins; ++b) {
-        const __int128 t = ((__int128)g[2 * nbins + b] << (2 * LIMB)) + ((__int128)g[nbins + b] << LIMB) + g[b];
-        o.num[b] = std::ldexp((double)t, -2 * k);
+        const long long hi = g[2 * nbins + b], mid = g[nbins + b], lo = g[b];
+        if (o.cnt[b] < 2048 && hi > -(1ll << 19) && hi < 1ll << 19) o.num[b] = (double)(hi * (1ll << (2 * LIMB)) + (mid << LIMB) + lo) * unit;
+        else o.num[b] = (double)(((__int128)hi << (2 * LIMB)) + ((__int128)mid << LIMB) + lo) * unit;
     }
     return o;
 }

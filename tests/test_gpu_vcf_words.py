@@ -146,3 +146,29 @@ def test_shares_of_few_cells(D, L, na, dr, nbins):
     want, wcnt = _pair_sums(c, vc, L, dr, nbins)
     np.testing.assert_array_equal(cnt, wcnt)
     assert np.all(np.abs(num - want) <= cnt * 2.0**-55 * (vc * vc).sum(1).max() + 2.0**-53 * np.abs(want))
+
+
+@pytest.mark.parametrize("nbins", [4096, 4097, 6000, 8192])
+@pytest.mark.parametrize("kind", ["alike", "wide"])
+def test_many_shells(nbins, kind):
+    """Both sides of the number of shells from which all pairs take a block's FP64
+    histogram."""
+    D, L, na = 2, 32.0, 500
+    c, x = _state(D, L, na, 77)
+    v = np.random.default_rng(78).standard_normal((2 * na, D)).astype(np.float32)
+    if kind == "wide":
+        v[10:12] *= 4096.0
+    dr = 23.0 / nbins                     # past every pair (L 2^-1/2 = 22.6)
+    _, _, num, cnt = _run(D, L, x, v, dr, nbins)
+    vc = 0.5 * (v[0::2].astype(np.longdouble) + v[1::2].astype(np.longdouble))
+    d = c[:, None, :] - c[None, :, :]
+    d -= L * np.rint(d / L)
+    b = np.floor(np.sqrt((d * d).sum(2)) / dr).astype(np.int64)
+    i, j = np.triu_indices(na, 1)
+    want, size = np.zeros(nbins, np.longdouble), np.zeros(nbins, np.longdouble)
+    np.add.at(want, b[i, j], (vc[i] * vc[j]).sum(1))
+    np.add.at(size, b[i, j], np.abs(vc[i] * vc[j]).sum(1))
+    np.testing.assert_array_equal(cnt, np.bincount(b[i, j], minlength=nbins))
+    v2 = (vc * vc).sum(1).max()
+    bound = (cnt + 3) * 2.0**-53 * size if kind == "wide" or nbins > 4096 else cnt * 2.0**-55 * v2 + 2.0**-53 * np.abs(want)
+    assert np.all(np.abs(num - want) <= bound)
