@@ -942,7 +942,7 @@ struct sur_ctx {
     float h_mu_y[NOUT], h_sd_y[NOUT];
     // activations, sized for cap rows
     __nv_bfloat16 *X0, *X0T, *A1, *A1T, *A2, *A2T, *dY, *dYT, *dZ1, *dZ1T, *dZ2, *dZ2T;
-    float *Z1, *Z2, *Y, *dA, *dY32, *T, *Xin, *loss, *Yall, *Yout, *Sout;
+    float *Z1, *Z2, *Y, *dY32, *T, *Xin, *loss, *Yall, *Yout, *Sout;
     Member *d_mem = nullptr;            // device copies of the tables
     Act *d_act = nullptr;
     void *extra = nullptr;              // activations of members 1.. in a batched step (training, small predictions)
@@ -1267,7 +1267,7 @@ int sur_create(int n_members, int max_rows, uint64_t seed, void *stream, sur_ctx
                  o_dY = take(2 * M * NOUT_P), o_dYT = take(2 * M * NOUT_P), o_dZ1 = take(2 * M * NH),
                  o_dZ1T = take(2 * M * NH), o_dZ2 = take(2 * M * NH), o_dZ2T = take(2 * M * NH),
                  o_Z1 = take(4 * M * NH), o_Z2 = take(4 * M * NH), o_Y = take(4 * M * NOUT_P),
-                 o_dA = take(4 * M * NH), o_dY32 = take(4 * M * NOUT_P), o_T = take(4 * M * NOUT),
+                 o_dY32 = take(4 * M * NOUT_P), o_T = take(4 * M * NOUT),
                  o_Xin = take(4 * M * NIN), o_loss = take(64), o_Yall = take(4 * M * NOUT_P * (size_t)s->K),
                  o_Yout = take(4 * M * NOUT), o_Sout = take(4 * M * NOUT), o_err = take(4);
     if (cudaMalloc(&s->pool, off) != cudaSuccess || cudaMallocHost((void **)&s->h_loss, 64) != cudaSuccess) {
@@ -1293,7 +1293,7 @@ int sur_create(int n_members, int max_rows, uint64_t seed, void *stream, sur_ctx
     s->dY = (__nv_bfloat16 *)(p + o_dY); s->dYT = (__nv_bfloat16 *)(p + o_dYT);
     s->dZ1 = (__nv_bfloat16 *)(p + o_dZ1); s->dZ1T = (__nv_bfloat16 *)(p + o_dZ1T);
     s->dZ2 = (__nv_bfloat16 *)(p + o_dZ2); s->dZ2T = (__nv_bfloat16 *)(p + o_dZ2T);
-    s->Z1 = (float *)(p + o_Z1); s->Z2 = (float *)(p + o_Z2); s->Y = (float *)(p + o_Y); s->dA = (float *)(p + o_dA);
+    s->Z1 = (float *)(p + o_Z1); s->Z2 = (float *)(p + o_Z2); s->Y = (float *)(p + o_Y);
     s->dY32 = (float *)(p + o_dY32); s->T = (float *)(p + o_T); s->Xin = (float *)(p + o_Xin);
     s->loss = (float *)(p + o_loss); s->Yall = (float *)(p + o_Yall); s->Yout = (float *)(p + o_Yout);
     s->Sout = (float *)(p + o_Sout);
