@@ -195,10 +195,12 @@ __global__ void __launch_bounds__(TILE_THREADS, B == 16 ? 5 : 8)
 // The persistent kernel holds its scan and scatter beside the force tile, which
 // spilled (288 bytes at the 56 registers that three 384-thread tiles leave), and
 // one launch shape for every replica: 0.74 ms a step for the 256 replicas of
-// 4.7 M beads, 0.55 of it the force phase.  As ordinary launches each phase has
-// its own registers, blocks come from the hardware queue instead of a counter, and
-// the force items go in classes of mean density with threads and shared memory of
-// their own (a dilute tile needs a third of a dense one's).
+// 4.7 M beads, 0.55 of it the force phase.  As ordinary launches the scan and the
+// scatter leave the force kernel's registers alone (it still spills 128 bytes at
+// 56, for the descriptor's pointers; a single box's spills none), blocks come from
+// the hardware queue instead of a counter, and the force items go in classes of mean
+// density with threads and shared memory of their own (a dilute tile needs a third
+// of a dense one's): 0.456 ms of force phase.
 // busy (a profiling launch): the blocks' working times in ns are added to it.
 __device__ __forceinline__ void add_busy(unsigned long long *busy, unsigned long long t0)
 {

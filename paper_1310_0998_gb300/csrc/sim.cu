@@ -324,7 +324,7 @@ int tile_capacity(const dpd_params *p, int B)
     // synchronising call
     int cap = (int)std::ceil(mean + 6.5 * std::sqrt(mean));
     cap = (cap + 31) & ~31;
-    return std::min(std::max(cap, 256), 4096);   // queue entries pack bead slots in 12 bits
+    return std::min(std::max(cap, 256), 4096);   // the queues of variants 3 to 5 pack bead slots in 12 bits (2: in 16)
 }
 
 // Cell-block side when the caller and the tuner leave it open, by the beads per

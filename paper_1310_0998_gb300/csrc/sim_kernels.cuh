@@ -1,13 +1,13 @@
 // Per-step device work of the DPD dimer simulator, written as device
-// functions so that the single-system kernels and the persistent ensemble
-// kernel share them.
+// functions so that the single-system kernels and the ensemble's share them.
 //
 // One step s -> s+1 (standard velocity-Verlet, Sec. 5 of arXiv:1310.0998):
 //   scan     cstart = exclusive_scan(counts), counts = 0, step += 1
 //   scatter  U (unsorted, with ranks) -> S sorted by cell, slot[id]
 //   force    per tile: pair forces (Eqs. DPDf, DPDcdr, weightFunc01), bond
 //            (Eq. stiffSpring), propulsion and drag (Eq. DPDnp); then
-//            v_s = v* + dt/2m f_s (skipped at set-up), FP64 thermo partials,
+//            v_s = v* + dt/2m f_s (skipped at set-up), thermo partials (whole
+//            numbers per tile in variant 2, FP64 in the others),
 //            v_{s+1/2} = v_s + dt/2m f_s, x_{s+1} = wrap(x_s + dt v_{s+1/2}),
 //            binning of x_{s+1} into counts (rank = atomic ticket) -> U.
 #pragma once

@@ -7,9 +7,11 @@
 // ln zeta, f_p); inputs and targets are standardised with statistics of the
 // training set.
 //
-// All matrix products are one kernel, C[M x N] = A[M x K] B[N x K]^T with
-// both operands K-contiguous BF16, computed by warps issuing
-// mma.sync.m16n8k16 (BF16 x BF16 -> FP32), with an epilogue chosen per use:
+// All matrix products are C[M x N] = A[M x K] B[N x K]^T with both operands
+// K-contiguous BF16 and FP32 accumulation: on the 5th-generation tensor cores
+// (tcgen05.mma: the layer kernels of training and small predictions, the fused
+// forward pass of large ones) or, as the backend to compare with, by one kernel
+// of warps issuing mma.sync.m16n8k16.  The epilogue is chosen per use:
 //   forward      Z = X W^T + b; A = silu(Z) stored as BF16 row-major and
 //                transposed (the transposed copy feeds the weight gradient)
 //   dW           dW = dZ^T X  (A = dZ^T, B = X^T, both batch-contiguous)

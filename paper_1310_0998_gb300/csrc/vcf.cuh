@@ -26,10 +26,11 @@
 //               overflow.  Whole-number sums do not depend on the order.
 // A warp takes 32 agents of a cell at a time, one per lane, against the agents of
 // a neighbour cell, whose data every lane reads at the same address.
-// Bound by instruction issue (54 warp instructions per 32 candidates, half of
-// them inside r_max).  1,572,864 agents, r < 16, 64 shells (9.5e8 pairs): 4.0 ms
-// against 27.7 with FP64 products and shared FP64 adds; a cube of 393,216, r < 4:
-// 1.4 against 6.0; all pairs of 1,382 agents (96 shells): 22 us against 410.
+// Bound by instruction issue (58 warp instructions per 32 candidates, half of
+// them inside r_max).  1,572,864 agents, r < 16, 64 shells (9.5e8 pairs): 4.5 ms
+// against 27.7 with FP64 products and shared FP64 adds (4.0 with FP32 cross terms,
+// which left a product good to 2^-49 of the largest |v|^2); a cube of 393,216, r <
+// 4: 1.4 against 6.0; all pairs of 1,382 agents (96 shells): 23 us against 410.
 #pragma once
 #include <algorithm>
 #include <cmath>

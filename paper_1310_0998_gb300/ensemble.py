@@ -9,8 +9,9 @@ from .sim import Sim, make_params
 
 
 class Ensemble:
-    """R replicas of uneven size and parameters, advanced together by one
-    persistent kernel per call.  `points`: list of dicts with L, n_beads and
+    """R replicas of uneven size and parameters, advanced together (variant 2:
+    one launch per phase of a step; the others: one persistent kernel per
+    call).  `points`: list of dicts with L, n_beads and
     any make_params keyword."""
 
     def __init__(self, points, stream=None):

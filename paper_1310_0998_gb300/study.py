@@ -54,7 +54,7 @@ def slope(E, k0: int, k1: int) -> float:
     return float(np.linalg.lstsq(A, y, rcond=None)[0][0])
 
 
-CHUNK = 10_000   # steps per persistent launch (a few seconds each at paper size)
+CHUNK = 10_000   # steps per call (a few seconds each at paper size)
 
 
 def _advance(ens, n: int):

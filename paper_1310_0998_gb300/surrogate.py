@@ -64,7 +64,7 @@ def _snapshot(sim, M, dr, nbins):
 def simulate(X, L=SUR_L, burn=2000, n_snap=10, every=200, M=128, dr=0.25, seed=0, batched=True, chunk=256):
     """Statistics [n][40] of the parameter rows X [n][4] = (phi, gamma, zeta,
     f_p).  batched: the points as ensembles of up to `chunk` replicas
-    (persistent kernel); else one simulation after another (the plain path).
+    advanced together; else one simulation after another (the plain path).
     Point i starts from the random initial condition of seed + i."""
     from .ensemble import Ensemble
     from .sim import Sim
@@ -73,7 +73,7 @@ def simulate(X, L=SUR_L, burn=2000, n_snap=10, every=200, M=128, dr=0.25, seed=0
     pts = [point_params(*X[i], L=L, seed=seed + i, replica=i) for i in range(X.shape[0])]
     snaps = [[[], [], [], []] for _ in pts]
     if batched:
-        # replicas in batches of at most `chunk` per persistent launch; replica
+        # replicas in batches of at most `chunk`; replica
         # i keeps seed + i and replica key i whatever batch it lands in
         for c0 in range(0, len(pts), chunk):
             ens = Ensemble(pts[c0:c0 + chunk])
