@@ -139,9 +139,9 @@ void dpd_destroy(dpd_ctx *ctx);
 /* Replace the interaction/integration parameters.  n_beads, L and r_c must be
  * unchanged (DPD_ERR_STATE otherwise: they fix the cell geometry), and so must
  * the tile: 0, the context's, or, where the context was created with tile 0, 8 (or
- * the tuned shape's), which stands for the default.  Takes effect at the next step; forces of the
- * current state are not recomputed.  A batch's own steps keep the parameters that
- * its replicas were created with. */
+ * the tuned shape's), which stands for the default.  Takes effect at the next
+ * step; forces of the current state are not recomputed.  A batch's own steps
+ * keep the parameters that its replicas were created with. */
 int dpd_set_params(dpd_ctx *ctx, const dpd_params *p);
 
 /* Set the canonical state at step `step`.  x: [N][2] positions (anywhere;
