@@ -833,8 +833,8 @@ __device__ void force_tile_global(const Sys &d, uint32_t g0, int n_own, uint32_t
 
 // Block reduction of a tile's thermo partials into the FP64 ring slot of
 // `step` (FP64 throughout): every thread's partials to shared memory (buf,
-// 3 blockDim doubles), then warp q adds quantity q (blockDim / 32 values per
-// lane, then across its lanes) and adds it to the slot.  A third of the FP64
+// 3 blockDim doubles), then one warp per quantity (two warps: one takes two) sums
+// it (blockDim / 32 values per lane, then across its lanes) and adds it to the slot.  A third of the FP64
 // additions of a shuffle tree in every warp (the FP64 pipe is narrow on this
 // part).  buf is read by warps 0-2 after the call: the caller synchronises
 // before reusing it.
@@ -845,12 +845,12 @@ __device__ __forceinline__ void thermo_flush_tile(const Sys &d, Thermo3 th, doub
     buf[nt + tid] = th.px;
     buf[2 * nt + tid] = th.py;
     __syncthreads();
-    if (wid < 3) {
+    for (int q = wid; q < 3; q += nt >> 5) {   // (a dilute tile has two warps)
         double a = 0.0;
-        for (int i = lane; i < nt; i += 32) a += buf[wid * nt + i];
+        for (int i = lane; i < nt; i += 32) a += buf[q * nt + i];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) atomicAdd(&d.thermo[4 * (size_t)(*d.step % THERMO_CAP) + wid], a);
+        if (lane == 0) atomicAdd(&d.thermo[4 * (size_t)(*d.step % THERMO_CAP) + q], a);
     }
 }
 
